@@ -128,9 +128,19 @@ typedef struct {
                         time a given set of arguments is met and replay it after */
   int32_t fp64_kernel; /* 0, or 1 + BSM_FP64_* to force that FP64 kernel (ignored by
                           the split precisions); out of range: BSM_ERR_INVALID_ARG.
-                          Without it (and without a tuned choice): PK12, or where
-                          C blocks have fewer than 4 products on average, G8 when
-                          C's blocks are at most 8 x 8, else T16_B2 */
+                          Without it (and without a tuned choice): PK12 or its form
+                          on the tensor cores (below), or where C blocks have fewer
+                          than 4 products on average, G8 when C's blocks are at most
+                          8 x 8, else T16_B2.
+                          The form on the tensor cores multiplies 62-bit integer
+                          images of the operands (on a scale per scalar row of A and
+                          column of B) exactly, digit by digit, and rounds to FP64
+                          once per 144 values of k; C blocks with an operand that such
+                          an image would hold less exactly than FP64 does (infinities,
+                          NaN, rows of widely different size in one block) are left to
+                          the packed kernel. It takes device memory for the images,
+                          about 1.6 times the operands' values each, kept with the
+                          context; without that memory PK12 runs */
   double *host_values; /* NULL, or page-locked host memory (cudaHostAlloc /
                           cudaHostRegister, device-mapped) of host_cap doubles that also
                           receives the result's values, in bsm_mat_get_values order,

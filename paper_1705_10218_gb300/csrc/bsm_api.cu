@@ -14,6 +14,7 @@
 
 #include <algorithm>
 #include <atomic>
+#include <cmath>
 #include <cstdio>
 #include <cstdlib>
 #include <cstring>
@@ -163,11 +164,25 @@ void cache_free(void *p) {
   }
 }
 
+// The context of the call that runs on this thread: an allocation that fails
+// takes back its digit workspace (which a multiply can do without) and retries.
+thread_local bsm_ctx t_ctx = nullptr;
+bool digit_reclaim(bsm_ctx ctx);
+
+cudaError_t cache_alloc_reclaim(void **p, size_t bytes) {
+  cudaError_t e = cache_alloc(p, bytes);
+  if (e == cudaErrorMemoryAllocation && t_ctx) {
+    cudaGetLastError();
+    if (digit_reclaim(t_ctx)) e = cache_alloc(p, bytes);
+  }
+  return e;
+}
+
 template <class T>
 int dev_alloc(T **p, int64_t n) {
   if (n <= 0) n = 1;
   void *q = nullptr;
-  cudaError_t e = cache_alloc(&q, (size_t)n * sizeof(T));
+  cudaError_t e = cache_alloc_reclaim(&q, (size_t)n * sizeof(T));
   if (e != cudaSuccess) {
     *p = nullptr;
     cudaGetLastError();
@@ -238,6 +253,11 @@ struct bsm_mat_s {
   void *split_left = nullptr, *split_right = nullptr;
   int64_t cap_left = 0, cap_right = 0;  // bytes
   int32_t *row_sizes = nullptr, *col_sizes = nullptr;
+  // first scalar row (column) of each block row (column), and their number in all
+  int32_t *row_first = nullptr, *col_first = nullptr;
+  int64_t scalar_rows = 0, scalar_cols = 0;
+  // the largest ceil(k / 8) / k of a block as a left and as a right operand
+  double digit_rate[2] = {0, 0};
   Buf front, back;
   int64_t nblk = 0, nnz = 0;  // valid when !pend.active
   int64_t hint_blk = 0, hint_nnz = 0;  // sizes of the last result computed into it
@@ -267,6 +287,7 @@ struct bsm_ctx_s {
   cudaEvent_t ev_up = nullptr;
   cudaEvent_t ev_t0 = nullptr, ev_t1 = nullptr;
   DevStatus *d_status = nullptr;
+  int32_t *d_ticket = nullptr;           // thread blocks done of the count pass (zero between launches)
   unsigned long long *d_work = nullptr;  // work counter of the dynamically scheduled kernels
   DevStatus *h_slots = nullptr;    // pinned ring of status copies
   unsigned char *h_stage = nullptr;  // pinned staging of uploaded index arrays
@@ -295,6 +316,10 @@ struct bsm_ctx_s {
   // its fallback list reuses cls_items / cls_segs
   PanelWs pw{};
   int64_t cap_pw_recs = 0, cap_pw_tiles = 0, cap_pw_rows = 0;
+  // digits of the operands of the multiply that runs (entries, block metadata,
+  // scales), for the FP64 products on the tensor cores; capacities in elements
+  Digits dg{};
+  int64_t cap_dg_units[2] = {0, 0}, cap_dg_meta[2] = {0, 0}, cap_dg_expo[2] = {0, 0};
   int32_t *cls_counts = nullptr, *cls_cursor = nullptr;  // [kMaxClasses]
   int64_t *cls_segs = nullptr;   // [2 * kMaxClasses]
   // captured multiplies (opts.graph), keyed by every kernel argument
@@ -345,6 +370,7 @@ static int prof_collect(bsm_ctx ctx, int s) {
 }
 
 static int ctx_set_device(bsm_ctx ctx) {
+  t_ctx = ctx;
   CK(cudaSetDevice(ctx->device));
   return BSM_OK;
 }
@@ -519,12 +545,85 @@ static int resolve(bsm_mat M, bsm_stats *timed = nullptr);
 // ---------------------------------------------------------------------------
 // the multiply pipeline
 // ---------------------------------------------------------------------------
-static int enqueue_norms(bsm_ctx ctx, bsm_mat M, cudaStream_t s) {
-  const int grid = ctx->nsm * 8;
-  CK(launch_block_norms(M->row_sizes, M->col_sizes, M->front.blk_row, M->front.col_idx,
-                        M->front.blk_off, M->front.vals, M->front.hdr, M->front.norms,
-                        M->front.normsf, grid, s));
+// rexp, cexp: also the scales of M's scalar rows / columns (or null).
+static int enqueue_norms(bsm_ctx ctx, bsm_mat M, cudaStream_t s, int32_t *rexp = nullptr,
+                         int32_t *cexp = nullptr) {
+  CK(launch_block_norms_scales(M->row_sizes, M->col_sizes, M->front.blk_row, M->front.col_idx,
+                               M->front.blk_off, M->front.vals, M->front.hdr, M->front.norms,
+                               M->front.normsf, M->row_first, M->col_first, rexp, cexp, ctx->nsm,
+                               s));
   return BSM_OK;
+}
+
+// The digit workspace. digit_reclaim: gives it back. digit_scales: the scale arrays of A's rows and B's
+// columns; digit_entries: the entries and block metadata. Both return false
+// (and leave the FP64 kernels to the multiply) where the operands have more
+// values or rows than the 32-bit indices reach, or the memory is not there.
+namespace {
+// Frees the entries and metadata (not the scales, which are small) once the
+// work that uses them is done; true if there were any.
+bool digit_reclaim(bsm_ctx ctx) {
+  DigitSide *sides[2] = {&ctx->dg.a, &ctx->dg.b};
+  bool any = false;
+  for (int x = 0; x < 2; x++) any = any || sides[x]->units || sides[x]->meta;
+  if (!any || cudaStreamSynchronize(ctx->stream) != cudaSuccess) return false;
+  for (int x = 0; x < 2; x++) {
+    dev_free(sides[x]->units);
+    dev_free(sides[x]->meta);
+    ctx->cap_dg_units[x] = ctx->cap_dg_meta[x] = 0;
+  }
+  return true;
+}
+}  // namespace
+
+template <class T>
+static bool digit_grow(bsm_ctx ctx, T *&p, int64_t &cap, int64_t n) {
+  if (cap >= n) return true;
+  if (p && cudaStreamSynchronize(ctx->stream) != cudaSuccess) return false;
+  dev_free(p);
+  cap = 0;
+  const bsm_ctx c = t_ctx;
+  t_ctx = nullptr;  // the digits take nothing back from themselves
+  const int rc = dev_alloc(&p, n + n / 8 + 64);
+  t_ctx = c;
+  if (rc) return false;
+  cap = n + n / 8 + 64;
+  return true;
+}
+
+static bool digit_scales(bsm_ctx ctx, bsm_mat A, bsm_mat B) {
+  if (A->scalar_rows >= (int64_t)INT32_MAX || B->scalar_cols >= (int64_t)INT32_MAX) return false;
+  ctx->dg.a.first = A->row_first;
+  ctx->dg.b.first = B->col_first;
+  return digit_grow(ctx, ctx->dg.a.expo, ctx->cap_dg_expo[0], A->scalar_rows) &&
+         digit_grow(ctx, ctx->dg.b.expo, ctx->cap_dg_expo[1], B->scalar_cols);
+}
+
+static bool digit_entries(bsm_ctx ctx, bsm_mat A, bsm_mat B, cudaStream_t s) {
+  DigitSide *sides[2] = {&ctx->dg.a, &ctx->dg.b};
+  bsm_mat mats[2] = {A, B};
+  for (int x = 0; x < 2; x++) {
+    bsm_mat M = mats[x];
+    // an operand of m rows (a right one: columns) and k up to s takes
+    // 4 m ceil(s / 8) units: room by the block's values, at the rate of the least
+    // favourable k, or half a unit a value and what the largest sizes add to
+    // each block, whichever is less
+    const double rate = 4.0 * M->digit_rate[x];
+    const int64_t pad = (7 * (int64_t)(x == 0 ? M->max_row : M->max_col) + 1) / 2;
+    const bool by_value = (rate - 0.5) * (double)M->nnz <= (double)(pad * M->nblk);
+    sides[x]->mul = by_value ? (int64_t)std::ceil(64.0 * rate) : 32;
+    sides[x]->pad = by_value ? 0 : pad;
+    const int64_t n = kDigitZeros + (M->nnz * sides[x]->mul >> 6) + M->nblk * sides[x]->pad + 1;
+    if (n >= (int64_t)UINT32_MAX) return false;
+    const void *old = sides[x]->units;
+    if (!digit_grow(ctx, sides[x]->units, ctx->cap_dg_units[x], n) ||
+        !digit_grow(ctx, sides[x]->meta, ctx->cap_dg_meta[x], M->nblk))
+      return false;
+    if (sides[x]->units != old &&
+        cudaMemsetAsync(sides[x]->units, 0x80, kDigitZeros * sizeof(uint4), s) != cudaSuccess)
+      return false;
+  }
+  return true;
 }
 
 // Slice buffers of M for the given layouts, sized for its current values.
@@ -538,7 +637,7 @@ static int split_buffers(bsm_mat M, int precision, bool left, bool right) {
     }
     p = nullptr;
     cap = 0;
-    cudaError_t e = cache_alloc(&p, (size_t)need);
+    cudaError_t e = cache_alloc_reclaim(&p, (size_t)need);
     if (e != cudaSuccess) {
       cudaGetLastError();
       return cuda_fail(e, "cudaMalloc(slices)");
@@ -620,7 +719,7 @@ static void tune_load(bsm_ctx ctx) {
         ctx->tune[key] = v;
         ctx->pk_tab[pk_tab_at(slots, m, n)] = (uint16_t)v;
       }
-    } else if (v >= 0 && v < kFp64NumVariants) {
+    } else if (v >= 0 && v < kFp64NumAll) {
       ctx->tune[key] = v;
     }
   }
@@ -677,21 +776,24 @@ static_assert((int)kFp64T16B2 == (int)BSM_FP64_T16_B2 && (int)kFp64T16B3 == (int
                   (int)kFp64NumVariants == (int)BSM_FP64_NUM_KERNELS,
               "public and internal FP64 kernel numbers differ");
 
-// The default FP64 kernel for a result C: the packed kernel, unless the last
-// multiply into C had fewer than 4 block products per C block (the sizes of
-// the previous result, or of this one once the symbolic totals were read).
-static int fp64_default(bsm_ctx ctx, bsm_mat C) {
+// The default FP64 kernel for a result C: the digit kernel where the operands'
+// digits are there (dg), else the packed kernel, unless the last multiply into
+// C had fewer than 4 block products per C block (the sizes of the previous
+// result, or of this one once the symbolic totals were read).
+static int fp64_default(bsm_ctx ctx, bsm_mat C, bool dg) {
   if (C->hint_blk > 0 && ctx->hint_prod < 4 * C->hint_blk)  // few products per C block
     return (C->max_row <= 8 && C->max_col <= 8) ? kFp64G8 : kFp64T16B2;
-  return kFp64Pk12;
+  return dg ? kFp64Dg : kFp64Pk12;
 }
 
-// The forced kernel, else the tuned one, else the default.
+// The forced kernel, else the tuned one, else the default. A tuned digit kernel
+// whose operands have no digits is the packed kernel.
 static int variant_or_default(bsm_ctx ctx, bsm_mat C, const bsm_opts &o,
-                              const std::string &key) {
+                              const std::string &key, bool dg) {
   if (o.fp64_kernel > 0) return o.fp64_kernel - 1;
   auto it = ctx->tune.find(key);
-  return it == ctx->tune.end() ? fp64_default(ctx, C) : it->second;
+  const int v = it == ctx->tune.end() ? fp64_default(ctx, C, dg) : it->second;
+  return (v == kFp64Dg && !dg) ? (int)kFp64Pk12 : v;
 }
 
 // The split-precision kernel of a multiply: the forced one, else the per-block
@@ -712,6 +814,8 @@ struct Launch {
   int slot;
   cudaStream_t s;
   bool use_cin, split, prof;
+  bool scales;        // the digit scales are computed with the norms
+  bool dg;            // the fill pass writes the operands' digits
   bool host_written;  // every numeric launch so far stored the host copy itself
   bool gated;         // call the context's slice gate between numeric slices
   DevMat dA, dB, dC;
@@ -724,10 +828,17 @@ static int stage_a(Launch &L, bool record) {
   bsm_ctx ctx = L.ctx;
   int rc;
   if (L.prof && record) CK(cudaEventRecord(ctx->prof_ev[L.slot][0], L.s));
-  if ((rc = enqueue_norms(ctx, L.A, L.s))) return rc;
+  int32_t *rexp = nullptr, *cexp = nullptr;
+  if (L.scales) {
+    rexp = ctx->dg.a.expo;
+    cexp = ctx->dg.b.expo;
+    CK(cudaMemsetAsync(rexp, 0, (size_t)L.A->scalar_rows * sizeof(int32_t), L.s));
+    CK(cudaMemsetAsync(cexp, 0, (size_t)L.B->scalar_cols * sizeof(int32_t), L.s));
+  }
+  if ((rc = enqueue_norms(ctx, L.A, L.s, rexp, L.B == L.A ? cexp : nullptr))) return rc;
   ctx->launches++;
   if (L.B != L.A) {
-    if ((rc = enqueue_norms(ctx, L.B, L.s))) return rc;
+    if ((rc = enqueue_norms(ctx, L.B, L.s, nullptr, cexp))) return rc;
     ctx->launches++;
   }
   if (L.split) {  // operand slices for the tensor-core products
@@ -745,10 +856,15 @@ static int stage_a(Launch &L, bool record) {
     }
   }
   if (L.prof && record) CK(cudaEventRecord(ctx->prof_ev[L.slot][1], L.s));
-  CK(launch_symbolic_count(L.dA, L.dB, L.dC, L.use_cin ? 1 : 0, L.eps, L.ws, ctx->nsm * 6, L.s));
+  // with few rows the count pass's last thread block does the scan
+  const bool fused = L.A->nbr <= kFusedScanRows;
+  CK(launch_symbolic_count(L.dA, L.dB, L.dC, L.use_cin ? 1 : 0, L.eps, L.ws, L.out, ctx->d_status,
+                           fused ? ctx->d_ticket : nullptr, ctx->nsm * 6, L.s));
   ctx->launches++;
-  CK(launch_symbolic_scan(L.A->nbr, L.ws, L.out, ctx->d_status, L.s));
-  ctx->launches++;
+  if (!fused) {
+    CK(launch_symbolic_scan(L.A->nbr, L.ws, L.out, ctx->d_status, L.s));
+    ctx->launches++;
+  }
   return BSM_OK;
 }
 
@@ -797,12 +913,24 @@ static int launch_numeric(Launch &L, int variant, const int32_t *items, const in
   } else {
     if (fp64_variant_uses_work(variant))
       CK(cudaMemsetAsync(ctx->d_work, 0, sizeof(unsigned long long), L.s));
-    ctx->last_fp64 = variant;
+    // the digit kernel is the packed choice's form on the tensor cores: reported as it
+    ctx->last_fp64 = variant == kFp64Dg ? (int)kFp64Pk12 : variant;
+    Digits dg = ctx->dg;
+    dg.list = L.ws.cnt;  // the fill pass's counters, free by now
+    if (variant == kFp64Dg) CK(cudaMemsetAsync(dg.range, 0, 2 * sizeof(int64_t), L.s));
     L.host_written = L.host_written && fp64_variant_writes_host(variant);
     CK(launch_numeric_fp64(variant, L.dA, L.dB, L.out, L.dC, L.alpha, L.beta, L.ws,
                            ctx->d_status, items, seg,
                            ctx->nsm * fp64_variant_blocks_per_sm(variant), ctx->d_work, max_m,
-                           max_n, L.s));
+                           max_n, &dg, L.s));
+    if (variant == kFp64Dg) {  // the C blocks it left to the packed kernel, if any
+      ctx->launches++;
+      CK(cudaMemsetAsync(ctx->d_work, 0, sizeof(unsigned long long), L.s));
+      CK(launch_numeric_fp64(kFp64Pk12, L.dA, L.dB, L.out, L.dC, L.alpha, L.beta, L.ws,
+                             ctx->d_status, dg.list, dg.range,
+                             ctx->nsm * fp64_variant_blocks_per_sm(kFp64Pk12), ctx->d_work, max_m,
+                             max_n, nullptr, L.s));
+    }
   }
   ctx->launches++;
   return BSM_OK;
@@ -919,7 +1047,7 @@ static int stage_b(Launch &L, bool record, bool may_tune) {
   int rc;
   L.host_written = true;  // the split kernels store it; FP64 launches update this
   CK(launch_symbolic_fill(L.dA, L.dB, L.dC, L.use_cin ? 1 : 0, L.eps, L.ws, L.out, ctx->d_status,
-                          ctx->nsm, fill_mask_words(L), L.s));
+                          ctx->nsm, fill_mask_words(L), L.dg ? &ctx->dg : nullptr, L.s));
   ctx->launches++;
   if (L.prof && record) CK(cudaEventRecord(ctx->prof_ev[L.slot][2], L.s));
   if (L.split && split_kernel_of(L.o, L.B) == BSM_SPLIT_PANEL) {
@@ -953,24 +1081,25 @@ static int stage_b(Launch &L, bool record, bool may_tune) {
       const std::string key = tune_key_class(m, n);
       const int64_t *seg = ctx->cls_segs + 2 * c;
       if (may_tune && L.o.autotune && !L.o.fp64_kernel && !L.split && !ctx->tune.count(key)) {
-        int best = fp64_default(ctx, L.C);
+        int best = fp64_default(ctx, L.C, L.dg);
         double best_ms = 1e30;
-        for (int v = 0; v < kFp64NumVariants; v++) {
+        for (int v = 0; v < (L.dg ? kFp64NumAll : kFp64NumVariants); v++) {
           double ms;
           if ((rc = time_variant(L, v, ctx->cls_items, seg, m, n, &ms))) return rc;
           if (ms < best_ms) best_ms = ms, best = v;
         }
         tune_save(ctx, key, best, best_ms);
       }
-      if ((rc = launch_numeric(L, variant_or_default(ctx, L.C, L.o, key), ctx->cls_items, seg, m, n)))
+      if ((rc = launch_numeric(L, variant_or_default(ctx, L.C, L.o, key, L.dg), ctx->cls_items, seg, m,
+                               n)))
         return rc;
     }
   } else {
     const std::string key = tune_key_all(L.A, L.B);
     if (may_tune && L.o.autotune && !L.o.fp64_kernel && !L.split && !ctx->tune.count(key)) {
-      int best = fp64_default(ctx, L.C);
+      int best = fp64_default(ctx, L.C, L.dg);
       double best_ms = 1e30;
-      for (int v = 0; v < kFp64NumVariants; v++) {
+      for (int v = 0; v < (L.dg ? kFp64NumAll : kFp64NumVariants); v++) {
         double ms;
         if ((rc = time_variant(L, v, nullptr, nullptr, L.A->max_row, L.B->max_col, &ms)))
           return rc;
@@ -978,7 +1107,7 @@ static int stage_b(Launch &L, bool record, bool may_tune) {
       }
       tune_save(ctx, key, best, best_ms);
     }
-    const int variant = variant_or_default(ctx, L.C, L.o, key);
+    const int variant = variant_or_default(ctx, L.C, L.o, key, L.dg);
     if (may_tune && L.o.autotune && !L.o.fp64_kernel && !L.split &&
         tiles_need_tuning(ctx, L.A, L.B, variant) && (rc = tune_pk_tiles(L, variant)))
       return rc;
@@ -1050,7 +1179,9 @@ static void graph_key(const Launch &L, std::vector<uint64_t> &k) {
   num(L.o.precision), num(L.o.launch), num(L.o.fp64_kernel), num((int64_t)L.ctx->tune_version);
   num(L.o.split_kernel), num(L.o.numeric_slices);
   put(L.out.host_vals), num(L.out.host_cap);
-  num(fp64_default(L.ctx, L.C));
+  num(fp64_default(L.ctx, L.C, L.dg)), num(L.dg), num(L.scales);
+  for (const DigitSide *d : {&L.ctx->dg.a, &L.ctx->dg.b})
+    put(d->units), put(d->meta), put(d->expo), put(d->first), num(d->mul), num(d->pad);
 }
 
 // Enqueue one multiply. sync_sizes: read the totals back after the scan and
@@ -1106,6 +1237,14 @@ static int run_multiply(bsm_ctx ctx, double alpha, bsm_mat A, bsm_mat B, double 
   // the panel kernel's work buffers before any capture (no allocation inside one)
   if (L.split && split_kernel_of(o, B) == BSM_SPLIT_PANEL && (rc = panel_ws(ctx, A->nbr)))
     return rc;
+  // The digit kernel may run: the scales are computed with the norms, and, once
+  // the sizes are known, the entries get their memory (after every other
+  // buffer; a multiply that cannot have it takes the FP64 kernels).
+  auto wants_digits = [&]() {
+    return o.autotune || !ctx->tune.empty() || fp64_default(ctx, C, true) == kFp64Dg;
+  };
+  L.scales = !L.split && !o.fp64_kernel && (sync_sizes || wants_digits()) && digit_scales(ctx, A, B);
+  if (!sync_sizes) L.dg = L.scales && digit_entries(ctx, A, B, L.s);
   const bool use_graph = o.graph && !sync_sizes;
   L.prof = ctx->prof && !use_graph;
   if (stats) CK(cudaEventRecord(ctx->ev_t0, L.s));
@@ -1178,6 +1317,7 @@ static int run_multiply(bsm_ctx ctx, double alpha, bsm_mat A, bsm_mat B, double 
         CK(launch_symbolic_scan(A->nbr, L.ws, L.out, ctx->d_status, L.s));
         ctx->launches++;
       }
+      L.dg = L.scales && wants_digits() && digit_entries(ctx, A, B, L.s);
     }
     if ((rc = stage_b(L, true, true))) return rc;
   }
@@ -1261,6 +1401,7 @@ const char *bsm_last_cuda_error(void) { return g_cuda_err; }
 int bsm_ctx_create(int device, bsm_ctx *out) {
   if (!out) return BSM_ERR_INVALID_ARG;
   *out = nullptr;
+  t_ctx = nullptr;
   int ndev = 0;
   CK(cudaGetDeviceCount(&ndev));
   if (device < 0 || device >= ndev) return BSM_ERR_INVALID_ARG;
@@ -1299,6 +1440,10 @@ int bsm_ctx_create(int device, bsm_ctx *out) {
   }
   if (rc == BSM_OK) {
     rc = dev_alloc(&ctx->cls_counts, kMaxClasses);
+    if (rc == BSM_OK) rc = dev_alloc(&ctx->dg.range, 2);
+    if (rc == BSM_OK) rc = dev_alloc(&ctx->d_ticket, 1);
+    if (rc == BSM_OK && (e = cudaMemsetAsync(ctx->d_ticket, 0, sizeof(int32_t), ctx->stream)) != cudaSuccess)
+      rc = cuda_fail(e, "cudaMemset");
     if (rc == BSM_OK) rc = dev_alloc(&ctx->cls_cursor, kMaxClasses);
     if (rc == BSM_OK) rc = dev_alloc(&ctx->cls_segs, 2 * kMaxClasses);
   }
@@ -1361,6 +1506,13 @@ int bsm_ctx_destroy(bsm_ctx ctx) {
   dev_free(ctx->cls_items);
   dev_free(ctx->ord_start);
   dev_free(ctx->d_pk_tab);
+  dev_free(ctx->d_ticket);
+  dev_free(ctx->dg.range);
+  for (DigitSide *d : {&ctx->dg.a, &ctx->dg.b}) {
+    dev_free(d->units);
+    dev_free(d->meta);
+    dev_free(d->expo);
+  }
   dev_free(ctx->pw.recs);
   dev_free(ctx->pw.tiles);
   dev_free(ctx->pw.row_nt);
@@ -1728,8 +1880,28 @@ int bsm_mat_create(bsm_ctx ctx, int32_t nbrows, const int32_t *row_sizes, int32_
     bsm_mat_destroy(M);
     return code;
   };
+  // first scalar row / column of each block row / column (32-bit: the digit
+  // kernel, their only reader, takes matrices of less than 2^31 of them)
+  std::vector<int32_t> h_row_first, h_col_first;
+  auto firsts = [](const std::vector<int32_t> &sizes, std::vector<int32_t> &first) {
+    int64_t at = 0;
+    first.resize(sizes.size() + 1);
+    for (size_t i = 0; i < sizes.size(); i++) first[i] = (int32_t)at, at += sizes[i];
+    first[sizes.size()] = (int32_t)at;
+    return at;
+  };
+  auto most = [](const std::vector<int32_t> &sizes) {  // largest ceil(v / 8) / v
+    double r = 0;
+    for (int32_t v : sizes) r = std::max(r, (double)((v - 1) / 8 + 1) / v);
+    return r;
+  };
+  M->digit_rate[0] = most(M->h_col_sizes);
+  M->digit_rate[1] = most(M->h_row_sizes);
+  M->scalar_rows = firsts(M->h_row_sizes, h_row_first);
+  M->scalar_cols = firsts(M->h_col_sizes, h_col_first);
   if ((rc = dev_alloc(&M->row_sizes, nbrows)) || (rc = dev_alloc(&M->col_sizes, nbcols)) ||
-      (rc = dev_alloc(&M->row_cls, nbrows)) || (rc = dev_alloc(&M->col_cls, nbcols)))
+      (rc = dev_alloc(&M->row_cls, nbrows)) || (rc = dev_alloc(&M->col_cls, nbcols)) ||
+      (rc = dev_alloc(&M->row_first, nbrows + 1)) || (rc = dev_alloc(&M->col_first, nbcols + 1)))
     return fail(rc);
   cudaStream_t s = ctx->stream;
   auto cp = [&](void *dst, const void *src, size_t bytes) -> cudaError_t {
@@ -1739,7 +1911,9 @@ int bsm_mat_create(bsm_ctx ctx, int32_t nbrows, const int32_t *row_sizes, int32_
   if ((e = cp(M->row_sizes, row_sizes, (size_t)nbrows * 4)) != cudaSuccess ||
       (e = cp(M->col_sizes, col_sizes, (size_t)nbcols * 4)) != cudaSuccess ||
       (e = cp(M->row_cls, h_row_cls.data(), (size_t)nbrows * 4)) != cudaSuccess ||
-      (e = cp(M->col_cls, h_col_cls.data(), (size_t)nbcols * 4)) != cudaSuccess)
+      (e = cp(M->col_cls, h_col_cls.data(), (size_t)nbcols * 4)) != cudaSuccess ||
+      (e = cp(M->row_first, h_row_first.data(), ((size_t)nbrows + 1) * 4)) != cudaSuccess ||
+      (e = cp(M->col_first, h_col_first.data(), ((size_t)nbcols + 1) * 4)) != cudaSuccess)
     return fail(cuda_fail(e, "bsm_mat_create copy"));
   if ((rc = upload_contents(M, nblocks, blk_row, blk_col, values, true))) return fail(rc);
   *out = M;
@@ -1791,6 +1965,8 @@ int bsm_mat_destroy(bsm_mat m) {
   dev_free(m->col_sizes);
   dev_free(m->row_cls);
   dev_free(m->col_cls);
+  dev_free(m->row_first);
+  dev_free(m->col_first);
   dev_free(m->row_order);
   if (m->ev_use) cudaEventDestroy(m->ev_use);
   // captured multiplies may name this matrix's buffers

@@ -85,14 +85,75 @@ struct DevStatus {
   int32_t error;    // nonzero: a device-side check failed
 };
 
+// ---------------------------------------------------------------------------
+// FP64 operands as digits (k_numeric_fp64.cu, digits.cuh). A scalar row r of a
+// left operand (a scalar column of a right one) has a scale 2^E, E from the
+// largest exponent in the whole row, and a block a class c >= 0, the largest with
+// every value of the block below 2^(E - 8 c). Its values are held as 62-bit integers
+// X = round(x * 2^(62 - E + 8 c)) = sum_i d_i 256^(7-i) in eight signed digits d_i
+// in [-128, 127] (|d_0| <= 64).
+// A unit is 16 bytes: the digits of two values of a row that follow each other
+// along k, digit i of both (as bytes d + 128) at 2 i and 2 i + 1; zeros past the end
+// of k. Eight values of k are an octet, four units of a row. A block (m x s as a
+// left operand; its columns as the rows of a right one) is ceil(s / 8) octets of
+// 4 units for each row, row after row: as much as its FP64 values, with k up to a
+// multiple of 8. Block b's units start at kDigitZeros + (blk_off[b] * mul >> 6) +
+// b * pad; the units before are zeros. meta[b]: {first unit, octets | class << 16 |
+// kDigitOutside}. A block is outside when a digit representation would lose more
+// than FP64 does: a value that is not finite, a scale beyond 2^+-300, a row (column)
+// of the block whose largest value is below 2^-kDigitRange of the scale less the
+// class (it would keep less than 62 - kDigitRange bits), or more than kDigitMaxRows
+// rows or kDigitMaxOctets octets; the C blocks it contributes to are computed by
+// FP64 FMAs.
+// ---------------------------------------------------------------------------
+constexpr int kDigits = 8;
+constexpr int kDigitZeros = 64;
+constexpr uint32_t kDigitOutside = 1u << 31;
+constexpr int kDigitRange = 11;
+constexpr int kDigitMaxRows = 128;
+constexpr int kDigitMaxOctets = 0xFFFF;
+constexpr int kDigitMaxClass = 60;
+// exponent fields (of the row's largest value) that have a scale
+constexpr int kDigitExpLo = 722, kDigitExpHi = 1322;
+
+struct DigitSide {
+  uint4 *units;
+  uint2 *meta;           // [nblk]
+  int32_t *expo;         // [scalar rows or columns] largest exponent field (0: all zero)
+  const int32_t *first;  // [block rows or columns + 1] first scalar row or column
+  int64_t mul, pad;
+};
+// The digits of a multiply's operands: A's as a left, B's as a right operand.
+struct Digits {
+  DigitSide a, b;
+  // C blocks that the digit kernel leaves to the packed one: their number
+  // (range[0] = 0, range[1]) and list
+  int64_t *range;
+  int32_t *list;
+};
+
 // ---- launchers (each enqueues on `stream`, returns cudaGetLastError()) ----
+// The norms, and the largest exponent fields of every scalar row (column) into
+// rexp (cexp) where these are not null (zero before the launch; rfirst, cfirst:
+// the first scalar row (column) of each block row (column)).
+cudaError_t launch_block_norms_scales(const int32_t *row_sizes, const int32_t *col_sizes,
+                                      const int32_t *blk_row, const int32_t *col_idx,
+                                      const int64_t *blk_off, const double *vals,
+                                      const int64_t *hdr, double *norms, float *normsf,
+                                      const int32_t *rfirst, const int32_t *cfirst, int32_t *rexp,
+                                      int32_t *cexp, int nsm, cudaStream_t stream);
 cudaError_t launch_block_norms(const int32_t *row_sizes, const int32_t *col_sizes,
                                const int32_t *blk_row, const int32_t *col_idx,
                                const int64_t *blk_off, const double *vals, const int64_t *hdr,
                                double *norms, float *normsf, int grid, cudaStream_t stream);
 
+// ticket: null, or a device counter that is zero (and is left zero): the last
+// thread block then also does the scan (nbr <= kFusedScanRows: one launch less,
+// where the scan's own thread block would take as long as its launch).
+constexpr int32_t kFusedScanRows = 2048;
 cudaError_t launch_symbolic_count(DevMat A, DevMat B, DevMat Cin, int use_cin, double eps,
-                                  DevWs ws, int grid, cudaStream_t stream);
+                                  DevWs ws, DevOut C, DevStatus *st, int32_t *ticket, int grid,
+                                  cudaStream_t stream);
 
 cudaError_t launch_symbolic_scan(int32_t nbr, DevWs ws, DevOut C, DevStatus *st,
                                  cudaStream_t stream);
@@ -100,9 +161,10 @@ cudaError_t launch_symbolic_scan(int32_t nbr, DevWs ws, DevOut C, DevStatus *st,
 // mask_words: words of the per-row bit matrix of the placement (a bound on C
 // blocks per row times the words per A row; rows beyond it take the slower
 // per-window passes); 0: the largest (8192).
+// digits: also write the digits of A (left) and B (right), or null.
 cudaError_t launch_symbolic_fill(DevMat A, DevMat B, DevMat Cin, int use_cin, double eps,
                                  DevWs ws, DevOut C, const DevStatus *st, int nsm, int mask_words,
-                                 cudaStream_t stream);
+                                 const Digits *digits, cudaStream_t stream);
 
 // FP64 numeric kernel variants (k_numeric_fp64.cu).
 enum {
@@ -112,7 +174,9 @@ enum {
   kFp64Pk12 = 3,
   kFp64Pk16 = 4,
   kFp64G8 = 5,
-  kFp64NumVariants = 6
+  kFp64NumVariants = 6,  // the kernels a caller can force
+  kFp64Dg = 6,           // digits on the tensor cores: what the default and the tuner add to them
+  kFp64NumAll = 7
 };
 int fp64_variant_blocks_per_sm(int variant);
 // The packed kernel's built-in slot shape (nT, G) of a tile of te elements
@@ -132,7 +196,7 @@ cudaError_t numeric_fp64_init();
 cudaError_t launch_numeric_fp64(int variant, DevMat A, DevMat B, DevOut C, DevMat Cin,
                                 double alpha, double beta, DevWs ws, const DevStatus *st,
                                 const int32_t *items, const int64_t *seg, int grid,
-                                unsigned long long *work, int max_m, int max_n,
+                                unsigned long long *work, int max_m, int max_n, const Digits *digits,
                                 cudaStream_t stream);
 inline bool fp64_variant_uses_work(int variant) { return variant != kFp64T32; }
 
@@ -222,7 +286,7 @@ cudaError_t launch_filter_fill(DevMat M, double eps, DevWs ws, DevOut O, const D
 // and the multiply did not overflow.
 cudaError_t launch_copy_out(DevOut O, const DevStatus *st, int nsm, cudaStream_t stream);
 inline bool fp64_variant_writes_host(int variant) {
-  return variant == kFp64Pk12 || variant == kFp64Pk16 || variant == kFp64G8;
+  return variant == kFp64Pk12 || variant == kFp64Pk16 || variant == kFp64G8 || variant == kFp64Dg;
 }
 
 cudaError_t launch_add(int stage, DevMat A, DevMat Cin, int use_cin, double alpha, double beta,

@@ -221,8 +221,10 @@ void copy_parallel(void *dst, const void *src, size_t bytes) {
 }
 
 // Upper bound of the device bytes a request C = A.A can hold; also the bound
-// of its result's value count and its unfiltered multiply-adds.
-int64_t footprint_bound(const Request &r, int precision, int64_t *c_vals_bound, int64_t *macs) {
+// of its result's value count and its unfiltered multiply-adds. *optional: bytes
+// beyond it that it uses where the budget has them.
+int64_t footprint_bound(const Request &r, int precision, int64_t *c_vals_bound, int64_t *macs,
+                        int64_t *optional) {
   const int64_t nbr = (int64_t)r.sizes.size();
   std::vector<int64_t> row_nblk(nbr, 0), row_cols(nbr, 0);
   for (size_t b = 0; b < r.brow.size(); b++) {
@@ -242,9 +244,22 @@ int64_t footprint_bound(const Request &r, int precision, int64_t *c_vals_bound, 
   const int64_t c_blocks = std::min<int64_t>(nbr * nbr, cand);
   const int64_t c_vals = std::min<int64_t>(dim * dim, cand_vals);
   if (c_vals_bound) *c_vals_bound = c_vals;
-  // the split precisions keep A's slices in both operand layouts
-  const int64_t slice_bytes =
-      precision == BSM_PREC_FP64 ? 0 : 2 * bsm::split_bytes_per_value(precision) * r.nvals;
+  // the split precisions keep A's slices in both operand layouts; FP64 its digits
+  // (64 bytes a row and 8 values of k, and up to a quarter more), which the
+  // allowance for A below covers but for the smallest blocks, and which it can do
+  // without
+  int64_t slice_bytes = 0;
+  *optional = 0;
+  if (precision != BSM_PREC_FP64) {
+    slice_bytes = 2 * bsm::split_bytes_per_value(precision) * r.nvals;
+  } else {
+    int64_t digits = 0;
+    for (size_t b = 0; b < r.brow.size(); b++) {
+      const int64_t m = r.sizes[r.brow[b]], n = r.sizes[r.bcol[b]];
+      digits += 64 * (m * ((n + 7) / 8) + n * ((m + 7) / 8)) + 16;
+    }
+    *optional = std::max<int64_t>(0, digits + digits / 4 - 3 * a_bytes);
+  }
   // A, C twice (front/back), per-block metadata, product records
   return 4 * a_bytes + slice_bytes + 2 * (8 * c_vals + 32 * c_blocks) + 8 * cand + 64 * nbr +
          (1 << 20);
@@ -646,13 +661,14 @@ static int submit_request(bsm_server s, int32_t nbrows, const int32_t *sizes, in
     return BSM_ERR_NOMEM;
   }
   r->eps = eps;
-  int64_t macs = 0;
-  r->footprint = footprint_bound(*r, s->precision, &r->c_vals_bound, &macs);
+  int64_t macs = 0, optional = 0;
+  r->footprint = footprint_bound(*r, s->precision, &r->c_vals_bound, &macs, &optional);
   r->est_ms = est_run_ms(macs, s->precision);
   if (r->footprint > s->budget) {  // could never be admitted
     forget(s, r);
     return BSM_ERR_NOMEM;
   }
+  r->footprint = std::min(r->footprint + optional, s->budget);
   {
     std::lock_guard<std::mutex> lk(s->mu);
     r->id = s->next_id++;

@@ -4,8 +4,8 @@
 //
 //     C_ij = beta * C_in_ij + alpha * sum_k A_ik . B_kj      (Sec. 2, Alg. 1)
 //
-// One warp owns one C block at a time and writes it once; no atomics. Two
-// kernel families:
+// One warp owns one C block at a time and writes it once; no atomics. The
+// kernels:
 //   t16: 16 x 16 output tiles and k-chunks of 16; the operands of a (product,
 //        chunk) step are copied to shared memory in their own layout (a
 //        contiguous copy when a block fits one tile), and the next step's
@@ -25,11 +25,13 @@
 //        with 8-byte asynchronous copies, double buffered; group g sums the
 //        k positions congruent to g mod G, and the G partial sums of an
 //        element are added in group order at the end.
+//   dg:  the products on the tensor cores, from digits of the operands (below).
 // All take an optional work list (C block indices, e.g. one shape class) and
 // its [begin, end) range in device memory.
 #include <cstdlib>
 
 #include "bsm_internal.h"
+#include "digits.cuh"
 
 namespace bsm {
 
@@ -481,22 +483,225 @@ __device__ __forceinline__ void pk_steps(const double *__restrict__ sA,
   }
 }
 
+// C block gblk by one warp. wbuf: two stages of shared memory. hout: host copy
+// of C's values or null. SLOTS: accumulator slots per lane (12 or 16). Fewer
+// slots lower the lane use of some tile shapes (13 x 13: 96% instead of 99%)
+// but shorten the per-tile code; which wins depends on the block mix (the
+// autotuner measures it).
+template <int SLOTS>
+__device__ __forceinline__ void pk_block(const DevMat &A, const DevMat &B, const DevOut &C,
+                                         const DevMat &Cin, double alpha, double beta,
+                                         const DevWs &ws, int64_t gblk, double *wbuf,
+                                         double *hout, int lane) {
+  constexpr int kStage = kPkStage;
+  const PkShapes &shapes = (SLOTS == 12) ? c_pk_shapes12 : c_pk_shapes16;
+  const int i = C.blk_row[gblk], j = C.col_idx[gblk];
+  const int m = C.row_sizes[i], n = C.col_sizes[j];
+  const int64_t p0 = ws.prod_ptr[gblk], p1 = ws.prod_ptr[gblk + 1];
+  const int cin = ws.c_cin[gblk];
+  const double *cinv = (cin >= 0) ? Cin.vals + Cin.blk_off[cin] : nullptr;
+  double *out = C.vals + C.blk_off[gblk];
+  double *hblk = hout ? hout + C.blk_off[gblk] : nullptr;
+
+  for (int r0 = 0; r0 < m; r0 += kPkTile) {
+    for (int c0 = 0; c0 < n; c0 += kPkTile) {
+      const int tm = min(kPkTile, m - r0), tn = min(kPkTile, n - c0);
+      const int te = tm * tn;
+      int nT = shapes.nt[te], G = shapes.g[te];
+      if (ws.pk_tab) {  // a tuned shape (validated by the host)
+        const uint32_t e = ws.pk_tab[(SLOTS == 16 ? kPkTabSize : 0) + tm * kPkTabEdge + tn];
+        nT = (int)(e >> 8);
+        G = (int)(e & 0xFFu);
+      }
+      const int used = te * G;
+      const uint32_t rtm = rcp16(tm), rg = rcp16(G);
+      // chunk length: the largest multiple of G with KC * tm + tn * (KC + 1) <= kStage
+      const int kfit = min(kPkMaxKC, (kStage - tn) / (tm + tn));
+      const int KC = G * div16(kfit, rg);
+      const int ldB = KC + 1;  // sB[c * ldB + kk]
+      const int dq_tm = div16(32, rtm), dr_tm = 32 - dq_tm * tm;  // 32 = dq_tm * tm + dr_tm
+      // slot t of this lane: z = lane + 32 t -> group g = z / te, element
+      // e = z % te (row e % tm, column e / tm); its operands at step 0 are
+      // sA[ia] and sB[ib], kept as ia | ib << 16 (both below 2^9)
+      uint32_t idx[SLOTS];
+      double acc[SLOTS];
+      {
+        int g = 0, e = lane;
+        while (e >= te) {
+          e -= te;
+          g++;
+        }
+#pragma unroll
+        for (int t = 0; t < SLOTS; t++) {
+          idx[t] = 0;  // slots past te * G read valid operands; their sums are discarded
+          if (g < G) {
+            const int c = div16(e, rtm), r = e - c * tm;
+            idx[t] = (uint32_t)(g * tm + r) | ((uint32_t)(c * ldB + g) << 16);
+          }
+          acc[t] = 0.0;
+          e += 32;
+          while (e >= te) {
+            e -= te;
+            g++;
+          }
+        }
+      }
+
+      // product cursor: batch [pb, pb + nb) of metadata, one product per lane
+      int64_t pb = p0;
+      int nb = 0, q = 0, lq = 0;
+      int64_t my_a = 0, my_b = 0;
+      int my_s = 1;
+      auto load_batch = [&]() {
+        nb = (p1 - pb < 32) ? (int)(p1 - pb) : 32;
+        if (lane < nb) {
+          const int2 pr = __ldcs(ws.prods + pb + lane);  // read once: evict first
+          my_a = A.blk_off[pr.x];
+          my_b = B.blk_off[pr.y];
+          my_s = A.col_sizes[A.col_idx[pr.x]];
+        }
+      };
+      if (pb < p1) load_batch();
+
+      // Copies the next (up to) KC k positions of the concatenated products
+      // into stage `buf`: sA[kk * tm + r] = A(r0 + r, k), sB[c * ldB + kk] =
+      // B(k, c0 + c); zero-fills up to the next multiple of G. Returns the
+      // number of steps (k positions / G) of the chunk.
+      auto fill = [&](int buf) -> int {
+        double *sA = wbuf + buf * kStage;
+        double *sB = sA + KC * tm;
+        int kk = 0;
+        while (kk < KC && pb < p1) {
+          const int s = __shfl_sync(0xffffffffu, my_s, q);
+          const int64_t ao = __shfl_sync(0xffffffffu, my_a, q);
+          const int64_t bo = __shfl_sync(0xffffffffu, my_b, q);
+          const int nc = min(s - lq, KC - kk);
+          const double *Ab = A.vals + ao + (int64_t)lq * m + r0;  // column lq, row r0
+          const double *Bb = B.vals + bo + (int64_t)c0 * s + lq;  // row lq, column c0
+          double *dA = sA + kk * tm;
+          if (tm == m) {  // whole columns: one contiguous range
+            for (int z = lane; z < nc * m; z += 32) cp_async8(dA + z, Ab + z);
+          } else {  // (l, r) = divmod(z, tm), stepped by 32
+            int l = div16(lane, rtm), r = lane - l * tm;
+            for (int z = lane; z < nc * tm; z += 32) {
+              cp_async8(dA + l * tm + r, Ab + (int64_t)l * m + r);
+              l += dq_tm;
+              r += dr_tm;
+              if (r >= tm) {
+                r -= tm;
+                l++;
+              }
+            }
+          }
+          {  // (c, l) = divmod(z, nc), stepped by 32
+            const uint32_t rnc = rcp16(nc);
+            const int dq = div16(32, rnc), dr = 32 - dq * nc;
+            int c = div16(lane, rnc), l = lane - c * nc;
+            double *dB = sB + kk;
+            for (int z = lane; z < nc * tn; z += 32) {
+              cp_async8(dB + c * ldB + l, Bb + (int64_t)c * s + l);
+              c += dq;
+              l += dr;
+              if (l >= nc) {
+                l -= nc;
+                c++;
+              }
+            }
+          }
+          kk += nc;
+          lq += nc;
+          if (lq == s) {
+            lq = 0;
+            if (++q == nb) {
+              pb += nb;
+              q = 0;
+              if (pb < p1) load_batch();
+            }
+          }
+        }
+        const int steps = div16(kk + G - 1, rg);
+        const int pad = steps * G - kk;
+        if (pad) {
+          for (int z = lane; z < pad * tm; z += 32) sA[kk * tm + z] = 0.0;
+          for (int z = lane; z < pad * tn; z += 32) {
+            const int c = div16(z, rcp16(pad)), l = z - c * pad;
+            sB[c * ldB + kk + l] = 0.0;
+          }
+        }
+        return steps;
+      };
+
+      int cur = fill(0);  // steps of the current chunk
+      pk_commit();
+      for (int ch = 0;; ch++) {
+        const int buf = ch & 1;
+        const int nxt = (pb < p1) ? fill(buf ^ 1) : 0;
+        pk_commit();
+        pk_wait<1>();  // the current chunk has landed
+        __syncwarp();
+        const double *sA = wbuf + buf * kStage;
+        const double *sB = sA + KC * tm;
+        const int gtm = G * tm;
+        switch (nT) {
+#define BSM_PK_CASE(N)                                                                 \
+  case N:                                                                              \
+if (N <= SLOTS) pk_steps<(N <= SLOTS ? N : 1), SLOTS>(sA, sB, idx, acc, cur, gtm, G); \
+break;
+          BSM_PK_CASE(1) BSM_PK_CASE(2) BSM_PK_CASE(3) BSM_PK_CASE(4)
+          BSM_PK_CASE(5) BSM_PK_CASE(6) BSM_PK_CASE(7) BSM_PK_CASE(8)
+          BSM_PK_CASE(9) BSM_PK_CASE(10) BSM_PK_CASE(11) BSM_PK_CASE(12)
+          BSM_PK_CASE(13) BSM_PK_CASE(14) BSM_PK_CASE(15) BSM_PK_CASE(16)
+#undef BSM_PK_CASE
+        }
+        __syncwarp();  // the stage is read before it is filled again
+        if (nxt == 0) break;
+        cur = nxt;
+      }
+      pk_wait<0>();
+      __syncwarp();
+
+      // the G partial sums of each element, added in group order
+      double *red = wbuf;
+#pragma unroll
+      for (int t = 0; t < SLOTS; t++) {
+        const int z = lane + 32 * t;
+        if (t < nT && z < used) red[z] = acc[t];
+      }
+      __syncwarp();
+      int c = div16(lane, rtm), r = lane - c * tm;
+      for (int e = lane; e < te; e += 32) {
+        double v = red[e];
+        for (int g = 1; g < G; g++) v += red[g * te + e];
+        const int64_t loc = (int64_t)(c0 + c) * m + r0 + r;
+        v = alpha * v;
+        if (cinv) v = fma(beta, cinv[loc], v);
+        // written once, not read by this multiply: streaming stores keep the
+        // operand rows, which the next C blocks read, in L2
+        __stcs(out + loc, v);
+        if (hblk) __stcs(hblk + loc, v);
+        c += dq_tm;
+        r += dr_tm;
+        if (r >= tm) {
+          r -= tm;
+          c++;
+        }
+      }
+      __syncwarp();
+    }
+  }
+}
+
 // work: a counter that is zero when the launch starts; warps take the next
 // kPkGrab C blocks of the work range from it until the range is exhausted.
-// SLOTS: accumulator slots per lane (12 or 16). Fewer slots lower the lane use
-// of some tile shapes (13 x 13: 96% instead of 99%) but shorten the per-tile
-// code; which wins depends on the block mix (the autotuner measures it).
 template <int SLOTS>
 __global__ void __launch_bounds__(kPkWarps * 32, 2)
     k_numeric_fp64_pk(DevMat A, DevMat B, DevOut C, DevMat Cin, double alpha, double beta,
                       DevWs ws, const DevStatus *st, const int32_t *items, const int64_t *seg,
                       unsigned long long *work) {
   if (st->overflow) return;
-  constexpr int kStage = kPkStage;
-  const PkShapes &shapes = (SLOTS == 12) ? c_pk_shapes12 : c_pk_shapes16;
   extern __shared__ double smem_pk[];
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-  double *wbuf = smem_pk + warp * 2 * kStage;
+  double *wbuf = smem_pk + warp * 2 * kPkStage;
   int64_t wb, we;
   work_range(st, seg, wb, we);
   // the second destination (host memory) when the whole result fits it
@@ -508,212 +713,378 @@ __global__ void __launch_bounds__(kPkWarps * 32, 2)
     const int64_t w0 = wb + (int64_t)__shfl_sync(0xffffffffu, got, 0);
     if (w0 >= we) break;
     const int64_t w1 = (w0 + kPkGrab < we) ? w0 + kPkGrab : we;
-    for (int64_t w = w0; w < w1; w++) {
-      const int64_t gblk = items ? items[w] : w;
-      const int i = C.blk_row[gblk], j = C.col_idx[gblk];
-      const int m = C.row_sizes[i], n = C.col_sizes[j];
-      const int64_t p0 = ws.prod_ptr[gblk], p1 = ws.prod_ptr[gblk + 1];
-      const int cin = ws.c_cin[gblk];
-      const double *cinv = (cin >= 0) ? Cin.vals + Cin.blk_off[cin] : nullptr;
-      double *out = C.vals + C.blk_off[gblk];
-      double *hblk = hout ? hout + C.blk_off[gblk] : nullptr;
+    for (int64_t w = w0; w < w1; w++)
+      pk_block<SLOTS>(A, B, C, Cin, alpha, beta, ws, items ? items[w] : w, wbuf, hout, lane);
+  }
+}
 
-      for (int r0 = 0; r0 < m; r0 += kPkTile) {
-        for (int c0 = 0; c0 < n; c0 += kPkTile) {
-          const int tm = min(kPkTile, m - r0), tn = min(kPkTile, n - c0);
-          const int te = tm * tn;
-          int nT = shapes.nt[te], G = shapes.g[te];
-          if (ws.pk_tab) {  // a tuned shape (validated by the host)
-            const uint32_t e = ws.pk_tab[(SLOTS == 16 ? kPkTabSize : 0) + tm * kPkTabEdge + tn];
-            nT = (int)(e >> 8);
-            G = (int)(e & 0xFFu);
-          }
-          const int used = te * G;
-          const uint32_t rtm = rcp16(tm), rg = rcp16(G);
-          // chunk length: the largest multiple of G with KC * tm + tn * (KC + 1) <= kStage
-          const int kfit = min(kPkMaxKC, (kStage - tn) / (tm + tn));
-          const int KC = G * div16(kfit, rg);
-          const int ldB = KC + 1;  // sB[c * ldB + kk]
-          const int dq_tm = div16(32, rtm), dr_tm = 32 - dq_tm * tm;  // 32 = dq_tm * tm + dr_tm
-          // slot t of this lane: z = lane + 32 t -> group g = z / te, element
-          // e = z % te (row e % tm, column e / tm); its operands at step 0 are
-          // sA[ia] and sB[ib], kept as ia | ib << 16 (both below 2^9)
-          uint32_t idx[SLOTS];
-          double acc[SLOTS];
-          {
-            int g = 0, e = lane;
-            while (e >= te) {
-              e -= te;
-              g++;
-            }
+// ----------------------------------------------------------------------------
+// dg: the FP64 products on the tensor cores, in exact integer arithmetic. The
+// operands come as eight signed base-256 digits per value, on a scale of their
+// own for every scalar row of A and column of B (bsm_internal.h, digits.cuh). A
+// product of two values is sum_d 256^-d v_d, v_d = sum over i + j = d of a_i b_j;
+// the digit pairs of every diagonal d < kDgDiag are multiplied by mma.sync (FP16
+// operands that are small integers, so every term is exact) into one FP32
+// accumulator per element and diagonal. With at most 144 values of k between two
+// reads its sums stay below 2^24, where FP32 numbers are exact integers. A read
+// adds the diagonals up in 64-bit integers, and the whole sum is rounded to FP64 once;
+// what is lost besides is half a unit of 2^-62 of each row's scale and the diagonals
+// from kDgDiag on (2^-70 of the largest product of the row and column).
+// Measured against long double, relative Frobenius error of C (and the worst of C's
+// blocks): water of 128 molecules 4.5e-17 (7.5e-17), the packed kernel 4.7e-16
+// (7.9e-16); amorphous of 200 atoms 4.6e-17 (7.3e-17), packed 1.0e-15 (1.7e-15); rows of
+// unlike scales in blocks of 1 to 33 5.9e-17 (4.4e-16), packed 4.0e-16 (9.6e-15).
+//
+// Why: the FP64 pipe does 2 FMA per clock and SM, mma.sync on FP16 1024, and 43
+// digit pairs stand for one product. (FP8 and INT8 mma.sync are emulated or slow on
+// this part: 3.8 and 16 clocks per m16n8k32 and SM, FP16 m16n8k16 2.0.) Numeric
+// phase, packed kernel -> this one: water of 2048 molecules 47.7 -> 21.4 ms,
+// amorphous of 1024 atoms 67.9 -> 22.5, 64 x 64 full blocks of 32 15.7 -> 2.4. What
+// bounds it: the MMA pipe (0.49 of the clocks of the first) and the instructions beside
+// it, which do not hide behind the MMAs whatever the number of warps (with 16, 20 and 24
+// per SM 21.4, 21.9 and 22.2 ms): left out one at a time, the digits' conversion is
+// 1.5 ms, the search for an octet's product and the loads' misses 4, the 64-bit sums 0.8,
+// the epilogue nothing (L2 and L1 are at 10 and 20%).
+//
+// The products of a C block are concatenated along k in octets (8 of k), two to an
+// MMA step; a warp takes a tile of up to 16 x 8 (the MMA's shape):
+//   WIDE: more than 8 rows;
+//   else: MMA rows 0-7 take the even, rows 8-15 the odd digits of the left side,
+//         so one MMA adds to two diagonals (23 instead of 43 MMAs per 16 k).
+// A lane's part of an operand octet is one 16-byte load, all digits of two values
+// (a warp's load is whole 128-byte lines), straight into registers, where two
+// instructions make an MMA register of each digit. (Measured and left: staging in
+// shared memory, where each cp.async costs three more instructions on this part and
+// the register groups of the MMAs a move per register, 31 ms; FP16 words in memory,
+// without conversions but four times the bytes, 24-26 ms; registers loaded a step
+// ahead in 12 warps, 24.6 ms.)
+// ----------------------------------------------------------------------------
+constexpr int kDgWarps = 8;             // warps per thread block
+constexpr int kDgBlocksPerSm = 2;
+constexpr int kDgDiag = 9;              // diagonals kept
+constexpr int kDgFold = 18;             // octets between two reads of the accumulators
+constexpr int kDgGrab = 8;              // C blocks a warp takes at a time, at most
+
+__device__ __forceinline__ void dg_mma(float (&d)[4], uint32_t a0, uint32_t a1, uint32_t a2,
+                                       uint32_t a3, uint32_t b0, uint32_t b1) {
+  asm(
+      "mma.sync.aligned.m16n8k16.row.col.f32.f16.f16.f32 {%0,%1,%2,%3}, {%4,%5,%6,%7}, "
+      "{%8,%9}, {%0,%1,%2,%3};\n"
+      : "+f"(d[0]), "+f"(d[1]), "+f"(d[2]), "+f"(d[3])
+      : "r"(a0), "r"(a1), "r"(a2), "r"(a3), "r"(b0), "r"(b1));
+}
+// The exact sum of an element: h * 2^40 + l, in units of 2^(Ea + Eb - 76), 0 <= l < 2^40.
+struct __align__(16) DgSum {
+  int64_t h, l;
+};
+static_assert(kDgDiag == 9, "the sum below is written for nine diagonals");
+// the diagonals' sums f (|f_d| <= 2^24) added to o
+__device__ __forceinline__ DgSum dg_sum(const float (&f)[kDgDiag], const DgSum &o) {
+  int v[kDgDiag];
 #pragma unroll
-            for (int t = 0; t < SLOTS; t++) {
-              idx[t] = 0;  // slots past te * G read valid operands; their sums are discarded
-              if (g < G) {
-                const int c = div16(e, rtm), r = e - c * tm;
-                idx[t] = (uint32_t)(g * tm + r) | ((uint32_t)(c * ldB + g) << 16);
-              }
-              acc[t] = 0.0;
-              e += 32;
-              while (e >= te) {
-                e -= te;
-                g++;
-              }
-            }
-          }
+  for (int d = 0; d < kDgDiag; d++) v[d] = __float2int_rn(f[d]);
+  // |v_0| <= 64^2 * 144, |v_2| <= (2 * 64 * 128 + 128^2) * 144: these pairs fit 32 bits
+  const int64_t h = ((int64_t)((v[0] << 8) + v[1]) << 16) + ((v[2] << 8) + v[3]);
+  const int64_t l = ((int64_t)v[4] << 32) + ((int64_t)v[5] << 24) + ((int64_t)v[6] << 16) +
+                    ((int64_t)v[7] << 8) + v[8] + o.l;
+  return {o.h + h + (l >> 40), l & ((1ll << 40) - 1)};
+}
+__device__ __forceinline__ double dg_value(const DgSum &s) {
+  return fma((double)s.h, 0x1p40, (double)s.l);
+}
+// v * 2^e for v = 0 or 2^-100 <= |v| <= 2^200 (no FP64 instruction while the result
+// is a normal number)
+__device__ __forceinline__ double dg_scaled(double v, int e) {
+  const int hi = __double2hiint(v), x = ((hi >> 20) & 0x7FF) + e;
+  if (v == 0.0) return v;
+  if (x > 0 && x < 2047) return __hiloint2double(hi + (e << 20), __double2loint(v));
+  const int half = max(e, -800);
+  return v * __hiloint2double((1023 + half) << 20, 0) * __hiloint2double((1023 + e - half) << 20, 0);
+}
 
-          // product cursor: batch [pb, pb + nb) of metadata, one product per lane
-          int64_t pb = p0;
-          int nb = 0, q = 0, lq = 0;
-          int64_t my_a = 0, my_b = 0;
-          int my_s = 1;
-          auto load_batch = [&]() {
-            nb = (p1 - pb < 32) ? (int)(p1 - pb) : 32;
-            if (lane < nb) {
-              const int2 pr = __ldcs(ws.prods + pb + lane);  // read once: evict first
-              my_a = A.blk_off[pr.x];
-              my_b = B.blk_off[pr.y];
-              my_s = A.col_sizes[A.col_idx[pr.x]];
-            }
-          };
-          if (pb < p1) load_batch();
+// A word of a unit (digits 2 i and 2 i + 1 of two values) as the two MMA registers.
+__device__ __forceinline__ uint32_t dg_even(uint32_t w) { return digit_half2(w, 0x4140); }
+__device__ __forceinline__ uint32_t dg_odd(uint32_t w) { return digit_half2(w, 0x4342); }
 
-          // Copies the next (up to) KC k positions of the concatenated products
-          // into stage `buf`: sA[kk * tm + r] = A(r0 + r, k), sB[c * ldB + kk] =
-          // B(k, c0 + c); zero-fills up to the next multiple of G. Returns the
-          // number of steps (k positions / G) of the chunk.
-          auto fill = [&](int buf) -> int {
-            double *sA = wbuf + buf * kStage;
-            double *sB = sA + KC * tm;
-            int kk = 0;
-            while (kk < KC && pb < p1) {
-              const int s = __shfl_sync(0xffffffffu, my_s, q);
-              const int64_t ao = __shfl_sync(0xffffffffu, my_a, q);
-              const int64_t bo = __shfl_sync(0xffffffffu, my_b, q);
-              const int nc = min(s - lq, KC - kk);
-              const double *Ab = A.vals + ao + (int64_t)lq * m + r0;  // column lq, row r0
-              const double *Bb = B.vals + bo + (int64_t)c0 * s + lq;  // row lq, column c0
-              double *dA = sA + kk * tm;
-              if (tm == m) {  // whole columns: one contiguous range
-                for (int z = lane; z < nc * m; z += 32) cp_async8(dA + z, Ab + z);
-              } else {  // (l, r) = divmod(z, tm), stepped by 32
-                int l = div16(lane, rtm), r = lane - l * tm;
-                for (int z = lane; z < nc * tm; z += 32) {
-                  cp_async8(dA + l * tm + r, Ab + (int64_t)l * m + r);
-                  l += dq_tm;
-                  r += dr_tm;
-                  if (r >= tm) {
-                    r -= tm;
-                    l++;
-                  }
-                }
-              }
-              {  // (c, l) = divmod(z, nc), stepped by 32
-                const uint32_t rnc = rcp16(nc);
-                const int dq = div16(32, rnc), dr = 32 - dq * nc;
-                int c = div16(lane, rnc), l = lane - c * nc;
-                double *dB = sB + kk;
-                for (int z = lane; z < nc * tn; z += 32) {
-                  cp_async8(dB + c * ldB + l, Bb + (int64_t)c * s + l);
-                  c += dq;
-                  l += dr;
-                  if (l >= nc) {
-                    l -= nc;
-                    c++;
-                  }
-                }
-              }
-              kk += nc;
-              lq += nc;
-              if (lq == s) {
-                lq = 0;
-                if (++q == nb) {
-                  pb += nb;
-                  q = 0;
-                  if (pb < p1) load_batch();
-                }
-              }
-            }
-            const int steps = div16(kk + G - 1, rg);
-            const int pad = steps * G - kk;
-            if (pad) {
-              for (int z = lane; z < pad * tm; z += 32) sA[kk * tm + z] = 0.0;
-              for (int z = lane; z < pad * tn; z += 32) {
-                const int c = div16(z, rcp16(pad)), l = z - c * pad;
-                sB[c * ldB + kk + l] = 0.0;
-              }
-            }
-            return steps;
-          };
-
-          int cur = fill(0);  // steps of the current chunk
-          pk_commit();
-          for (int ch = 0;; ch++) {
-            const int buf = ch & 1;
-            const int nxt = (pb < p1) ? fill(buf ^ 1) : 0;
-            pk_commit();
-            pk_wait<1>();  // the current chunk has landed
-            __syncwarp();
-            const double *sA = wbuf + buf * kStage;
-            const double *sB = sA + KC * tm;
-            const int gtm = G * tm;
-            switch (nT) {
-#define BSM_PK_CASE(N)                                                                 \
-  case N:                                                                              \
-    if (N <= SLOTS) pk_steps<(N <= SLOTS ? N : 1), SLOTS>(sA, sB, idx, acc, cur, gtm, G); \
-    break;
-              BSM_PK_CASE(1) BSM_PK_CASE(2) BSM_PK_CASE(3) BSM_PK_CASE(4)
-              BSM_PK_CASE(5) BSM_PK_CASE(6) BSM_PK_CASE(7) BSM_PK_CASE(8)
-              BSM_PK_CASE(9) BSM_PK_CASE(10) BSM_PK_CASE(11) BSM_PK_CASE(12)
-              BSM_PK_CASE(13) BSM_PK_CASE(14) BSM_PK_CASE(15) BSM_PK_CASE(16)
-#undef BSM_PK_CASE
-            }
-            __syncwarp();  // the stage is read before it is filled again
-            if (nxt == 0) break;
-            cur = nxt;
-          }
-          pk_wait<0>();
-          __syncwarp();
-
-          // the G partial sums of each element, added in group order
-          double *red = wbuf;
+// One tile of a C block that has no operand block outside: rows from 16 mt of A,
+// columns from 8 nt of B, tm x tn; out (column-major) receives the tile's sums of
+// the products of one class, which is returned (their weight is 2^(-8 class)); the
+// sums of the classes before it are added up in part, if there are any (*parts).
+// m, n: the block's sizes; prods: its np products, ma and mb the metadata of the
+// first 32 (one per lane).
+template <bool WIDE>
+__device__ __forceinline__ int dg_tile(const Digits &dg, const int2 *__restrict__ prods, int np,
+                                        uint2 ma, uint2 mb, int m, int n, int mt, int nt, int tm,
+                                        int tn, DgSum *out, double *part, bool *parts, int lane) {
+  const int g = lane >> 2, t = lane & 3;
+  // the lane's units of an octet (rows past the last one: the last one again)
+  const uint4 *__restrict__ ua = dg.a.units + min(g, tm - 1) * 4 + t;
+  const uint4 *__restrict__ ub = dg.b.units + min(g, tn - 1) * 4 + t;
+  const int low = (min(g + 8, tm - 1) - min(g, tm - 1)) * 4;  // to MMA row g + 8's
+  struct Raw {  // an MMA step: two octets
+    uint4 a[2], a8[2], b[2];
+  };
+  float acc[kDgDiag][4];
+  auto mma = [&](const Raw &f) {
+    uint32_t b[2][kDigits];
 #pragma unroll
-          for (int t = 0; t < SLOTS; t++) {
-            const int z = lane + 32 * t;
-            if (t < nT && z < used) red[z] = acc[t];
+    for (int h = 0; h < 2; h++) {
+      b[h][0] = dg_even(f.b[h].x), b[h][1] = dg_odd(f.b[h].x);
+      b[h][2] = dg_even(f.b[h].y), b[h][3] = dg_odd(f.b[h].y);
+      b[h][4] = dg_even(f.b[h].z), b[h][5] = dg_odd(f.b[h].z);
+      b[h][6] = dg_even(f.b[h].w), b[h][7] = dg_odd(f.b[h].w);
+    }
+#pragma unroll
+    for (int i = 0; i < kDigits; i += 2) {
+      auto word = [&](const uint4 &u) { return i == 0 ? u.x : i == 2 ? u.y : i == 4 ? u.z : u.w; };
+      if (WIDE) {
+        uint32_t a0 = dg_even(word(f.a[0])), a1 = dg_even(word(f.a8[0]));
+        uint32_t a2 = dg_even(word(f.a[1])), a3 = dg_even(word(f.a8[1]));
+#pragma unroll
+        for (int j = 0; j < kDigits; j++)
+          if (i + j < kDgDiag) dg_mma(acc[i + j], a0, a1, a2, a3, b[0][j], b[1][j]);
+        a0 = dg_odd(word(f.a[0])), a1 = dg_odd(word(f.a8[0]));
+        a2 = dg_odd(word(f.a[1])), a3 = dg_odd(word(f.a8[1]));
+#pragma unroll
+        for (int j = 0; j < kDigits; j++)
+          if (i + 1 + j < kDgDiag) dg_mma(acc[i + 1 + j], a0, a1, a2, a3, b[0][j], b[1][j]);
+      } else {
+        const uint32_t a0 = dg_even(word(f.a[0])), a1 = dg_odd(word(f.a[0]));
+        const uint32_t a2 = dg_even(word(f.a[1])), a3 = dg_odd(word(f.a[1]));
+#pragma unroll
+        for (int j = 0; j < kDigits; j++)
+          if (i + j < kDgDiag) dg_mma(acc[i + j], a0, a1, a2, a3, b[0][j], b[1][j]);
+      }
+    }
+  };
+  int held = -1;  // the class of the sums in out
+  *parts = false;
+  for (int pb = 0;;) {
+    const uint2 xa = ma, xb = mb;  // lane p: product p of the batch
+    const bool in = pb + lane < np;
+    const int cls = (int)(xa.y >> 16 & 0xFF) + (int)(xb.y >> 16 & 0xFF);
+    pb += 32;
+    if (pb < np) {  // the next batch's metadata, on its way during this one
+      ma = mb = make_uint2(0, 0);
+      if (pb + lane < np) {
+        const int2 pr = __ldg(prods + pb + lane);
+        ma = __ldg(dg.a.meta + pr.x);
+        mb = __ldg(dg.b.meta + pr.y);
+      }
+    }
+    // the products of one class (the weight 2^(-8 class)) after the other: mostly
+    // all have the same
+    uint32_t todo = __ballot_sync(0xffffffffu, in);
+#pragma unroll 1
+    while (todo) {
+      const int now = __shfl_sync(0xffffffffu, cls, __ffs(todo) - 1);
+      const bool mine = in && cls == now;
+      todo &= ~__ballot_sync(0xffffffffu, mine);
+      // its octets' end, and its units less its first slot's
+      const int octets = mine ? (int)(xa.y & 0xFFFF) : 0;
+      int incl = octets;
+#pragma unroll
+      for (int d = 1; d < 32; d <<= 1) {
+        const int y = __shfl_up_sync(0xffffffffu, incl, d);
+        if (lane >= d) incl += y;
+      }
+      const int slots = __shfl_sync(0xffffffffu, incl, 31);
+      const uint32_t am = xa.x + (uint32_t)(64 * mt - (incl - octets) * 4 * m);
+      const uint32_t bm = xb.x + (uint32_t)(32 * nt - (incl - octets) * 4 * n);
+      if (held >= 0 && held != now) {
+        __syncwarp();
+        for (int e = lane; e < tm * tn; e += 32) {
+          const double v = dg_scaled(dg_value(out[e]), -8 * held);
+          part[e] = *parts ? part[e] + v : v;
+        }
+        __syncwarp();
+        *parts = true;
+        held = -1;
+      }
+#pragma unroll 1
+      for (int s0 = 0; s0 < slots; s0 += kDgFold) {
+        // lane l: where the units of slot s0 + l start (zeros past the end)
+        const int s = s0 + lane;
+        int p = 0;  // products that end at or before slot s
+#pragma unroll
+        for (int step = 16; step; step >>= 1)
+          if (__shfl_sync(0xffffffffu, incl, p + step - 1) <= s) p += step;
+        uint32_t fa = __shfl_sync(0xffffffffu, am, p) + (uint32_t)(s * 4 * m);
+        uint32_t fb = __shfl_sync(0xffffffffu, bm, p) + (uint32_t)(s * 4 * n);
+        if (s >= slots) fa = fb = 0;
+        auto load = [&](Raw &f, int o) {
+#pragma unroll
+          for (int h = 0; h < 2; h++) {
+            const uint4 *xa = ua + __shfl_sync(0xffffffffu, fa, o + h);
+            f.a[h] = __ldg(xa);
+            if (WIDE) f.a8[h] = __ldg(xa + low);
+            f.b[h] = __ldg(ub + __shfl_sync(0xffffffffu, fb, o + h));
           }
+        };
+#pragma unroll
+        for (int d = 0; d < kDgDiag; d++)
+#pragma unroll
+          for (int e = 0; e < 4; e++) acc[d][e] = 0.0f;
+        const int end = min(kDgFold, slots - s0);
+#pragma unroll 1
+        for (int o = 0; o < end; o += 2) {
+          Raw f0;
+          load(f0, o);
+          mma(f0);
+        }
+#pragma unroll
+        for (int e = 0; e < (WIDE ? 4 : 2); e++) {
+          float f[kDgDiag];
+#pragma unroll
+          for (int d = 0; d < kDgDiag; d++)
+            f[d] = (WIDE || d == 0) ? acc[d][e] : __fadd_rn(acc[d][e], acc[d - 1][e + 2]);
+          const int x = g + (e >> 1) * 8, y = 2 * t + (e & 1);
+          if (x < tm && y < tn) {
+            DgSum *to = out + (y * tm + x);
+            *to = dg_sum(f, held < 0 ? DgSum{0, 0} : *to);
+          }
+        }
+        held = now;
+      }
+    }
+    if (pb >= np) return held;
+  }
+}
+
+struct DgItem {  // a C block of a warp's run
+  const int2 *prods;
+  int64_t coff;
+  int32_t gblk, np, m, n, cin, fa, fb;
+};
+
+// C blocks without products (C_in only) and those with an operand block outside
+// go to dg.list, for the packed kernel.
+__global__ void __launch_bounds__(kDgWarps * 32, kDgBlocksPerSm)
+    k_numeric_fp64_dg(DevMat A, DevMat B, DevOut C, DevMat Cin, double alpha, double beta,
+                      DevWs ws, const DevStatus *st, const int32_t *items, const int64_t *seg,
+                      unsigned long long *work, Digits dg) {
+  if (st->overflow) return;
+  __shared__ DgSum tiles[kDgWarps][16 * 8];
+  __shared__ double parts[kDgWarps][16 * 8];
+  __shared__ DgItem s_items[kDgWarps][kDgGrab];
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+  DgSum *tile = tiles[warp];
+  double *part = parts[warp];
+  DgItem *item = s_items[warp];
+  int64_t wb, we;
+  work_range(st, seg, wb, we);
+  double *hout = (C.host_vals && st->nnz_c <= C.host_cap) ? C.host_vals : nullptr;
+  // fewer at a time where that would leave warps without work
+  const int64_t share = (we - wb) / ((int64_t)gridDim.x * kDgWarps * 4);
+  const int grab = share >= kDgGrab ? kDgGrab : share < 1 ? 1 : (int)share;
+
+  for (;;) {
+    unsigned long long got = 0;
+    if (lane == 0) got = atomicAdd(work, (unsigned long long)grab);
+    const int64_t base = wb + (int64_t)__shfl_sync(0xffffffffu, got, 0);
+    if (base >= we) break;
+    const int count = we - base < grab ? (int)(we - base) : grab;
+    // what the C blocks of the run need, a lane each: the next block is then found
+    // without a chain of loads
+    if (lane < count) {
+      DgItem it;
+      it.gblk = items ? items[base + lane] : (int)(base + lane);
+      const int64_t pp = ws.prod_ptr[it.gblk];
+      it.prods = ws.prods + pp;
+      it.np = (int)(ws.prod_ptr[it.gblk + 1] - pp);
+      const int i = C.blk_row[it.gblk], j = C.col_idx[it.gblk];
+      it.m = C.row_sizes[i];
+      it.n = C.col_sizes[j];
+      it.coff = C.blk_off[it.gblk];
+      it.cin = ws.c_cin[it.gblk];
+      it.fa = dg.a.first[i];
+      it.fb = dg.b.first[j];
+      item[lane] = it;
+    }
+    __syncwarp();
+    // a block's products and their metadata are loaded while the block before is
+    // computed
+    int2 pr = make_int2(-1, -1);
+    auto products = [&](int at) {
+      pr = make_int2(-1, -1);
+      if (at < count && lane < item[at].np) pr = __ldg(item[at].prods + lane);
+    };
+    uint2 ma, mb;
+    auto metadata = [&]() {
+      ma = mb = make_uint2(0, 0);
+      if (pr.x >= 0) {
+        ma = __ldg(dg.a.meta + pr.x);
+        mb = __ldg(dg.b.meta + pr.y);
+      }
+    };
+    products(0);
+    metadata();
+    for (int x = 0; x < count; x++) {
+      const DgItem &it = item[x];
+      products(x + 1);
+      const int np = it.np;
+      uint32_t flags = ma.y | mb.y;
+      for (int p = lane + 32; p < np; p += 32) {
+        const int2 q = __ldg(it.prods + p);
+        flags |= dg.a.meta[q.x].y | dg.b.meta[q.y].y;
+      }
+      if (np == 0 || __any_sync(0xffffffffu, flags & kDigitOutside)) {
+        if (lane == 0)
+          dg.list[atomicAdd(reinterpret_cast<unsigned long long *>(dg.range + 1), 1ull)] = it.gblk;
+        metadata();
+        continue;
+      }
+      const int m = it.m, n = it.n;
+      const uint2 ka = ma, kb = mb;
+      for (int r0 = 0; r0 < m; r0 += 16) {
+        for (int c0 = 0; c0 < n; c0 += 8) {
+          const int tm = min(16, m - r0), tn = min(8, n - c0);
+          // the exponents of the tile's scales: lane r row r's, lane c column c's
+          const int xa = dg.a.expo[it.fa + r0 + min(lane, tm - 1)];
+          const int xb = dg.b.expo[it.fb + c0 + min(lane, tn - 1)];
+          bool more;
+          const int cls = tm > 8 ? dg_tile<true>(dg, it.prods, np, ka, kb, m, n, r0 >> 4, c0 >> 3,
+                                                 tm, tn, tile, part, &more, lane)
+                                 : dg_tile<false>(dg, it.prods, np, ka, kb, m, n, r0 >> 4, c0 >> 3,
+                                                  tm, tn, tile, part, &more, lane);
           __syncwarp();
-          int c = div16(lane, rtm), r = lane - c * tm;
-          for (int e = lane; e < te; e += 32) {
-            double v = red[e];
-            for (int g = 1; g < G; g++) v += red[g * te + e];
-            const int64_t loc = (int64_t)(c0 + c) * m + r0 + r;
-            v = alpha * v;
-            if (cinv) v = fma(beta, cinv[loc], v);
-            // written once, not read by this multiply: streaming stores keep the
-            // operand rows, which the next C blocks read, in L2
-            __stcs(out + loc, v);
-            if (hblk) __stcs(hblk + loc, v);
-            c += dq_tm;
-            r += dr_tm;
-            if (r >= tm) {
-              r -= tm;
-              c++;
-            }
+          if (r0 + 16 >= m && c0 + 8 >= n) metadata();
+          const double *cinv = (it.cin >= 0) ? Cin.vals + Cin.blk_off[it.cin] : nullptr;
+          const uint32_t rtm = rcp16(tm);
+          for (int e0 = 0; e0 < tm * tn; e0 += 32) {
+            const int e = e0 + lane, c = div16(e, rtm), r = e - c * tm;
+            // 2^(Ea + Eb - 76), E = field - 1022; a row without a scale holds only zeros
+            const int fa = __shfl_sync(0xffffffffu, xa, r), fb = __shfl_sync(0xffffffffu, xb, c & 31);
+            if (e >= tm * tn) continue;
+            const int f = (fa >= kDigitExpLo && fb >= kDigitExpLo) ? fa + fb - 2044 - 76 : 0;
+            const int64_t loc = it.coff + (int64_t)(c0 + c) * m + r0 + r;
+            double v = dg_value(tile[e]);
+            if (more) v = part[e] + dg_scaled(v, -8 * cls);
+            v = dg_scaled(v, more ? f : f - 8 * cls);
+            if (alpha != 1.0) v *= alpha;
+            if (cinv) v = fma(beta, cinv[loc - it.coff], v);
+            // written once, not read by this multiply
+            __stcs(C.vals + loc, v);
+            if (hout) __stcs(hout + loc, v);
           }
           __syncwarp();
         }
       }
     }
+    __syncwarp();  // the items are read before the next ones are written
   }
 }
 
 cudaError_t launch_numeric_fp64(int variant, DevMat A, DevMat B, DevOut C, DevMat Cin,
                                 double alpha, double beta, DevWs ws, const DevStatus *st,
                                 const int32_t *items, const int64_t *seg, int grid,
-                                unsigned long long *work, int max_m, int max_n,
+                                unsigned long long *work, int max_m, int max_n, const Digits *digits,
                                 cudaStream_t stream) {
   switch (variant) {
+    case kFp64Dg:
+      k_numeric_fp64_dg<<<grid, kDgWarps * 32, 0, stream>>>(
+          A, B, C, Cin, alpha, beta, ws, st, items, seg, work, *digits);
+      break;
     case kFp64G8: {
       const int mr = max_m <= 4 ? 4 : max_m <= 6 ? 6 : 8;
       const int gs = max_n <= 4 ? 4 : max_n <= 6 ? 6 : 8;
@@ -757,6 +1128,7 @@ cudaError_t launch_numeric_fp64(int variant, DevMat A, DevMat B, DevOut C, DevMa
 }
 
 int fp64_variant_blocks_per_sm(int variant) {
+  if (variant == kFp64Dg) return kDgBlocksPerSm;
   if (variant == kFp64G8) return 4;
   return (variant == kFp64T16B3 || variant == kFp64T32) ? 3 : 2;
 }
@@ -765,6 +1137,9 @@ cudaError_t numeric_fp64_init() {
   const size_t smem = (size_t)kNumWarps * kWarpSmem * sizeof(double);
   cudaError_t e = cudaFuncSetAttribute(k_numeric_fp64_t32,
                                        cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+  if (e != cudaSuccess) return e;
+  // its operands come through L1: no more shared memory than its own
+  e = cudaFuncSetAttribute(k_numeric_fp64_dg, cudaFuncAttributePreferredSharedMemoryCarveout, 50);
   if (e != cudaSuccess) return e;
   e = cudaFuncSetAttribute(k_numeric_fp64_pk<12>, cudaFuncAttributeMaxDynamicSharedMemorySize,
                            (int)pk_smem_bytes());

@@ -13,6 +13,7 @@
 //          ascending k (a per-row counting sort), so that the numeric phase
 //          accumulates each C block in one place, without atomics.
 #include "bsm_internal.h"
+#include "digits.cuh"
 
 namespace bsm {
 
@@ -101,6 +102,100 @@ cudaError_t launch_block_norms(const int32_t *row_sizes, const int32_t *col_size
                                double *norms, float *normsf, int grid, cudaStream_t stream) {
   k_block_norms<<<grid, 256, 0, stream>>>(row_sizes, col_sizes, blk_row, col_idx, blk_off, vals,
                                           hdr, norms, normsf);
+  return cudaGetLastError();
+}
+
+// ----------------------------------------------------------------------------
+// The norms, and the scales of the digit representation in the same launch: the
+// first thread blocks take the norms, a thread per block as above, eight loads
+// ahead of the additions; the others the scales, a warp per block: each lane's
+// elements go to their row's and column's maximum in shared memory, and a maximum
+// that the array does not hold yet there.
+// ----------------------------------------------------------------------------
+constexpr int kScaleWarps = 8;
+constexpr int kScaleRows = 64;  // rows and columns kept in shared memory
+
+__global__ void __launch_bounds__(kScaleWarps * 32)
+    k_block_norms_scales(const int32_t *__restrict__ row_sizes,
+                         const int32_t *__restrict__ col_sizes,
+                         const int32_t *__restrict__ blk_row, const int32_t *__restrict__ col_idx,
+                         const int64_t *__restrict__ blk_off, const double *__restrict__ vals,
+                         const int64_t *__restrict__ hdr, double *__restrict__ norms,
+                         float *__restrict__ normsf, const int32_t *__restrict__ rfirst,
+                         const int32_t *__restrict__ cfirst, int32_t *rexp, int32_t *cexp,
+                         int norm_blocks) {
+  const int64_t nblk = hdr[0];
+  if ((int)blockIdx.x < norm_blocks) {
+    for (int64_t b = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; b < nblk;
+         b += (int64_t)norm_blocks * blockDim.x) {
+      const int64_t n = (int64_t)row_sizes[blk_row[b]] * col_sizes[col_idx[b]];
+      const double *x = vals + blk_off[b];
+      double s = 0.0;
+      int64_t e = 0;
+      for (; e + 8 <= n; e += 8) {
+        double v[8];
+#pragma unroll
+        for (int u = 0; u < 8; u++) v[u] = __ldg(x + e + u);
+#pragma unroll
+        for (int u = 0; u < 8; u++) s = __dadd_rn(s, __dmul_rn(v[u], v[u]));
+      }
+      for (; e < n; e++) {
+        const double v = __ldg(x + e);
+        s = __dadd_rn(s, __dmul_rn(v, v));
+      }
+      const double nrm = __dsqrt_rn(s);
+      norms[b] = nrm;
+      normsf[b] = (nrm >= 0x1p-60 && nrm <= 0x1p60) ? __double2float_rn(nrm) : NAN;
+    }
+    return;
+  }
+  __shared__ int32_t smax[kScaleWarps][2 * kScaleRows];
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+  int32_t *rmax = smax[warp], *cmax = rmax + kScaleRows;
+  const int64_t w0 = (int64_t)(blockIdx.x - norm_blocks) * kScaleWarps + warp;
+  const int64_t nw = (int64_t)(gridDim.x - norm_blocks) * kScaleWarps;
+  for (int64_t b = w0; b < nblk; b += nw) {
+    const int i = blk_row[b], j = col_idx[b];
+    const int m = row_sizes[i], n = col_sizes[j];
+    const double *x = vals + blk_off[b];
+    int32_t *re = rexp ? rexp + rfirst[i] : nullptr, *ce = cexp ? cexp + cfirst[j] : nullptr;
+    const bool shared = m <= kScaleRows && n <= kScaleRows;
+    if (shared) {
+      for (int r = lane; r < 2 * kScaleRows; r += 32) rmax[r] = 0;
+      __syncwarp();
+    }
+    const int64_t len = (int64_t)m * n;
+    for (int64_t e = lane; e < len; e += 32) {
+      const int f = digit_field(__ldg(x + e));
+      const int c = (int)(e / m), r = (int)(e - (int64_t)c * m);
+      if (shared) {
+        if (re) atomicMax(&rmax[r], f);
+        if (ce) atomicMax(&cmax[c], f);
+      } else {
+        if (re && re[r] < f) atomicMax(re + r, f);
+        if (ce && ce[c] < f) atomicMax(ce + c, f);
+      }
+    }
+    if (!shared) continue;
+    __syncwarp();
+    for (int r = lane; r < m; r += 32)  // a stale smaller value only costs an atomic
+      if (re && re[r] < rmax[r]) atomicMax(re + r, rmax[r]);
+    for (int c = lane; c < n; c += 32)
+      if (ce && ce[c] < cmax[c]) atomicMax(ce + c, cmax[c]);
+    __syncwarp();
+  }
+}
+
+cudaError_t launch_block_norms_scales(const int32_t *row_sizes, const int32_t *col_sizes,
+                                      const int32_t *blk_row, const int32_t *col_idx,
+                                      const int64_t *blk_off, const double *vals,
+                                      const int64_t *hdr, double *norms, float *normsf,
+                                      const int32_t *rfirst, const int32_t *cfirst, int32_t *rexp,
+                                      int32_t *cexp, int nsm, cudaStream_t stream) {
+  const int norm_blocks = nsm * 8, scale_blocks = (rexp || cexp) ? nsm * 4 : 0;
+  k_block_norms_scales<<<norm_blocks + scale_blocks, kScaleWarps * 32, 0, stream>>>(
+      row_sizes, col_sizes, blk_row, col_idx, blk_off, vals, hdr, norms, normsf, rfirst, cfirst,
+      rexp, cexp, norm_blocks);
   return cudaGetLastError();
 }
 
@@ -195,61 +290,10 @@ __device__ void row_bitmap(const DevMat &A, const DevMat &B, const DevMat &Cin, 
 }
 
 // ----------------------------------------------------------------------------
-// Count pass: one thread block per C block row (grid-stride).
+// Scan: one thread block. Exclusive sums over block rows, totals, capacity check,
+// C's header and the sentinel of the product ranges.
 // ----------------------------------------------------------------------------
-__global__ void __launch_bounds__(kSymThreads) k_symbolic_count(DevMat A, DevMat B, DevMat Cin,
-                                                                int use_cin, double eps,
-                                                                DevWs ws) {
-  extern __shared__ uint32_t smem_bits[];
-  const int nbc = B.nbc;
-  const bool whole = nbc <= kWindowCols;
-  for (int i = blockIdx.x; i < A.nbr; i += gridDim.x) {
-    int64_t cand = 0, kept = 0, flops = 0, colsum = 0, nblk = 0;
-    for (int w0 = 0; w0 < nbc; w0 += kWindowCols) {
-      const int wn = min(kWindowCols, nbc - w0);
-      const int nwords = (wn + 31) >> 5;
-      row_bitmap<true>(A, B, Cin, use_cin, eps, i, w0, wn, whole, smem_bits, nwords, cand, kept,
-                       flops);
-      for (int t = threadIdx.x; t < nwords; t += blockDim.x) {
-        uint32_t bits = smem_bits[t];
-        nblk += __popc(bits);
-        while (bits) {
-          const int b = __ffs(bits) - 1;
-          bits &= bits - 1;
-          colsum += B.col_sizes[w0 + 32 * t + b];
-        }
-      }
-      __syncthreads();
-    }
-    cand = block_sum(cand);
-    kept = block_sum(kept);
-    flops = block_sum(flops);
-    colsum = block_sum(colsum);
-    nblk = block_sum(nblk);
-    if (threadIdx.x == 0) {
-      ws.row_cblk[i] = (int32_t)nblk;
-      ws.row_prod[i] = kept;
-      ws.row_nnz[i] = (int64_t)A.row_sizes[i] * colsum;
-      ws.row_cand[i] = cand;
-      ws.row_flops[i] = flops;
-    }
-  }
-}
-
-cudaError_t launch_symbolic_count(DevMat A, DevMat B, DevMat Cin, int use_cin, double eps,
-                                  DevWs ws, int grid, cudaStream_t stream) {
-  const int nwords = (min(B.nbc, kWindowCols) + 31) / 32;
-  const size_t smem = (size_t)max(nwords, 1) * sizeof(uint32_t);
-  k_symbolic_count<<<grid, kSymThreads, smem, stream>>>(A, B, Cin, use_cin, eps, ws);
-  return cudaGetLastError();
-}
-
-// ----------------------------------------------------------------------------
-// Scan pass: one thread block of 1024 threads. Exclusive sums over block rows,
-// totals, capacity check, C's header and the sentinel of the product ranges.
-// ----------------------------------------------------------------------------
-__global__ void __launch_bounds__(1024) k_symbolic_scan(int32_t nbr, DevWs ws, DevOut C,
-                                                        DevStatus *st) {
+__device__ void symbolic_scan(int32_t nbr, const DevWs &ws, const DevOut &C, DevStatus *st) {
   // rows in tiles of blockDim.x, a row per thread (coalesced loads), the
   // running totals carried from tile to tile
   int64_t tb = 0, tp = 0, tn = 0, sc = 0, sf = 0;
@@ -299,6 +343,79 @@ __global__ void __launch_bounds__(1024) k_symbolic_scan(int32_t nbr, DevWs ws, D
   }
 }
 
+// ----------------------------------------------------------------------------
+// Count pass: one thread block per C block row (grid-stride).
+// ----------------------------------------------------------------------------
+__global__ void __launch_bounds__(kSymThreads) k_symbolic_count(DevMat A, DevMat B, DevMat Cin,
+                                                                int use_cin, double eps,
+                                                                DevWs ws, DevOut C, DevStatus *st,
+                                                                int32_t *ticket) {
+  extern __shared__ uint32_t smem_bits[];
+  const int nbc = B.nbc;
+  const bool whole = nbc <= kWindowCols;
+  for (int i = blockIdx.x; i < A.nbr; i += gridDim.x) {
+    int64_t cand = 0, kept = 0, flops = 0, colsum = 0, nblk = 0;
+    for (int w0 = 0; w0 < nbc; w0 += kWindowCols) {
+      const int wn = min(kWindowCols, nbc - w0);
+      const int nwords = (wn + 31) >> 5;
+      row_bitmap<true>(A, B, Cin, use_cin, eps, i, w0, wn, whole, smem_bits, nwords, cand, kept,
+                       flops);
+      for (int t = threadIdx.x; t < nwords; t += blockDim.x) {
+        uint32_t bits = smem_bits[t];
+        nblk += __popc(bits);
+        while (bits) {
+          const int b = __ffs(bits) - 1;
+          bits &= bits - 1;
+          colsum += B.col_sizes[w0 + 32 * t + b];
+        }
+      }
+      __syncthreads();
+    }
+    cand = block_sum(cand);
+    kept = block_sum(kept);
+    flops = block_sum(flops);
+    colsum = block_sum(colsum);
+    nblk = block_sum(nblk);
+    if (threadIdx.x == 0) {
+      ws.row_cblk[i] = (int32_t)nblk;
+      ws.row_prod[i] = kept;
+      ws.row_nnz[i] = (int64_t)A.row_sizes[i] * colsum;
+      ws.row_cand[i] = cand;
+      ws.row_flops[i] = flops;
+    }
+  }
+  if (ticket) {  // the last thread block to get here has every row's counts
+    __shared__ int last;
+    if (threadIdx.x == 0) {
+      __threadfence();
+      last = atomicAdd(ticket, 1) == (int)gridDim.x - 1;
+    }
+    __syncthreads();
+    if (!last) return;
+    __threadfence();
+    symbolic_scan(A.nbr, ws, C, st);
+    if (threadIdx.x == 0) *ticket = 0;
+  }
+}
+
+cudaError_t launch_symbolic_count(DevMat A, DevMat B, DevMat Cin, int use_cin, double eps,
+                                  DevWs ws, DevOut C, DevStatus *st, int32_t *ticket, int grid,
+                                  cudaStream_t stream) {
+  const int nwords = (min(B.nbc, kWindowCols) + 31) / 32;
+  const size_t smem = (size_t)max(nwords, 1) * sizeof(uint32_t);
+  if (ticket) grid = min(grid, max(A.nbr, 1));  // fewer to wait for
+  k_symbolic_count<<<grid, kSymThreads, smem, stream>>>(A, B, Cin, use_cin, eps, ws, C, st, ticket);
+  return cudaGetLastError();
+}
+
+// ----------------------------------------------------------------------------
+// Scan pass of its own: one thread block of 1024 threads.
+// ----------------------------------------------------------------------------
+__global__ void __launch_bounds__(1024) k_symbolic_scan(int32_t nbr, DevWs ws, DevOut C,
+                                                        DevStatus *st) {
+  symbolic_scan(nbr, ws, C, st);
+}
+
 cudaError_t launch_symbolic_scan(int32_t nbr, DevWs ws, DevOut C, DevStatus *st,
                                  cudaStream_t stream) {
   k_symbolic_scan<<<1, 1024, 0, stream>>>(nbr, ws, C, st);
@@ -339,7 +456,7 @@ __device__ __forceinline__ int bit_rank(const uint32_t *bitmap, const int32_t *w
 __global__ void __launch_bounds__(kSymThreads) k_symbolic_fill(DevMat A, DevMat B, DevMat Cin,
                                                                int use_cin, double eps, DevWs ws,
                                                                DevOut C, const DevStatus *st,
-                                                               int mask_words) {
+                                                               int mask_words, Digits dg) {
   if (st->overflow) return;
   extern __shared__ uint32_t smem_bits[];
   const int nbc = B.nbc;
@@ -553,14 +670,26 @@ __global__ void __launch_bounds__(kSymThreads) k_symbolic_fill(DevMat A, DevMat 
       slot_base += nw;
     }
   }
+
+  // the operands' digits, where the numeric phase takes them: bandwidth-bound
+  // work that fits between the latency-bound rows of other thread blocks
+  if (dg.a.units) {
+    __syncthreads();
+    int32_t *seg = reinterpret_cast<int32_t *>(smem_bits) + warp * kDigitMaxRows;
+    const bool same = A.vals == B.vals;
+    const int64_t w0 = (int64_t)blockIdx.x * nwarps + warp, nw = (int64_t)gridDim.x * nwarps;
+    digits_of(A, &dg.a, same ? &dg.b : nullptr, seg, w0, nw, lane);
+    if (!same) digits_of(B, nullptr, &dg.b, seg, w0, nw, lane);
+  }
 }
 
 cudaError_t launch_symbolic_fill(DevMat A, DevMat B, DevMat Cin, int use_cin, double eps,
                                  DevWs ws, DevOut C, const DevStatus *st, int nsm, int mask_words,
-                                 cudaStream_t stream) {
+                                 const Digits *digits, cudaStream_t stream) {
   const int nwords = (min(B.nbc, kWindowCols) + 31) / 32;
   const int mw = (mask_words > 0 && mask_words < kMaskWords) ? mask_words : kMaskWords;
-  const size_t smem = ((size_t)max(nwords, 1) * 2 + mw) * sizeof(uint32_t);
+  size_t smem = ((size_t)max(nwords, 1) * 2 + mw) * sizeof(uint32_t);
+  if (digits) smem = max(smem, sizeof(int32_t) * kDigitMaxRows * (kSymThreads / 32));
   // one wave of resident blocks (rows taken in a grid stride): more resident
   // blocks hide more of each row's load latency, a second wave only adds a tail
   int per_sm = 0;
@@ -568,7 +697,8 @@ cudaError_t launch_symbolic_fill(DevMat A, DevMat B, DevMat Cin, int use_cin, do
                                                                 kSymThreads, smem);
   if (e != cudaSuccess) return e;
   const int grid = nsm * (per_sm > 0 ? per_sm : 1);
-  k_symbolic_fill<<<grid, kSymThreads, smem, stream>>>(A, B, Cin, use_cin, eps, ws, C, st, mw);
+  k_symbolic_fill<<<grid, kSymThreads, smem, stream>>>(A, B, Cin, use_cin, eps, ws, C, st, mw,
+                                                       digits ? *digits : Digits{});
   return cudaGetLastError();
 }
 
