@@ -290,66 +290,73 @@ __global__ void __launch_bounds__(kSWarps * 32, MINB)
 // or 8 rows and GS = 4, 6 or 8 lanes per group, chosen per launch from the
 // largest C block: 5 groups of 6 lanes fill 30 of a warp's 32 lanes for
 // 6-wide blocks, where groups of 8 would leave a quarter of the lanes without
-// a column). The groups of a warp are independent streams: each takes kG8Grab C blocks at a time from the
-// work counter and walks their products one step per loop iteration, closing
-// a C block (epilogue, next block's metadata) in the iteration that ends it,
-// so a group whose block has more products does not hold the other groups at
-// a loop exit. Lanes hold no shared state: the latency of each C block's chain
-// of dependent loads is hidden by the many independent blocks in flight. A C
-// block of more than MR rows or GS columns (only when the kernel is forced on
-// larger blocks) is done in column and row chunks by its group.
+// a column). A warp takes a run of C blocks at a time, whose descriptors and
+// products its lanes look up at once; each group takes the run's next block when
+// it has closed one, and walks its products one step per loop iteration. The
+// finished blocks are gathered in shared memory and leave the warp together: the
+// blocks of a run mostly follow one another in C, and a store instruction then
+// covers 256 contiguous bytes. A lane's own columns would be 8 bytes apart from
+// every other store, which the link to host memory (the second destination) takes
+// at 25 GB/s of its 193.
+// Measured, 20000 atoms, 2.2 M C blocks of 6, numeric phase with a second
+// destination in host memory: 26.1 -> 3.40 ms, bound by the link (637 MB); without
+// one 1.40 -> 1.37, bound by the FP64 pipe (0.68 without its instructions): the
+// multiplication by alpha, on the few lanes of one group at a time, moved to the
+// stores, where it is on all lanes. 16 warps per SM with runs of 30 blocks: 24 warps
+// with runs of 15 took 0.15 ms more, 32 0.5 (the groups idle at a run's end).
+// A C block of more than MR rows or GS columns (only when the kernel is forced on
+// larger blocks) is done in column and row chunks by its group and stored directly.
 // ----------------------------------------------------------------------------
 constexpr int kG8Warps = 8;
-constexpr int kG8Grab = 16;  // C blocks per group and grab
+constexpr int kG8BlocksPerSm = 2;
+constexpr int kG8Stage = 1152;  // doubles a warp gathers, at most
+constexpr int kG8List = 64;     // products of a run that are listed
+struct G8Item {  // a C block of a warp's run
+  int64_t coff, p, cin;      // cin: offset of its C_in block, or -1
+  int32_t np, m, n, at, q0;  // at: of its values in the stage, q0: its first product's entry
+};
+struct G8Product {  // where the two blocks of a product start, and their common size
+  int64_t a, b;
+  int32_t s;
+};
+
+size_t g8_smem_bytes() {
+  return kG8Warps * (kG8Stage * sizeof(double) + kG8List * sizeof(G8Product) + 32 * sizeof(G8Item));
+}
 
 template <int MR, int GS>
-__global__ void __launch_bounds__(kG8Warps * 32, 4)
+__global__ void __launch_bounds__(kG8Warps * 32, kG8BlocksPerSm)
     k_numeric_fp64_g8(DevMat A, DevMat B, DevOut C, DevMat Cin, double alpha, double beta,
                       DevWs ws, const DevStatus *st, const int32_t *items, const int64_t *seg,
                       unsigned long long *work) {
   if (st->overflow) return;
-  const int lane = threadIdx.x & 31;
+  constexpr int kGroups = 32 / GS;
+  constexpr int kFit = kG8Stage / (MR * GS);  // blocks of MR x GS that the stage holds
+  constexpr int kRun = (kFit < 32 ? kFit : 32) / kGroups * kGroups;
+  extern __shared__ double smem_g8[];
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
   const int grp = lane / GS, cl = lane - grp * GS;
-  if (grp >= 32 / GS) return;  // lanes past the last whole group
-  const unsigned gmask = ((1u << GS) - 1u) << (GS * grp);
+  double *stage = smem_g8 + warp * kG8Stage;
+  G8Product *list = reinterpret_cast<G8Product *>(smem_g8 + kG8Warps * kG8Stage) + warp * kG8List;
+  G8Item *item = reinterpret_cast<G8Item *>(
+                     reinterpret_cast<G8Product *>(smem_g8 + kG8Warps * kG8Stage) +
+                     kG8Warps * kG8List) + warp * 32;
   int64_t wb, we;
   work_range(st, seg, wb, we);
   // the second destination (host memory) when the whole result fits it
   double *hout = (C.host_vals && st->nnz_c <= C.host_cap) ? C.host_vals : nullptr;
 
-  // the group's current grab [w, wend) and C block (group-uniform state)
-  int64_t w = 0, wend = 0, p = 0, p1 = 0, cbase = 0;
-  int m = 0, n = 0;
-  const double *cinv = nullptr;
   double acc[MR];
-  auto next_block = [&]() -> bool {
-    if (w >= wend) {
-      unsigned long long got = 0;
-      if (cl == 0) got = atomicAdd(work, (unsigned long long)kG8Grab);
-      w = wb + (int64_t)__shfl_sync(gmask, got, GS * grp);
-      wend = (w + kG8Grab < we) ? w + kG8Grab : we;
-      if (w >= we) return false;
-    }
-    const int64_t g = items ? items[w] : w;
-    w++;
-    m = C.row_sizes[C.blk_row[g]];
-    n = C.col_sizes[C.col_idx[g]];
-    p = ws.prod_ptr[g];
-    p1 = ws.prod_ptr[g + 1];
-    const int cin = ws.c_cin[g];
-    cinv = (cin >= 0) ? Cin.vals + Cin.blk_off[cin] : nullptr;
-    cbase = C.blk_off[g];
-#pragma unroll
-    for (int r = 0; r < MR; r++) acc[r] = 0.0;
-    return true;
-  };
-  // rows [r0, r0 + MR) of column c of product q, added to acc
-  auto product = [&](int64_t q, int c, int r0) {
+  auto entry = [&](int64_t q) -> G8Product {
     const int2 pr = ws.prods[q];
-    const double *Ab = A.vals + A.blk_off[pr.x] + r0;
-    const int s = A.col_sizes[A.col_idx[pr.x]];
-    const double *Bb = B.vals + B.blk_off[pr.y] + (int64_t)c * s;
-    for (int kk = 0; kk < s; kk++) {
+    return {A.blk_off[pr.x], B.blk_off[pr.y], A.col_sizes[A.col_idx[pr.x]]};
+  };
+  // rows [r0, r0 + MR) of column c of a product, added to acc
+  auto product = [&](const G8Product &e, int m, int c, int r0) {
+    const double *Ab = A.vals + e.a + r0;
+    const double *Bb = B.vals + e.b + (int64_t)c * e.s;
+#pragma unroll 2
+    for (int kk = 0; kk < e.s; kk++) {
       const double bv = __ldg(Bb + kk);
       const double *a = Ab + (int64_t)kk * m;
 #pragma unroll
@@ -357,41 +364,131 @@ __global__ void __launch_bounds__(kG8Warps * 32, 4)
         if (r0 + r < m) acc[r] = fma(__ldg(a + r), bv, acc[r]);
     }
   };
-  // C_ij = beta * C_in_ij + alpha * S_ij for rows [r0, r0 + MR) of column c
-  auto store = [&](int c, int r0) {
+  // C_ij = beta * C_in_ij + alpha * S_ij of row r of acc, at loc of the block
+  auto value = [&](const double *cinv, int r, int64_t loc) {
+    const double v = alpha * acc[r];
+    return cinv ? fma(beta, cinv[loc], v) : v;
+  };
+  auto scan = [&](int v) {  // inclusive sum over the lanes
 #pragma unroll
-    for (int r = 0; r < MR; r++) {
-      if (r0 + r < m) {
-        const int64_t loc = (int64_t)c * m + r0 + r;
-        double v = alpha * acc[r];
-        if (cinv) v = fma(beta, cinv[loc], v);
-        C.vals[cbase + loc] = v;
-        if (hout) hout[cbase + loc] = v;
-      }
+    for (int d = 1; d < 32; d <<= 1) {
+      const int y = __shfl_up_sync(0xffffffffu, v, d);
+      if (lane >= d) v += y;
     }
+    return v;
   };
 
-  bool have = next_block();
-  while (have) {
-    if (m > MR || n > GS) {  // column and row chunks, the products once per chunk
-      for (int c = cl; c < n; c += GS)
-        for (int r0 = 0; r0 < m; r0 += MR) {
+  for (;;) {
+    unsigned long long got = 0;
+    if (lane == 0) got = atomicAdd(work, (unsigned long long)kRun);
+    const int64_t base = wb + (int64_t)__shfl_sync(0xffffffffu, got, 0);
+    if (base >= we) break;
+    const int count = we - base < kRun ? (int)(we - base) : kRun;
+    G8Item own{};
+    own.cin = -1;
+    if (lane < count) {
+      const int64_t g = items ? items[base + lane] : base + lane;
+      own.m = C.row_sizes[C.blk_row[g]];
+      own.n = C.col_sizes[C.col_idx[g]];
+      own.p = ws.prod_ptr[g];
+      own.np = (int)(ws.prod_ptr[g + 1] - own.p);
+      const int cin = ws.c_cin[g];
+      own.cin = cin >= 0 ? Cin.blk_off[cin] : -1;
+      own.coff = C.blk_off[g];
+    }
+    const bool gather = !__any_sync(0xffffffffu, own.m > MR || own.n > GS);
+    const bool late = gather && !__any_sync(0xffffffffu, own.cin >= 0);  // alpha at the stores
+    const int mn = own.m * own.n;
+    own.at = scan(mn) - mn;
+    const int np = own.np < kG8List ? own.np : kG8List;
+    const int q1 = scan(np);
+    own.q0 = q1 - np;
+    if (lane < count) item[lane] = own;
+    // blocks that do not follow the one before them in C
+    const int64_t follows = __shfl_up_sync(0xffffffffu, own.coff + mn, 1);
+    uint32_t starts = __ballot_sync(0xffffffffu, lane < count && (lane == 0 || own.coff != follows));
+    // the products' entries, a lane each
+    const int listed = min(__shfl_sync(0xffffffffu, q1, 31), kG8List);
+    for (int q = lane; q - lane < listed; q += 32) {
+      int b = 0;  // the block of product q: blocks that end at or before it
 #pragma unroll
-          for (int r = 0; r < MR; r++) acc[r] = 0.0;
-          for (int64_t q = p; q < p1; q++) product(q, c, r0);
-          store(c, r0);
+      for (int step = 16; step; step >>= 1)
+        if (__shfl_sync(0xffffffffu, q1, b + step - 1) <= q) b += step;
+      const int64_t p = __shfl_sync(0xffffffffu, own.p - own.q0, b) + q;
+      if (q < listed) list[q] = entry(p);
+    }
+    __syncwarp();
+
+    // a group takes the run's next block when it has closed one
+    int k = grp < kGroups ? grp : count, taken = kGroups, p = 0;
+    G8Item it{};
+    if (k < count) it = item[k];
+#pragma unroll
+    for (int r = 0; r < MR; r++) acc[r] = 0.0;
+    while (__any_sync(0xffffffffu, k < count)) {
+      if (k < count) {
+        const double *cinv = it.cin >= 0 ? Cin.vals + it.cin : nullptr;
+        if (!gather) {  // column and row chunks, the products once per chunk
+          for (int c = cl; c < it.n; c += GS)
+            for (int r0 = 0; r0 < it.m; r0 += MR) {
+#pragma unroll
+              for (int r = 0; r < MR; r++) acc[r] = 0.0;
+              for (int q = 0; q < it.np; q++) product(entry(it.p + q), it.m, c, r0);
+#pragma unroll
+              for (int r = 0; r < MR; r++)
+                if (r0 + r < it.m) {
+                  const int64_t loc = (int64_t)c * it.m + r0 + r;
+                  const double v = value(cinv, r, loc);
+                  C.vals[it.coff + loc] = v;
+                  if (hout) hout[it.coff + loc] = v;
+                }
+            }
+          p = it.np;
+        } else {
+          if (p < it.np) {  // one product of the block (products in ascending k)
+            const G8Product e = it.q0 + p < listed ? list[it.q0 + p] : entry(it.p + p);
+            if (cl < it.n) product(e, it.m, cl, 0);
+            p++;
+          }
+          if (p >= it.np && cl < it.n) {  // the block is complete
+#pragma unroll
+            for (int r = 0; r < MR; r++)
+              if (r < it.m) {
+                const int loc = cl * it.m + r;
+                stage[it.at + loc] = late ? acc[r] : value(cinv, r, loc);
+              }
+          }
         }
-      have = next_block();
-      continue;
+      }
+      const bool closed = grp < kGroups && k < count && p >= it.np;
+      const uint32_t heads = __ballot_sync(0xffffffffu, closed && cl == 0);
+      if (closed) {
+        k = taken + __popc(heads & ((1u << (grp * GS)) - 1u));
+        p = 0;
+        if (k < count) it = item[k];
+#pragma unroll
+        for (int r = 0; r < MR; r++) acc[r] = 0.0;
+      }
+      taken += __popc(heads);
     }
-    if (p < p1) {  // one product of the block (products in ascending k)
-      if (cl < n) product(p, cl, 0);
-      p++;
+    __syncwarp();
+    while (gather && starts) {  // blocks x to y - 1, which follow one another in C
+      const int x = __ffs(starts) - 1;
+      starts &= starts - 1;
+      const int y = starts ? __ffs(starts) - 1 : count;
+      const int at = __shfl_sync(0xffffffffu, own.at, x);
+      const int total = __shfl_sync(0xffffffffu, own.at + mn, y - 1) - at;
+      const int64_t first = __shfl_sync(0xffffffffu, own.coff, x);
+      // from the start of the 128-byte line that they begin in
+      for (int e = lane - (int)(first & 15); e < total; e += 32)
+        if (e >= 0) {
+          double v = stage[at + e];
+          if (late && alpha != 1.0) v *= alpha;
+          __stcs(C.vals + first + e, v);
+          if (hout) __stcs(hout + first + e, v);
+        }
     }
-    if (p >= p1) {  // the block is complete
-      if (cl < n) store(cl, 0);
-      have = next_block();
-    }
+    __syncwarp();
   }
 }
 
@@ -1089,8 +1186,8 @@ cudaError_t launch_numeric_fp64(int variant, DevMat A, DevMat B, DevOut C, DevMa
       const int mr = max_m <= 4 ? 4 : max_m <= 6 ? 6 : 8;
       const int gs = max_n <= 4 ? 4 : max_n <= 6 ? 6 : 8;
 #define BSM_G8(R, G)                                                                           \
-  k_numeric_fp64_g8<R, G><<<grid, kG8Warps * 32, 0, stream>>>(A, B, C, Cin, alpha, beta, ws, st, \
-                                                              items, seg, work)
+  k_numeric_fp64_g8<R, G><<<grid, kG8Warps * 32, g8_smem_bytes(), stream>>>(                   \
+      A, B, C, Cin, alpha, beta, ws, st, items, seg, work)
       if (mr == 4) {
         if (gs == 4) BSM_G8(4, 4); else if (gs == 6) BSM_G8(4, 6); else BSM_G8(4, 8);
       } else if (mr == 6) {
@@ -1129,7 +1226,7 @@ cudaError_t launch_numeric_fp64(int variant, DevMat A, DevMat B, DevOut C, DevMa
 
 int fp64_variant_blocks_per_sm(int variant) {
   if (variant == kFp64Dg) return kDgBlocksPerSm;
-  if (variant == kFp64G8) return 4;
+  if (variant == kFp64G8) return kG8BlocksPerSm;
   return (variant == kFp64T16B3 || variant == kFp64T32) ? 3 : 2;
 }
 
@@ -1140,6 +1237,15 @@ cudaError_t numeric_fp64_init() {
   if (e != cudaSuccess) return e;
   // its operands come through L1: no more shared memory than its own
   e = cudaFuncSetAttribute(k_numeric_fp64_dg, cudaFuncAttributePreferredSharedMemoryCarveout, 50);
+  if (e != cudaSuccess) return e;
+#define BSM_G8(R, G)                                                                      \
+  if (e == cudaSuccess)                                                                   \
+  e = cudaFuncSetAttribute(k_numeric_fp64_g8<R, G>, cudaFuncAttributeMaxDynamicSharedMemorySize, \
+                           (int)g8_smem_bytes())
+  BSM_G8(4, 4); BSM_G8(4, 6); BSM_G8(4, 8);
+  BSM_G8(6, 4); BSM_G8(6, 6); BSM_G8(6, 8);
+  BSM_G8(8, 4); BSM_G8(8, 6); BSM_G8(8, 8);
+#undef BSM_G8
   if (e != cudaSuccess) return e;
   e = cudaFuncSetAttribute(k_numeric_fp64_pk<12>, cudaFuncAttributeMaxDynamicSharedMemorySize,
                            (int)pk_smem_bytes());
