@@ -142,10 +142,6 @@ cudaError_t launch_block_norms_scales(const int32_t *row_sizes, const int32_t *c
                                       const int64_t *hdr, double *norms, float *normsf,
                                       const int32_t *rfirst, const int32_t *cfirst, int32_t *rexp,
                                       int32_t *cexp, int nsm, cudaStream_t stream);
-cudaError_t launch_block_norms(const int32_t *row_sizes, const int32_t *col_sizes,
-                               const int32_t *blk_row, const int32_t *col_idx,
-                               const int64_t *blk_off, const double *vals, const int64_t *hdr,
-                               double *norms, float *normsf, int grid, cudaStream_t stream);
 
 // ticket: null, or a device counter that is zero (and is left zero): the last
 // thread block then also does the scan (nbr <= kFusedScanRows: one launch less,

@@ -286,13 +286,14 @@ extern "C" int bsm_multiply_noalloc(double alpha, const bsm_dev_csr *A, const bs
   out.cap_blk = cap_blk;
   out.cap_nnz = C->cap_nnz;
 
-  if ((e = launch_block_norms(A->row_sizes, A->col_sizes, brow_a, A->col_idx, A->blk_off,
-                              A->values, hdr_a, norms_a, normsf_a, nsm * 8, s)) != cudaSuccess)
+  if ((e = launch_block_norms_scales(A->row_sizes, A->col_sizes, brow_a, A->col_idx, A->blk_off,
+                                     A->values, hdr_a, norms_a, normsf_a, nullptr, nullptr, nullptr,
+                                     nullptr, nsm, s)) != cudaSuccess)
     return noalloc_cuda_fail(e);
-  if (!same && (e = launch_block_norms(B->row_sizes, B->col_sizes, brow_b, B->col_idx,
-                                       B->blk_off, B->values, hdr_b, norms_b, normsf_b, nsm * 8,
-                                       s)) !=
-                   cudaSuccess)
+  if (!same &&
+      (e = launch_block_norms_scales(B->row_sizes, B->col_sizes, brow_b, B->col_idx, B->blk_off,
+                                     B->values, hdr_b, norms_b, normsf_b, nullptr, nullptr, nullptr,
+                                     nullptr, nsm, s)) != cudaSuccess)
     return noalloc_cuda_fail(e);
   if ((e = launch_symbolic_count(dA, dB, none, 0, eps, ws, out, st, nullptr, nsm * 6, s)) != cudaSuccess)
     return noalloc_cuda_fail(e);

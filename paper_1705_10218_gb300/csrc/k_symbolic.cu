@@ -12,6 +12,8 @@
 //          value offset, and the kept products written grouped by C block in
 //          ascending k (a per-row counting sort), so that the numeric phase
 //          accumulates each C block in one place, without atomics.
+#include <type_traits>
+
 #include "bsm_internal.h"
 #include "digits.cuh"
 
@@ -69,53 +71,102 @@ __device__ __forceinline__ int lower_bound_i32(const int32_t *a, int lo, int hi,
 }
 
 // ----------------------------------------------------------------------------
-// Block norms: canonical Frobenius norm, column-major, no fused multiply-add.
-// One thread per block, grid-stride; the block count is read on the device so
-// a matrix produced by an earlier multiply needs no host round trip.
+// Block norms: canonical Frobenius norm, column-major, no fused multiply-add; the
+// block count is read on the device so that a matrix produced by an earlier multiply
+// needs no host round trip. And the scales of the digit representation in the same
+// launch (rexp, cexp: where they are wanted): the first thread blocks take the norms, the others the scales, a warp per block: each
+// lane's elements go to their row's and column's maximum in shared memory, and a
+// maximum that the array does not hold yet there.
+//
+// A norm's additions have a fixed order, so a block's chain of them is one lane's. The
+// FP64 pipe takes a warp's instruction in 64 clocks of a quarter SM, whatever its
+// active lanes: many blocks are a lane each (its loads eight ahead). Where that would
+// leave quarters idle, LANES lanes share a block: each loads and squares every
+// LANES-th value, and all follow the additions, so that the chain is an addition per
+// value instead of an addition and a multiplication, with loads of whole sectors; and
+// consecutive warps' blocks go to different SMs. 2795 + 2487 blocks of up to 33 x 33:
+// 140 + 138 -> 74 + 74 us, of which 17 + 17 are the scales.
 // ----------------------------------------------------------------------------
-__global__ void k_block_norms(const int32_t *__restrict__ row_sizes,
-                              const int32_t *__restrict__ col_sizes,
-                              const int32_t *__restrict__ blk_row,
-                              const int32_t *__restrict__ col_idx,
-                              const int64_t *__restrict__ blk_off,
-                              const double *__restrict__ vals, const int64_t *__restrict__ hdr,
-                              double *__restrict__ norms, float *__restrict__ normsf) {
-  const int64_t nblk = hdr[0];
-  for (int64_t b = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; b < nblk;
-       b += (int64_t)gridDim.x * blockDim.x) {
-    const int64_t n = (int64_t)row_sizes[blk_row[b]] * col_sizes[col_idx[b]];
-    const double *x = vals + blk_off[b];
-    double s = 0.0;
-    for (int64_t e = 0; e < n; e++) {
-      const double v = __ldg(x + e);
-      s = __dadd_rn(s, __dmul_rn(v, v));
+constexpr int kScaleWarps = 8;
+constexpr int kNormAhead = 8;   // loads of a lane in flight
+constexpr int kNormBlocksPerSm = 8;
+constexpr int kScaleRows = 64;  // rows and columns kept in shared memory
+
+
+// The sum of squares of the n values at x, in order; LANES lanes of a warp have the
+// same x and n, sub is the lane's number among them. All lanes of the warp take part.
+template <int LANES>
+__device__ __forceinline__ double sum_of_squares(const double *__restrict__ x, int64_t n, int sub) {
+  double s = 0.0;
+  if (LANES == 1) {
+    double v[kNormAhead];
+    int64_t e = 0;
+    for (; e + kNormAhead <= n; e += kNormAhead) {
+#pragma unroll
+      for (int u = 0; u < kNormAhead; u++) v[u] = __ldg(x + e + u);
+#pragma unroll
+      for (int u = 0; u < kNormAhead; u++) s = __dadd_rn(s, __dmul_rn(v[u], v[u]));
     }
+    for (; e < n; e++) {
+      const double y = __ldg(x + e);
+      s = __dadd_rn(s, __dmul_rn(y, y));
+    }
+    return s;
+  }
+  constexpr int kAhead = kNormAhead / 2, kStep = LANES * kAhead;
+  double v[kAhead];
+  auto load = [&](int64_t e) {
+#pragma unroll
+    for (int u = 0; u < kAhead; u++)
+      v[u] = e + u * LANES + sub < n ? __ldg(x + e + u * LANES + sub) : 0.0;
+  };
+  load(0);
+  int64_t most = n;
+  for (int d = LANES; d < 32; d <<= 1)
+    most = max(most, __shfl_xor_sync(0xffffffffu, most, d));
+  for (int64_t e = 0; e < most; e += kStep) {
+    double q[kAhead];
+#pragma unroll
+    for (int u = 0; u < kAhead; u++) q[u] = __dmul_rn(v[u], v[u]);
+    load(e + kStep);
+#pragma unroll
+    for (int u = 0; u < kAhead; u++)
+#pragma unroll
+      for (int l = 0; l < LANES; l++) {
+        const double y = __shfl_sync(0xffffffffu, q[u], l, LANES);
+        if (e + u * LANES + l < n) s = __dadd_rn(s, y);
+      }
+  }
+  return s;
+}
+
+template <int LANES>
+__device__ __forceinline__ void block_norms(const int32_t *__restrict__ row_sizes,
+                                            const int32_t *__restrict__ col_sizes,
+                                            const int32_t *__restrict__ blk_row,
+                                            const int32_t *__restrict__ col_idx,
+                                            const int64_t *__restrict__ blk_off,
+                                            const double *__restrict__ vals, int64_t nblk,
+                                            double *__restrict__ norms, float *__restrict__ normsf,
+                                            int norm_blocks, int nsm) {
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+  constexpr int kPerWarp = 32 / LANES;
+  // the thread blocks of an SM start with warps of different quarters of it
+  const int turn = (warp + blockIdx.x / nsm) % kScaleWarps;
+  for (int64_t w = (int64_t)turn * norm_blocks + blockIdx.x; w * kPerWarp < nblk;
+       w += (int64_t)norm_blocks * kScaleWarps) {
+    const int64_t b = w * kPerWarp + lane / LANES;
+    const bool in = b < nblk;
+    const int64_t n = in ? (int64_t)row_sizes[blk_row[b]] * col_sizes[col_idx[b]] : 0;
+    const double s = sum_of_squares<LANES>(vals + (in ? blk_off[b] : 0), n, lane % LANES);
+    if (!in || lane % LANES) continue;
     const double nrm = __dsqrt_rn(s);
     norms[b] = nrm;
     normsf[b] = (nrm >= 0x1p-60 && nrm <= 0x1p60) ? __double2float_rn(nrm) : NAN;
   }
 }
 
-cudaError_t launch_block_norms(const int32_t *row_sizes, const int32_t *col_sizes,
-                               const int32_t *blk_row, const int32_t *col_idx,
-                               const int64_t *blk_off, const double *vals, const int64_t *hdr,
-                               double *norms, float *normsf, int grid, cudaStream_t stream) {
-  k_block_norms<<<grid, 256, 0, stream>>>(row_sizes, col_sizes, blk_row, col_idx, blk_off, vals,
-                                          hdr, norms, normsf);
-  return cudaGetLastError();
-}
-
-// ----------------------------------------------------------------------------
-// The norms, and the scales of the digit representation in the same launch: the
-// first thread blocks take the norms, a thread per block as above, eight loads
-// ahead of the additions; the others the scales, a warp per block: each lane's
-// elements go to their row's and column's maximum in shared memory, and a maximum
-// that the array does not hold yet there.
-// ----------------------------------------------------------------------------
-constexpr int kScaleWarps = 8;
-constexpr int kScaleRows = 64;  // rows and columns kept in shared memory
-
-__global__ void __launch_bounds__(kScaleWarps * 32)
+__global__ void __launch_bounds__(kScaleWarps * 32, 5)
     k_block_norms_scales(const int32_t *__restrict__ row_sizes,
                          const int32_t *__restrict__ col_sizes,
                          const int32_t *__restrict__ blk_row, const int32_t *__restrict__ col_idx,
@@ -126,27 +177,18 @@ __global__ void __launch_bounds__(kScaleWarps * 32)
                          int norm_blocks) {
   const int64_t nblk = hdr[0];
   if ((int)blockIdx.x < norm_blocks) {
-    for (int64_t b = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; b < nblk;
-         b += (int64_t)norm_blocks * blockDim.x) {
-      const int64_t n = (int64_t)row_sizes[blk_row[b]] * col_sizes[col_idx[b]];
-      const double *x = vals + blk_off[b];
-      double s = 0.0;
-      int64_t e = 0;
-      for (; e + 8 <= n; e += 8) {
-        double v[8];
-#pragma unroll
-        for (int u = 0; u < 8; u++) v[u] = __ldg(x + e + u);
-#pragma unroll
-        for (int u = 0; u < 8; u++) s = __dadd_rn(s, __dmul_rn(v[u], v[u]));
-      }
-      for (; e < n; e++) {
-        const double v = __ldg(x + e);
-        s = __dadd_rn(s, __dmul_rn(v, v));
-      }
-      const double nrm = __dsqrt_rn(s);
-      norms[b] = nrm;
-      normsf[b] = (nrm >= 0x1p-60 && nrm <= 0x1p60) ? __double2float_rn(nrm) : NAN;
-    }
+    auto norms_by = [&](auto lanes) {
+      block_norms<decltype(lanes)::value>(row_sizes, col_sizes, blk_row, col_idx, blk_off, vals,
+                                          nblk, norms, normsf, norm_blocks, norm_blocks / kNormBlocksPerSm);
+    };
+    // the most lanes that need no more warps than there are quarters of SMs
+    const int64_t quarters = norm_blocks / kNormBlocksPerSm * 4;
+    if (nblk <= 2 * quarters)
+      norms_by(std::integral_constant<int, 16>{});
+    else if (nblk <= 8 * quarters)
+      norms_by(std::integral_constant<int, 4>{});
+    else
+      norms_by(std::integral_constant<int, 1>{});
     return;
   }
   __shared__ int32_t smax[kScaleWarps][2 * kScaleRows];
@@ -164,10 +206,17 @@ __global__ void __launch_bounds__(kScaleWarps * 32)
       for (int r = lane; r < 2 * kScaleRows; r += 32) rmax[r] = 0;
       __syncwarp();
     }
+    // element e: column c, row r; 32 elements on, four loads ahead
     const int64_t len = (int64_t)m * n;
+    const int dc = 32 / m, dr = 32 - dc * m;
+    int c = lane / m, r = lane - c * m;
+    double v[4];
+#pragma unroll
+    for (int u = 0; u < 4; u++) v[u] = lane + 32 * u < len ? __ldg(x + lane + 32 * u) : 0.0;
     for (int64_t e = lane; e < len; e += 32) {
-      const int f = digit_field(__ldg(x + e));
-      const int c = (int)(e / m), r = (int)(e - (int64_t)c * m);
+      const int f = digit_field(v[0]);
+      v[0] = v[1], v[1] = v[2], v[2] = v[3];
+      v[3] = e + 128 < len ? __ldg(x + e + 128) : 0.0;
       if (shared) {
         if (re) atomicMax(&rmax[r], f);
         if (ce) atomicMax(&cmax[c], f);
@@ -175,6 +224,8 @@ __global__ void __launch_bounds__(kScaleWarps * 32)
         if (re && re[r] < f) atomicMax(re + r, f);
         if (ce && ce[c] < f) atomicMax(ce + c, f);
       }
+      r += dr, c += dc;
+      if (r >= m) r -= m, c++;
     }
     if (!shared) continue;
     __syncwarp();
@@ -192,7 +243,7 @@ cudaError_t launch_block_norms_scales(const int32_t *row_sizes, const int32_t *c
                                       const int64_t *hdr, double *norms, float *normsf,
                                       const int32_t *rfirst, const int32_t *cfirst, int32_t *rexp,
                                       int32_t *cexp, int nsm, cudaStream_t stream) {
-  const int norm_blocks = nsm * 8, scale_blocks = (rexp || cexp) ? nsm * 4 : 0;
+  const int norm_blocks = nsm * kNormBlocksPerSm, scale_blocks = (rexp || cexp) ? nsm * 4 : 0;
   k_block_norms_scales<<<norm_blocks + scale_blocks, kScaleWarps * 32, 0, stream>>>(
       row_sizes, col_sizes, blk_row, col_idx, blk_off, vals, hdr, norms, normsf, rfirst, cfirst,
       rexp, cexp, norm_blocks);

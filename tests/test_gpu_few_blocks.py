@@ -1,0 +1,52 @@
+"""Matrices of few large and of many small blocks: norms by several lanes a block, C
+blocks in parts, sums over short runs of blocks."""
+import numpy as np
+import pytest
+
+import synth
+from synth import BlockMatrix
+from tests import helpers as H
+
+pytestmark = pytest.mark.gpu
+
+
+# number of blocks: 16 lanes a block, 4, one, more than one pass
+@pytest.mark.parametrize("nblk,top", [(1, 40), (37, 70), (1300, 33), (4800, 20), (9800, 9), (90000, 4)])
+def test_norms_are_the_canonical_ones(gpu_ctx, oracle_mod, nblk, top):
+    """Every block has to pass a filter at its own canonical norm and none at the
+    next larger number: the norms of the blocks sorted, the filter at some of
+    them keeps exactly the blocks from there on."""
+    rng = np.random.default_rng(nblk)
+    n = max(1, int(np.sqrt(nblk)) + 1)
+    rs, cs = rng.integers(1, top + 1, n), rng.integers(1, top + 1, n)
+    rs[0] = cs[0] = top
+    at = np.sort(np.concatenate([[0], 1 + rng.permutation(n * n - 1)[:nblk - 1]]))
+    r, c = np.divmod(at, n)
+    num = int((rs[r].astype(np.int64) * cs[c]).sum())
+    M = BlockMatrix(rs.astype(np.int32), cs.astype(np.int32), r.astype(np.int32), c.astype(np.int32),
+                    rng.standard_normal(num))
+    norms = oracle_mod.norms(M)
+    for eps in [np.sort(norms)[int(q * (nblk - 1))] for q in (0.0, 0.3, 0.7, 1.0)]:
+        for e in (eps, np.nextafter(eps, np.inf)):
+            D = gpu_ctx.from_blocks(M)
+            D.filter(float(e))
+            kr, kc = D.pattern()
+            keep = ~(norms < e)
+            assert np.array_equal(kr, M.blk_row[keep]) and np.array_equal(kc, M.blk_col[keep])
+            D.destroy()
+
+
+# one block; fewer than the warps of the launch; more than one block a warp and step
+@pytest.mark.parametrize("n,top,density", [(1, 33, 1.0), (40, 33, 0.5), (170, 4, 0.9)])
+def test_sum_of_matrices(gpu_ctx, n, top, density):
+    rng = np.random.default_rng(n)
+    rs, cs = rng.integers(1, top + 1, n), rng.integers(1, top + 1, n)
+    A = synth.random_blocks(rng, rs, cs, density, kind="int", shuffle=True)
+    B = synth.random_blocks(rng, rs, cs, density, kind="int", shuffle=True)
+    dA, dB = gpu_ctx.from_blocks(A), gpu_ctx.from_blocks(B)
+    gpu_ctx.add(-3.0, dA, 2.0, dB)
+    r, c = dB.pattern()
+    got = H.to_dense(BlockMatrix(A.row_sizes, A.col_sizes, r, c, dB.values()))
+    assert np.array_equal(got, 2.0 * H.to_dense(B) - 3.0 * H.to_dense(A))
+    for M in (dA, dB):
+        M.destroy()
