@@ -922,14 +922,14 @@ static int launch_numeric(Launch &L, int variant, const int32_t *items, const in
     CK(launch_numeric_fp64(variant, L.dA, L.dB, L.out, L.dC, L.alpha, L.beta, L.ws,
                            ctx->d_status, items, seg,
                            ctx->nsm * fp64_variant_blocks_per_sm(variant), ctx->d_work, max_m,
-                           max_n, &dg, L.s));
+                           max_n, variant == kFp64Dg ? &dg : nullptr, L.s));
     if (variant == kFp64Dg) {  // the C blocks it left to the packed kernel, if any
       ctx->launches++;
       CK(cudaMemsetAsync(ctx->d_work, 0, sizeof(unsigned long long), L.s));
       CK(launch_numeric_fp64(kFp64Pk12, L.dA, L.dB, L.out, L.dC, L.alpha, L.beta, L.ws,
                              ctx->d_status, dg.list, dg.range,
                              ctx->nsm * fp64_variant_blocks_per_sm(kFp64Pk12), ctx->d_work, max_m,
-                             max_n, nullptr, L.s));
+                             max_n, &dg, L.s));
     }
   }
   ctx->launches++;

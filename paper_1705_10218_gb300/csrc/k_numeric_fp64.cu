@@ -560,6 +560,7 @@ __device__ __forceinline__ void pk_wait() {
 
 // C blocks a warp takes from the work counter at a time.
 constexpr int kPkGrab = 1;
+constexpr int kPkUnits = 16;  // units of work per warp up to which C blocks are split
 
 // `steps` steps of one chunk for a tile of NT slots per lane: slot t adds
 // sA[ia_t + u * G * tm] * sB[ib_t + u * G] at step u. NT is a compile-time
@@ -588,7 +589,7 @@ __device__ __forceinline__ void pk_steps(const double *__restrict__ sA,
 template <int SLOTS>
 __device__ __forceinline__ void pk_block(const DevMat &A, const DevMat &B, const DevOut &C,
                                          const DevMat &Cin, double alpha, double beta,
-                                         const DevWs &ws, int64_t gblk, double *wbuf,
+                                         const DevWs &ws, int64_t gblk, int part, int parts, double *wbuf,
                                          double *hout, int lane) {
   constexpr int kStage = kPkStage;
   const PkShapes &shapes = (SLOTS == 12) ? c_pk_shapes12 : c_pk_shapes16;
@@ -600,8 +601,10 @@ __device__ __forceinline__ void pk_block(const DevMat &A, const DevMat &B, const
   double *out = C.vals + C.blk_off[gblk];
   double *hblk = hout ? hout + C.blk_off[gblk] : nullptr;
 
+  int at = 0;  // the tile's number
   for (int r0 = 0; r0 < m; r0 += kPkTile) {
     for (int c0 = 0; c0 < n; c0 += kPkTile) {
+      if (parts > 1 && at++ % parts != part) continue;
       const int tm = min(kPkTile, m - r0), tn = min(kPkTile, n - c0);
       const int te = tm * tn;
       int nT = shapes.nt[te], G = shapes.g[te];
@@ -789,12 +792,16 @@ break;
 }
 
 // work: a counter that is zero when the launch starts; warps take the next
-// kPkGrab C blocks of the work range from it until the range is exhausted.
+// kPkGrab C blocks of the work range from it until the range is exhausted. With
+// ntiles > 0 (the tiles that a C block has at most), a few C blocks are split into
+// parts, every parts-th of a block's tiles each: those that another kernel leaves are
+// few, and a large one that is a warp's alone takes as long as a whole multiply (2% of
+// 8695 blocks of up to 33 x 33: 449 -> 115 us).
 template <int SLOTS>
 __global__ void __launch_bounds__(kPkWarps * 32, 2)
     k_numeric_fp64_pk(DevMat A, DevMat B, DevOut C, DevMat Cin, double alpha, double beta,
                       DevWs ws, const DevStatus *st, const int32_t *items, const int64_t *seg,
-                      unsigned long long *work) {
+                      unsigned long long *work, int ntiles) {
   if (st->overflow) return;
   extern __shared__ double smem_pk[];
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
@@ -803,6 +810,12 @@ __global__ void __launch_bounds__(kPkWarps * 32, 2)
   work_range(st, seg, wb, we);
   // the second destination (host memory) when the whole result fits it
   double *hout = (C.host_vals && st->nnz_c <= C.host_cap) ? C.host_vals : nullptr;
+  int parts = 1;
+  if (ntiles > 0) {
+    const int64_t warps = (int64_t)gridDim.x * kPkWarps;
+    parts = (int)min((int64_t)ntiles, max((int64_t)1, kPkUnits * warps / max((int64_t)1, we - wb)));
+    we = wb + (we - wb) * parts;
+  }
 
   for (;;) {
     unsigned long long got = 0;
@@ -810,8 +823,11 @@ __global__ void __launch_bounds__(kPkWarps * 32, 2)
     const int64_t w0 = wb + (int64_t)__shfl_sync(0xffffffffu, got, 0);
     if (w0 >= we) break;
     const int64_t w1 = (w0 + kPkGrab < we) ? w0 + kPkGrab : we;
-    for (int64_t w = w0; w < w1; w++)
-      pk_block<SLOTS>(A, B, C, Cin, alpha, beta, ws, items ? items[w] : w, wbuf, hout, lane);
+    for (int64_t w = w0; w < w1; w++) {
+      const int64_t b = parts > 1 ? wb + (w - wb) / parts : w;
+      pk_block<SLOTS>(A, B, C, Cin, alpha, beta, ws, items ? items[b] : b,
+                      parts > 1 ? (int)((w - wb) % parts) : 0, parts, wbuf, hout, lane);
+    }
   }
 }
 
@@ -836,12 +852,17 @@ __global__ void __launch_bounds__(kPkWarps * 32, 2)
 // digit pairs stand for one product. (FP8 and INT8 mma.sync are emulated or slow on
 // this part: 3.8 and 16 clocks per m16n8k32 and SM, FP16 m16n8k16 2.0.) Numeric
 // phase, packed kernel -> this one: water of 2048 molecules 47.7 -> 21.4 ms,
-// amorphous of 1024 atoms 67.9 -> 22.5, 64 x 64 full blocks of 32 15.7 -> 2.4. What
+// amorphous of 1024 atoms 67.9 -> 22.5, 64 x 64 full blocks of 32 15.7 -> 2.0. What
 // bounds it: the MMA pipe (0.49 of the clocks of the first) and the instructions beside
 // it, which do not hide behind the MMAs whatever the number of warps (with 16, 20 and 24
 // per SM 21.4, 21.9 and 22.2 ms): left out one at a time, the digits' conversion is
 // 1.5 ms, the search for an octet's product and the loads' misses 4, the 64-bit sums 0.8,
 // the epilogue nothing (L2 and L1 are at 10 and 20%).
+//
+// A warp takes whole C blocks while there are kDgUnits per warp, else parts of their
+// tiles (dense matrices of 8 x 8, 16 x 16, 32 x 32 and 64 x 64 blocks of 32: 0.144,
+// 0.326, 0.628 and 2.40 ms with whole blocks, 0.041, 0.061, 0.281 and 2.04 with parts; up
+// to 16 and 32 units a warp gain nothing more and cost up to 5% on blocks of one tile).
 //
 // The products of a C block are concatenated along k in octets (8 of k), two to an
 // MMA step; a warp takes a tile of up to 16 x 8 (the MMA's shape):
@@ -861,6 +882,7 @@ constexpr int kDgBlocksPerSm = 2;
 constexpr int kDgDiag = 9;              // diagonals kept
 constexpr int kDgFold = 18;             // octets between two reads of the accumulators
 constexpr int kDgGrab = 8;              // C blocks a warp takes at a time, at most
+constexpr int kDgUnits = 8;              // units of work per warp up to which C blocks are split
 
 __device__ __forceinline__ void dg_mma(float (&d)[4], uint32_t a0, uint32_t a1, uint32_t a2,
                                        uint32_t a3, uint32_t b0, uint32_t b1) {
@@ -1052,6 +1074,7 @@ struct DgItem {  // a C block of a warp's run
   const int2 *prods;
   int64_t coff;
   int32_t gblk, np, m, n, cin, fa, fb;
+  int32_t part, nparts;  // the part of its tiles that is to be done
 };
 
 // C blocks without products (C_in only) and those with an operand block outside
@@ -1059,7 +1082,7 @@ struct DgItem {  // a C block of a warp's run
 __global__ void __launch_bounds__(kDgWarps * 32, kDgBlocksPerSm)
     k_numeric_fp64_dg(DevMat A, DevMat B, DevOut C, DevMat Cin, double alpha, double beta,
                       DevWs ws, const DevStatus *st, const int32_t *items, const int64_t *seg,
-                      unsigned long long *work, Digits dg) {
+                      unsigned long long *work, Digits dg, int ntiles) {
   if (st->overflow) return;
   __shared__ DgSum tiles[kDgWarps][16 * 8];
   __shared__ double parts[kDgWarps][16 * 8];
@@ -1072,7 +1095,12 @@ __global__ void __launch_bounds__(kDgWarps * 32, kDgBlocksPerSm)
   work_range(st, seg, wb, we);
   double *hout = (C.host_vals && st->nnz_c <= C.host_cap) ? C.host_vals : nullptr;
   // fewer at a time where that would leave warps without work
-  const int64_t share = (we - wb) / ((int64_t)gridDim.x * kDgWarps * 4);
+  const int64_t warps = (int64_t)gridDim.x * kDgWarps;
+  // the parts of a C block (every nparts-th of its tiles), a unit of work each
+  const int nparts =
+      (int)min((int64_t)ntiles, max((int64_t)1, kDgUnits * warps / max((int64_t)1, we - wb)));
+  we = wb + (we - wb) * nparts;
+  const int64_t share = (we - wb) / (warps * 4);
   const int grab = share >= kDgGrab ? kDgGrab : share < 1 ? 1 : (int)share;
 
   for (;;) {
@@ -1085,7 +1113,10 @@ __global__ void __launch_bounds__(kDgWarps * 32, kDgBlocksPerSm)
     // without a chain of loads
     if (lane < count) {
       DgItem it;
-      it.gblk = items ? items[base + lane] : (int)(base + lane);
+      const int64_t unit = base + lane - wb, blk = nparts > 1 ? wb + unit / nparts : base + lane;
+      it.part = nparts > 1 ? (int)(unit % nparts) : 0;
+      it.nparts = nparts;
+      it.gblk = items ? items[blk] : (int)blk;
       const int64_t pp = ws.prod_ptr[it.gblk];
       it.prods = ws.prods + pp;
       it.np = (int)(ws.prod_ptr[it.gblk + 1] - pp);
@@ -1126,15 +1157,17 @@ __global__ void __launch_bounds__(kDgWarps * 32, kDgBlocksPerSm)
         flags |= dg.a.meta[q.x].y | dg.b.meta[q.y].y;
       }
       if (np == 0 || __any_sync(0xffffffffu, flags & kDigitOutside)) {
-        if (lane == 0)
+        if (lane == 0 && it.part == 0)
           dg.list[atomicAdd(reinterpret_cast<unsigned long long *>(dg.range + 1), 1ull)] = it.gblk;
         metadata();
         continue;
       }
       const int m = it.m, n = it.n;
       const uint2 ka = ma, kb = mb;
+      int at = 0;  // the tile's number
       for (int r0 = 0; r0 < m; r0 += 16) {
         for (int c0 = 0; c0 < n; c0 += 8) {
+          if (it.nparts > 1 && at++ % it.nparts != it.part) continue;
           const int tm = min(16, m - r0), tn = min(8, n - c0);
           // the exponents of the tile's scales: lane r row r's, lane c column c's
           const int xa = dg.a.expo[it.fa + r0 + min(lane, tm - 1)];
@@ -1145,7 +1178,6 @@ __global__ void __launch_bounds__(kDgWarps * 32, kDgBlocksPerSm)
                                  : dg_tile<false>(dg, it.prods, np, ka, kb, m, n, r0 >> 4, c0 >> 3,
                                                   tm, tn, tile, part, &more, lane);
           __syncwarp();
-          if (r0 + 16 >= m && c0 + 8 >= n) metadata();
           const double *cinv = (it.cin >= 0) ? Cin.vals + Cin.blk_off[it.cin] : nullptr;
           const uint32_t rtm = rcp16(tm);
           for (int e0 = 0; e0 < tm * tn; e0 += 32) {
@@ -1167,6 +1199,7 @@ __global__ void __launch_bounds__(kDgWarps * 32, kDgBlocksPerSm)
           __syncwarp();
         }
       }
+      metadata();
     }
     __syncwarp();  // the items are read before the next ones are written
   }
@@ -1180,7 +1213,8 @@ cudaError_t launch_numeric_fp64(int variant, DevMat A, DevMat B, DevOut C, DevMa
   switch (variant) {
     case kFp64Dg:
       k_numeric_fp64_dg<<<grid, kDgWarps * 32, 0, stream>>>(
-          A, B, C, Cin, alpha, beta, ws, st, items, seg, work, *digits);
+          A, B, C, Cin, alpha, beta, ws, st, items, seg, work, *digits,
+          ((max_m + 15) / 16) * ((max_n + 7) / 8));
       break;
     case kFp64G8: {
       const int mr = max_m <= 4 ? 4 : max_m <= 6 ? 6 : 8;
@@ -1210,12 +1244,14 @@ cudaError_t launch_numeric_fp64(int variant, DevMat A, DevMat B, DevOut C, DevMa
       break;
     }
     case kFp64Pk12:
+      // digits: the blocks that the digit kernel left, tile by tile
       k_numeric_fp64_pk<12><<<grid, kPkWarps * 32, pk_smem_bytes(), stream>>>(
-          A, B, C, Cin, alpha, beta, ws, st, items, seg, work);
+          A, B, C, Cin, alpha, beta, ws, st, items, seg, work,
+          digits ? ((max_m + kPkTile - 1) / kPkTile) * ((max_n + kPkTile - 1) / kPkTile) : 0);
       break;
     case kFp64Pk16:
       k_numeric_fp64_pk<16><<<grid, kPkWarps * 32, pk_smem_bytes(), stream>>>(
-          A, B, C, Cin, alpha, beta, ws, st, items, seg, work);
+          A, B, C, Cin, alpha, beta, ws, st, items, seg, work, 0);
       break;
     default:
       k_numeric_fp64_t16<2><<<grid, kSWarps * 32, 0, stream>>>(A, B, C, Cin, alpha, beta, ws, st,

@@ -50,3 +50,29 @@ def test_sum_of_matrices(gpu_ctx, n, top, density):
     assert np.array_equal(got, 2.0 * H.to_dense(B) - 3.0 * H.to_dense(A))
     for M in (dA, dB):
         M.destroy()
+
+
+# C blocks of many tiles, few (parts of one tile each, and of several) to many (whole)
+@pytest.mark.parametrize("launch", [0, 1])
+@pytest.mark.parametrize("n,sizes", [(1, [70]), (3, [33, 100, 1]), (40, [17, 33, 5]), (150, [9, 17])])
+def test_parts_of_blocks(gpu_ctx, n, sizes, launch):
+    """Small integers, so exact; one block of A in ten has a row of its own scale
+    that digits do not hold beside the others (its C blocks go to the packed
+    kernel, in parts)."""
+    rng = np.random.default_rng(n)
+    rs, cs = rng.choice(sizes, n), rng.choice(sizes, n)
+    ks = rng.choice(sizes + [3], 7)
+    A = synth.random_blocks(rng, rs, ks, 0.8 if n > 1 else 1.0, kind="int")
+    B = synth.random_blocks(rng, ks, cs, 0.8 if n > 1 else 1.0, kind="int")
+    off = H.block_list_offsets(A)
+    for b in range(0, len(A.blk_row), 10):
+        blk = A.values[off[b]:off[b + 1]].reshape(-1, A.row_sizes[A.blk_row[b]])
+        blk[:, 0] *= 2.0 ** -30
+    dA, dB = gpu_ctx.from_blocks(A), gpu_ctx.from_blocks(B)
+    dC = gpu_ctx.empty(A.row_sizes, B.col_sizes)
+    gpu_ctx.multiply(1.0, dA, dB, 0.0, dC, 0.0, launch=launch, blocking=True)
+    r, c = dC.pattern()
+    got = H.to_dense(BlockMatrix(A.row_sizes, B.col_sizes, r, c, dC.values()))
+    assert np.array_equal(got, H.to_dense(A) @ H.to_dense(B))
+    for M in (dA, dB, dC):
+        M.destroy()
