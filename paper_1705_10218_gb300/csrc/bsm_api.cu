@@ -2227,6 +2227,10 @@ int bsm_sync(bsm_ctx ctx) {
 
 namespace bsm {
 
+// Values are uploaded in pieces of 4 MB: the copies of other lanes' small matrices
+// take their turn between a large one's pieces instead of waiting for all of it.
+constexpr int64_t kUploadPiece = 1 << 19;
+
 int mat_create_diag(bsm_ctx ctx, int nparts, const DiagPart *parts, bsm_mat *out) {
   if (!ctx || !out || nparts < 0 || (nparts > 0 && !parts)) return BSM_ERR_INVALID_ARG;
   *out = nullptr;
@@ -2295,9 +2299,11 @@ int mat_create_diag(bsm_ctx ctx, int nparts, const DiagPart *parts, bsm_mat *out
   int64_t hdr[2] = {nblk, nnz};
   cudaError_t e;
   for (int p = 0; p < nparts; p++)
-    if ((e = cp(M->front.vals + val0[p], parts[p].vals, (size_t)(val0[p + 1] - val0[p]) * 8)) !=
-        cudaSuccess)
-      return fail(cuda_fail(e, "diagonal upload values"));
+    for (int64_t v = val0[p]; v < val0[p + 1]; v += kUploadPiece) {
+      const int64_t n = std::min(kUploadPiece, val0[p + 1] - v);
+      if ((e = cp(M->front.vals + v, parts[p].vals + (v - val0[p]), (size_t)n * 8)) != cudaSuccess)
+        return fail(cuda_fail(e, "diagonal upload values"));
+    }
   if ((e = cp(M->front.row_ptr, h_row_ptr, ((size_t)nbr + 1) * 4)) != cudaSuccess ||
       (e = cp(M->front.col_idx, h_col, (size_t)nblk * 4)) != cudaSuccess ||
       (e = cp(M->front.blk_row, h_row, (size_t)nblk * 4)) != cudaSuccess ||
