@@ -198,7 +198,7 @@ __device__ __forceinline__ void mma_tf32_k8(float (&d)[4], const uint32_t (&a)[4
 }
 
 // ---------------------------------------------------------------------------
-// Numeric kernel (below). A warp computes one C block at a time, or its
+// Numeric kernels (below). A warp computes one C block at a time, or its
 // transpose, whichever needs fewer 16x8 MMA tiles. Operands: L (Mp rows along
 // k) and R (Np rows along k), both k-piece-major. Not transposed: L = A_ik (A's
 // left layout), R = B_kj (B's right layout); transposed (C^T = B^T A^T): L =
@@ -221,78 +221,6 @@ __device__ __forceinline__ void two_sum_acc(float &hi, float &lo, float x) {
   lo = __fadd_rn(lo, err);
 }
 
-// ---------------------------------------------------------------------------
-// Pipelined kernel. Two instances: C blocks whose MMA problem fits 16 x 16
-// (the water and small-block case; 1x2 tiles per warp, 16-row slots), and the
-// others up to 32 x 32 (2x4 tiles per warp, 32-row slots, tiles outside the
-// problem skipped). Each warp streams its C blocks' products through a ring
-// of STAGES shared-memory slots. For every product one lane starts two bulk
-// asynchronous copies (cp.async.bulk: all slice planes of the left operand in
-// one, of the right one in the other) whose completion is counted in bytes on
-// the slot's mbarrier, STAGES - 1 products ahead of the tensor-core work, so
-// the L2 latency of a product's operands is hidden behind the products before
-// it; the fragments are read from the slot with ldmatrix, conflict-free thanks
-// to the k-piece-major planes. The (A offset, B offset, k) of the products are
-// read 32 at a time into a per-warp table in shared memory.
-// ---------------------------------------------------------------------------
-// Ring depth: deeper rings hide more copy latency, shallower ones leave room
-// for more warps per SM. Measured on water (k of 5 and 13): 2 stages beat 3, 4
-// and 6 (6 stages leave 8 warps per SM): each warp's chain of dependent
-// fragment loads and MMAs needs many warps to fill the issue slots.
-constexpr int kPipeStages = 2;
-constexpr int kPipeWarps = 4;
-// Products summed plainly in FP32 before each compensated fold: a partial sum
-// of kFold products carries kFold times the rounding of one, still far below
-// the slice truncation error, and the fold costs 6 FP32 operations per value.
-constexpr int kFold = 4;
-constexpr int kMetaEntries = 64;
-constexpr int kMetaBytes = kMetaEntries * (8 + 8 + 4);
-// A waiting thread is suspended until the phase completes or kWaitHintNs
-// pass (no issue slots spent on polling); after kWaitPolls such waits (about
-// a second) a warp gives up on a copy that does not land: it then raises the
-// status error flag, waits (again bounded) for the copies it has in flight and
-// stops.
-constexpr uint32_t kWaitHintNs = 1000;
-constexpr int kWaitPolls = 1 << 20;
-
-__device__ __forceinline__ void mbar_init(uint32_t bar, uint32_t count) {
-  asm volatile("mbarrier.init.shared::cta.b64 [%0], %1;\n" ::"r"(bar), "r"(count) : "memory");
-}
-__device__ __forceinline__ void mbar_init_fence() {
-  asm volatile("fence.mbarrier_init.release.cluster;\n" ::: "memory");
-}
-// generic-proxy accesses of shared memory (ldmatrix reads of a slot) before
-// async-proxy writes of it (the next bulk copy into the slot)
-__device__ __forceinline__ void fence_proxy_async_smem() {
-  asm volatile("fence.proxy.async.shared::cta;\n" ::: "memory");
-}
-__device__ __forceinline__ void mbar_expect_tx(uint32_t bar, uint32_t bytes) {
-  asm volatile("mbarrier.arrive.expect_tx.shared::cta.b64 _, [%0], %1;\n" ::"r"(bar), "r"(bytes)
-               : "memory");
-}
-__device__ __forceinline__ void bulk_copy_g2s(uint32_t dst, const void *src, uint32_t bytes,
-                                              uint32_t bar) {
-  asm volatile(
-      "cp.async.bulk.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1], %2, [%3];\n" ::
-          "r"(dst),
-      "l"(src), "r"(bytes), "r"(bar)
-      : "memory");
-}
-__device__ __forceinline__ bool mbar_test(uint32_t bar, uint32_t parity) {
-  uint32_t ok;
-  asm volatile(
-      "{\n .reg .pred p;\n mbarrier.try_wait.parity.shared::cta.b64 p, [%1], %2, %3;\n"
-      " selp.u32 %0, 1, 0, p;\n}\n"
-      : "=r"(ok)
-      : "r"(bar), "r"(parity), "r"(kWaitHintNs)
-      : "memory");
-  return ok != 0;
-}
-__device__ __forceinline__ bool mbar_wait(uint32_t bar, uint32_t parity) {
-  for (int i = 0; i < kWaitPolls; i++)
-    if (mbar_test(bar, parity)) return true;
-  return false;
-}
 __device__ __forceinline__ void ldsm_x4(uint32_t &r0, uint32_t &r1, uint32_t &r2, uint32_t &r3,
                                         uint32_t addr) {
   asm volatile("ldmatrix.sync.aligned.m8n8.x4.shared.b16 {%0, %1, %2, %3}, [%4];\n"
@@ -305,448 +233,338 @@ __device__ __forceinline__ void ldsm_x2(uint32_t &r0, uint32_t &r1, uint32_t add
                : "r"(addr));
 }
 
-// Bytes of one row of a plane (k up to s, whole 16-byte pieces), and of one
-// operand slot: all planes of at most `rows` rows (16, or 32 in the large-block
-// instance) of k up to smax.
-__host__ __device__ __forceinline__ int pipe_row_bytes(int precision, int s) {
-  return precision == BSM_PREC_SPLIT_BF16X3 ? 2 * ((s + 7) & ~7) : 4 * ((s + 3) & ~3);
-}
-__host__ __device__ __forceinline__ int pipe_operand_bytes(int precision, int smax, int rows) {
-  return (precision == BSM_PREC_SPLIT_BF16X3 ? 3 : 2) * rows * pipe_row_bytes(precision, smax);
-}
-// per warp: the slots, the product table, one mbarrier per slot (16-byte multiple)
-__host__ __device__ __forceinline__ int pipe_warp_bytes(int precision, int smax, int stages,
-                                                        int rows) {
-  return stages * 2 * pipe_operand_bytes(precision, smax, rows) + kMetaBytes +
-         ((8 * stages + 15) & ~15);
-}
-// The large-block instance (MMA problems up to 32x32, 2x4 tiles of 16x8 per
-// warp, 32-row slots): 2 warps per thread block, 2 stages.
-constexpr int kPipeWarpsBig = 2;
+// ---------------------------------------------------------------------------
+// Per-block kernel. The operands' slices go from L1/L2 straight into the MMA's
+// registers. Of the four lanes that share a row of an MMA operand, lanes 0 and 1 take
+// the halves of a 16-byte piece, lanes 2 and 3 those of the next: their values are the
+// MMA's k positions of these lanes (2t, 2t + 1, 2t + 8, 2t + 9 of a BF16 k16 step, t and
+// t + 4 of a TF32 k8 step), as an MMA's sum does not depend on the order of its k
+// positions if both operands have the same. So two pieces of k are a k step, and eight
+// rows of a plane one load instruction over two runs of 128 bytes; nothing is staged.
+// (Whole pieces, a 16-byte load a lane over four runs: each quarter of a load touches
+// four lines, and the L1 is busy 0.78 of the time. Single words in the order of the
+// MMA's registers: the same time. Loads of a step ahead, or 24 warps per SM: registers
+// spill, slower.)
+//
+// The products of a C block follow one another in steps of two pieces, 16 of which are
+// looked up at a time (a lane each piece, into shared memory); a product's last step is
+// filled up with a piece of zeros. (Steps across products would be fewer, 4.6 instead of
+// 6.3 ms below, but would change the order of the roundings: sums stay the bits that the
+// products one after another give.) L is the operand on the MMA's 16 rows, R on its 8
+// columns; a warp takes a tile of up to 16 x 16:
+//   kHalf: up to 8 x 8 (the lower half of the MMA's rows repeats the upper one);
+//   kOne:  up to 16 x 8;  kTwo: up to 16 x 16.
+// The blocks of a warp's run that follow one another in C are gathered and leave in
+// 256-byte stores, which the link to host memory needs (a block at a time: 141 of its
+// 193 GB/s).
+//
+// Against one bulk copy per operand and product into a ring in shared memory and
+// ldmatrix, which cost 45 clocks of an SM per copy; numeric phase: water of 1024
+// molecules, BF16x3, values also to host memory 10.4 -> 6.28 ms, without 7.8 -> 6.27;
+// amorphous of 600 atoms, TF32x2 8.96 -> 6.87. Bound by the L1 (0.61 of its load slots:
+// the runs are not aligned to lines) and the latency of its misses; 16 warps per SM
+// issue 1.9 instructions a clock, 24 no more; the MMAs are 0.2 of the time.
+// ---------------------------------------------------------------------------
+constexpr int kSbWarps = 8;
+constexpr int kSbBlocksPerSm = 2;
+constexpr int kSbStage = 512;    // values gathered at most
+constexpr int kSbCarveout = 60;  // % of an SM's L1 as shared memory: what two blocks need
+constexpr int kSbGrab = 8;  // C blocks a warp takes at a time, at most
 
-// A C block of the pipelined kernel's stream: gb < 0 marks the end of the work.
-struct PipeBlock {
-  int64_t gb, p0;
-  int np, m, n;
+__device__ const uint4 g_zero_pieces[32] = {};  // a piece of zeros for each row
+
+struct SbItem {  // a C block of a warp's run
+  const int2 *prods;
+  int64_t coff, cin;  // cin: offset of its C_in block, or -1
+  int32_t np, m, n;
+};
+struct SbPiece {  // a piece of k: where row 0's lies in both operands' first planes, and
+  const uint4 *a, *b;  // the distance of the planes in rows
+};
+struct SbWarp {  // a warp's shared memory
+  float2 tile[16 * 16];  // hi and lo of a tile, column-major as in C
+  double stage[kSbStage];  // values of finished blocks that follow one another in C
+  SbPiece piece[32];
+  int32_t pieces[32];  // the product's pieces (0: a piece of zeros)
+  SbItem item[kSbGrab];
 };
 
-// Minimum resident blocks per SM the register budget is fitted to: the kernel
-// is bound by instruction issue and latency, so more resident warps pay, but
-// not at the price of spills (6 blocks of the 2-stage instance spill; the
-// TF32 slots are larger: 5 blocks of 2 stages fill the shared memory).
-// The large-block instance: 4 blocks of 2 warps (up to 255 registers).
-template <int PREC, int STAGES, bool BIG>
-constexpr int pipe_min_blocks() {
-  return BIG ? 4
-             : PREC == BSM_PREC_SPLIT_BF16X3 ? (STAGES == 2 ? 5 : STAGES == 3 ? 5 : 4)
-                                             : (STAGES == 2 ? 5 : 4);
-}
+constexpr int kSbFold = 1 << 8;  // in SbWarp::pieces: the sums are folded after the step
+// Products summed plainly in FP32 before each compensated fold: a partial sum
+// of kFold products carries kFold times the rounding of one, still far below
+// the slice truncation error.
+constexpr int kFold = 4;
 
-// sel: 0 every C block, 1 those whose MMA problem fits 16x16, 2 the others.
-template <int PREC, int STAGES, bool BIG>
-__global__ void __launch_bounds__((BIG ? kPipeWarpsBig : kPipeWarps) * 32,
-                                  pipe_min_blocks<PREC, STAGES, BIG>())
-    k_numeric_split_pipe(DevMat A, DevMat B, DevOut C, DevMat Cin, const void *__restrict__ a_left,
-                         const void *__restrict__ b_right, double alpha, double beta, DevWs ws,
-                         const DevStatus *st, const int32_t *__restrict__ items,
-                         const int64_t *__restrict__ seg, int smax, int sel,
-                         unsigned long long *work) {
-  if (st->overflow) return;
+enum SbTile { kHalf, kOne, kTwo };
+
+// One tile, into w.tile: rows l0 to l0 + tl - 1 of L, r0 to r0 + tr - 1 of R (swap: L is
+// B). a, b, pc: where the operands of product `lane` start, and its pieces of k (0: none).
+template <int PREC, SbTile TILE>
+__device__ __forceinline__ void sb_tile(SbWarp &w, const uint4 *a, const uint4 *b, int pc,
+                                        const SbItem &it, int l0, int tl, int r0, int tr, bool swap,
+                                        const DevMat &A, const DevMat &B,
+                                        const uint4 *__restrict__ a_left,
+                                        const uint4 *__restrict__ b_right, int lane) {
   constexpr bool BF = (PREC == BSM_PREC_SPLIT_BF16X3);
-  constexpr int NSL = BF ? 3 : 2;
-  constexpr int ROWS = BIG ? 32 : 16;  // slot rows
-  constexpr int MT = BIG ? 2 : 1, NT = BIG ? 4 : 2;  // 16x8 tiles per warp
-  constexpr int NP = NT / 2;  // pairs of 8-column tiles (one x4 fragment load)
-  // slice bytes per FP64 value of an operand's offset
-  constexpr int64_t kUnit = BF ? 2 * kBf16HalfwordsPerValue : 4 * kTf32WordsPerValue;
-  extern __shared__ __align__(16) unsigned char smem_pipe[];
-  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+  constexpr int NSL = BF ? 3 : 2, NPQ = BF ? 6 : 3, VPP = BF ? 8 : 4;
+  constexpr int64_t kUnit = BF ? 3 : 2;  // pieces per FP64 value of an operand's offset
+  constexpr int NT = TILE == kTwo ? 2 : 1;
+  // slice products, smallest first: (3,1) (2,2) (1,3) (2,1) (1,2) (1,1); (2,1) (1,2) (1,1)
+  constexpr int PA[6] = {BF ? 2 : 1, BF ? 1 : 0, 0, 1, 0, 0};
+  constexpr int PB[6] = {0, 1, BF ? 2 : 0, 0, 1, 0};
   const int g = lane >> 2, t = lane & 3;
-  const int opb = pipe_operand_bytes(PREC, smax, ROWS);
-  unsigned char *wbase = smem_pipe + warp * pipe_warp_bytes(PREC, smax, STAGES, ROWS);
-  // the product table, a ring indexed by stream position: source addresses of
-  // the two operands' slices and k
-  const unsigned char **meta_a = reinterpret_cast<const unsigned char **>(wbase + STAGES * 2 * opb);
-  const unsigned char **meta_b = meta_a + kMetaEntries;
-  int *meta_s = reinterpret_cast<int *>(meta_b + kMetaEntries);
-  const uint32_t sbase = (uint32_t)__cvta_generic_to_shared(wbase);
-  const uint32_t bar0 = sbase + (uint32_t)(STAGES * 2 * opb + kMetaBytes);
-  if (lane == 0) {
+  const int nl = swap ? it.n : it.m, nr = swap ? it.m : it.n;
+  // the lane's rows (past the last one: the last one again)
+  const int rl = l0 + min(g, tl - 1), rl8 = l0 + min(g + 8, tl - 1) - rl;
+  const int rr = r0 + min(g, tr - 1), rr8 = r0 + min(g + 8, tr - 1) - rr;
+  float hi[NT][4], lo[NT][4], acc[NT][4];
 #pragma unroll
-    for (int x = 0; x < STAGES; x++) mbar_init(bar0 + 8 * x, 1);
-    mbar_init_fence();
-  }
-  __syncwarp();
-  // which 8 x 8 piece (rows 0-7 or 8-15, k piece 0 or 1 of the step) this
-  // lane addresses in ldmatrix: "a" order for the left operand (and for the
-  // right one in BF16 k8 steps), "b" order for the right one
-  const int ra = (lane & 7) + ((lane >> 3) & 1) * 8, pa = lane >> 4;
-  const int rb_ = (lane & 7) + (lane >> 4) * 8, pb = (lane >> 3) & 1;
-
-  int64_t wb = 0, we = st->nblk_c;
-  if (seg) {
-    wb = seg[0];
-    we = seg[1];
-  }
-  const bool plain = (alpha == 1.0 && beta == 0.0);
-  // The products of the C blocks a warp takes form one stream; stream position
-  // u uses ring slot u % STAGES (mbarrier phase (u / STAGES) & 1) and table
-  // entry u % kMetaEntries. Copies run STAGES - 1 positions ahead of the
-  // tensor-core work, across C block boundaries (into the next block's first
-  // products), so the ring does not drain between blocks.
-  uint32_t u_issue = 0, u_done = 0;  // next position to copy / to compute
-  bool failed = false;
-  unsigned long long next = 0;  // the work counter's next index, fetched ahead
-  if (lane == 0) next = atomicAdd(work, 1ull);
-  PipeBlock cur, nxt;
-  int cur_issued = 0, nxt_issued = 0;  // products of the block started so far
-  bool have_nxt = false;
-
-  // the next C block of this launch (warp-uniform); gb < 0: none left
-  auto take = [&](PipeBlock &b) {
-    for (;;) {
-      const int64_t w = wb + (int64_t)__shfl_sync(0xffffffffu, next, 0);
-      if (w >= we) {
-        b.gb = -1;
-        b.np = 0;
-        return;
+  for (int nt = 0; nt < NT; nt++)
+#pragma unroll
+    for (int x = 0; x < 4; x++) hi[nt][x] = lo[nt][x] = acc[nt][x] = 0.f;
+  for (int pb = 0; pb < it.np; pb += 32) {
+    if (pb > 0) {
+      pc = 0;
+      if (pb + lane < it.np) {
+        const int2 pr = __ldg(it.prods + pb + lane);
+        a = a_left + kUnit * A.blk_off[pr.x];
+        b = b_right + kUnit * B.blk_off[pr.y];
+        pc = (A.col_sizes[A.col_idx[pr.x]] + VPP - 1) / VPP;
       }
-      if (lane == 0) next = atomicAdd(work, 1ull);
-      const int64_t gb = items ? items[w] : w;
-      const int i = C.blk_row[gb], j = C.col_idx[gb];
-      const int m = C.row_sizes[i], n = C.col_sizes[j];
-      const int tiles_n = ((m + 15) >> 4) * ((n + 7) >> 3);
-      const int tiles_t = ((n + 15) >> 4) * ((m + 7) >> 3);
-      const bool tr = tiles_t < tiles_n;
-      const int Mp = tr ? n : m, Np = tr ? m : n;
-      const bool small = Mp <= 16 && Np <= 16;
-      if ((sel == 1 && !small) || (sel == 2 && small)) continue;
-      b.gb = gb;
-      b.p0 = ws.prod_ptr[gb];
-      b.np = (int)(ws.prod_ptr[gb + 1] - b.p0);
-      b.m = m;
-      b.n = n;
-      return;
     }
-  };
-  // start the copies of product q of block b at stream position u_issue (all
-  // lanes call; the table holds the next 32 products of b from q % 32 == 0)
-  auto issue = [&](const PipeBlock &b, int q) {
-    const uint32_t u = u_issue++;
-    if ((q & 31) == 0) {
-      const int qq = q + lane;
-      if (qq < b.np) {
-        const int2 pr = ws.prods[b.p0 + qq];
-        const int e = (int)((u + (uint32_t)lane) & (kMetaEntries - 1));
-        meta_a[e] = static_cast<const unsigned char *>(a_left) + kUnit * A.blk_off[pr.x];
-        meta_b[e] = static_cast<const unsigned char *>(b_right) + kUnit * B.blk_off[pr.y];
-        meta_s[e] = A.col_sizes[A.col_idx[pr.x]];
-      }
+    const int even = (pc + 1) & ~1;
+    int incl = even;
+#pragma unroll
+    for (int d = 1; d < 32; d <<= 1) {
+      const int y = __shfl_up_sync(0xffffffffu, incl, d);
+      if (lane >= d) incl += y;
+    }
+    const int slots = __shfl_sync(0xffffffffu, incl, 31);
+    // where the product's piece number 0 of the whole batch would be
+    const uint4 *a0 = a - (int64_t)(incl - even) * it.m, *b0 = b - (int64_t)(incl - even) * it.n;
+#pragma unroll 1
+    for (int s0 = 0; s0 < slots; s0 += 32) {
+      const int s = s0 + lane;
+      int p = 0;  // products that end at or before slot s
+#pragma unroll
+      for (int step = 16; step; step >>= 1)
+        if (__shfl_sync(0xffffffffu, incl, p + step - 1) <= s) p += step;
+      SbPiece e;
+      e.a = (const uint4 *)__shfl_sync(0xffffffffu, (unsigned long long)a0, p) + s * it.m;
+      e.b = (const uint4 *)__shfl_sync(0xffffffffu, (unsigned long long)b0, p) + s * it.n;
+      int num = __shfl_sync(0xffffffffu, pc, p);
+      const int begin = __shfl_sync(0xffffffffu, incl - even, p);
+      // the step of this slot is the last one before a fold: of every kFold-th product
+      // and of the last one
+      const bool fold = s - begin >= num - 2 && ((p % kFold) == kFold - 1 || pb + p == it.np - 1);
+      if (s - begin >= num) e.a = e.b = g_zero_pieces, num = 0;
+      if (fold) num |= kSbFold;
       __syncwarp();
-    }
-    if (lane == 0) {
-      const int e = (int)(u & (kMetaEntries - 1));
-      const int rb = pipe_row_bytes(PREC, meta_s[e]);
-      const uint32_t bytes_a = (uint32_t)(NSL * b.m * rb), bytes_b = (uint32_t)(NSL * b.n * rb);
-      const uint32_t slot = u % STAGES;
-      const uint32_t dst = sbase + slot * 2 * (uint32_t)opb, bar = bar0 + 8 * slot;
-      fence_proxy_async_smem();
-      mbar_expect_tx(bar, bytes_a + bytes_b);
-      bulk_copy_g2s(dst, meta_a[e], bytes_a, bar);
-      bulk_copy_g2s(dst + (uint32_t)opb, meta_b[e], bytes_b, bar);
-    }
-  };
-
-  take(cur);
-  while (cur_issued < cur.np && (int)(u_issue - u_done) < STAGES - 1) issue(cur, cur_issued++);
-  while (cur.gb >= 0) {
-    const int m = cur.m, n = cur.n;
-    const int tiles_n = ((m + 15) >> 4) * ((n + 7) >> 3);
-    const int tiles_t = ((n + 15) >> 4) * ((m + 7) >> 3);
-    const bool tr = tiles_t < tiles_n;
-    const int Mp = tr ? n : m, Np = tr ? m : n;
-    const bool two = Np > 8;  // a second 8-column tile
-    float hi[MT][NT][4], lo[MT][NT][4], acc[MT][NT][4];
-#pragma unroll
-    for (int mt = 0; mt < MT; mt++)
-#pragma unroll
-      for (int nt = 0; nt < NT; nt++)
-#pragma unroll
-        for (int x = 0; x < 4; x++) hi[mt][nt][x] = lo[mt][nt][x] = acc[mt][nt][x] = 0.f;
-
-    for (int q = 0; q < cur.np; q++) {
-      const uint32_t u = u_done, slot = u % STAGES;
-      if (!__all_sync(0xffffffffu, mbar_wait(bar0 + 8 * slot, (u / STAGES) & 1u))) {
-        failed = true;
-        break;
-      }
-      u_done++;
+      w.piece[lane] = swap ? SbPiece{e.b, e.a} : e;
+      w.pieces[lane] = num;
       __syncwarp();
-      // refill the slot the previous position used: the next product of this
-      // block, else the first ones of the next block
-      if (cur_issued < cur.np) {
-        issue(cur, cur_issued++);
-      } else {
-        if (!have_nxt) {
-          take(nxt);
-          nxt_issued = 0;
-          have_nxt = true;
+      const int end = min(32, slots - s0);
+      struct Raw {  // two pieces of k of both operands
+        uint2 l[NSL], l8[NSL], r[NSL][NT];
+      };
+      auto load = [&](Raw &f, int o) {
+        const SbPiece at = w.piece[o + (t >> 1)];
+        const int np = w.pieces[o + (t >> 1)] & (kSbFold - 1);
+        const uint2 *xl = reinterpret_cast<const uint2 *>(at.a + rl) + (t & 1);
+        const uint2 *xr = reinterpret_cast<const uint2 *>(at.b + rr) + (t & 1);
+#pragma unroll
+        for (int q = 0; q < NSL; q++) {
+          f.l[q] = __ldg(xl + 2 * q * np * nl);
+          f.l8[q] = TILE == kHalf ? f.l[q] : __ldg(xl + 2 * (q * np * nl + rl8));
+          f.r[q][0] = __ldg(xr + 2 * q * np * nr);
+          if (TILE == kTwo) f.r[q][NT - 1] = __ldg(xr + 2 * (q * np * nr + rr8));
         }
-        if (nxt_issued < nxt.np) issue(nxt, nxt_issued++);
-      }
-      const int s = meta_s[u & (kMetaEntries - 1)];
-      const int rb = pipe_row_bytes(PREC, s);
-      const uint32_t sA = sbase + slot * 2 * (uint32_t)opb, sB = sA + (uint32_t)opb;
-      // L (Mp rows) and R (Np rows) in the slot; plane strides rows * rb
-      const uint32_t sL = tr ? sB : sA, sR = tr ? sA : sB;
-      const uint32_t lpl = (uint32_t)(Mp * rb), rpl = (uint32_t)(Np * rb);
-      // this lane's piece address at k step 0; a k piece column is rows * 16 bytes
-      const uint32_t adL = sL + 16u * (uint32_t)(pa * Mp + ra);
-      const uint32_t adR = sR + 16u * (uint32_t)(pb * Np + rb_);
-      const uint32_t adR2 = sR + 16u * (uint32_t)ra;  // "a" order on R (half steps)
-      if constexpr (BIG) {
-        // tile (mt, nt) is live when it holds part of the Mp x Np problem
-        bool live[MT][NT];
+      };
+      auto mma = [&](const Raw &f, bool fold) {
 #pragma unroll
-        for (int mt = 0; mt < MT; mt++)
+        for (int pq = 0; pq < NPQ; pq++)
 #pragma unroll
-          for (int nt = 0; nt < NT; nt++) live[mt][nt] = mt * 16 < Mp && nt * 8 < Np;
-        if (BF) {
-          constexpr int PA[6] = {2, 1, 0, 1, 0, 0};
-          constexpr int PB[6] = {0, 1, 2, 0, 1, 0};
-          for (int kk = 0; kk < s; kk += 16) {
-            const uint32_t koL = 16u * (uint32_t)((kk >> 3) * Mp), koR = 16u * (uint32_t)((kk >> 3) * Np);
-            if (s - kk <= 8) {  // one k piece left: m16n8k8
-              uint32_t a[3][MT][2], b[3][NP][2];
-#pragma unroll
-              for (int q3 = 0; q3 < 3; q3++) {
-#pragma unroll
-                for (int mt = 0; mt < MT; mt++)
-                  ldsm_x2(a[q3][mt][0], a[q3][mt][1], adL + q3 * lpl + koL + 256u * mt);
-#pragma unroll
-                for (int p2 = 0; p2 < NP; p2++)
-                  ldsm_x2(b[q3][p2][0], b[q3][p2][1], adR2 + q3 * rpl + koR + 256u * p2);
-              }
-#pragma unroll
-              for (int pq = 0; pq < 6; pq++)
-#pragma unroll
-                for (int mt = 0; mt < MT; mt++)
-#pragma unroll
-                  for (int nt = 0; nt < NT; nt++)
-                    if (live[mt][nt])
-                      mma_bf16_k8(acc[mt][nt], a[PA[pq]][mt][0], a[PA[pq]][mt][1],
-                                  b[PB[pq]][nt >> 1][nt & 1]);
-            } else {
-              uint32_t a[3][MT][4], b[3][NP][4];
-#pragma unroll
-              for (int q3 = 0; q3 < 3; q3++) {
-#pragma unroll
-                for (int mt = 0; mt < MT; mt++)
-                  ldsm_x4(a[q3][mt][0], a[q3][mt][1], a[q3][mt][2], a[q3][mt][3],
-                          adL + q3 * lpl + koL + 256u * mt);
-#pragma unroll
-                for (int p2 = 0; p2 < NP; p2++)
-                  ldsm_x4(b[q3][p2][0], b[q3][p2][1], b[q3][p2][2], b[q3][p2][3],
-                          adR + q3 * rpl + koR + 256u * p2);
-              }
-#pragma unroll
-              for (int pq = 0; pq < 6; pq++)
-#pragma unroll
-                for (int mt = 0; mt < MT; mt++)
-#pragma unroll
-                  for (int nt = 0; nt < NT; nt++)
-                    if (live[mt][nt])
-                      mma_bf16_k16(acc[mt][nt], a[PA[pq]][mt], b[PB[pq]][nt >> 1][2 * (nt & 1)],
-                                   b[PB[pq]][nt >> 1][2 * (nt & 1) + 1]);
-            }
+          for (int nt = 0; nt < NT; nt++) {
+            const uint2 &x = f.l[PA[pq]], &y = f.l8[PA[pq]], &z = f.r[PB[pq]][nt];
+            const uint32_t u[4] = {x.x, y.x, x.y, y.y};
+            if (BF)
+              mma_bf16_k16(acc[nt], u, z.x, z.y);
+            else
+              mma_tf32_k8(acc[nt], u, z.x, z.y);
           }
-        } else {
-          constexpr int PA[3] = {1, 0, 0};
-          constexpr int PB[3] = {0, 1, 0};
-          for (int kk = 0; kk < s; kk += 8) {
-            const uint32_t koL = 16u * (uint32_t)((kk >> 2) * Mp), koR = 16u * (uint32_t)((kk >> 2) * Np);
-            uint32_t a[2][MT][4], b[2][NP][4];
-            if (s - kk <= 4) {  // one k piece left: the other half is zero
-#pragma unroll
-              for (int q2 = 0; q2 < 2; q2++) {
-#pragma unroll
-                for (int mt = 0; mt < MT; mt++) {
-                  ldsm_x2(a[q2][mt][0], a[q2][mt][1], adL + q2 * lpl + koL + 256u * mt);
-                  a[q2][mt][2] = a[q2][mt][3] = 0u;
-                }
-#pragma unroll
-                for (int p2 = 0; p2 < NP; p2++) {
-                  ldsm_x2(b[q2][p2][0], b[q2][p2][2], adR2 + q2 * rpl + koR + 256u * p2);
-                  b[q2][p2][1] = b[q2][p2][3] = 0u;
-                }
-              }
-            } else {
-#pragma unroll
-              for (int q2 = 0; q2 < 2; q2++) {
-#pragma unroll
-                for (int mt = 0; mt < MT; mt++)
-                  ldsm_x4(a[q2][mt][0], a[q2][mt][1], a[q2][mt][2], a[q2][mt][3],
-                          adL + q2 * lpl + koL + 256u * mt);
-#pragma unroll
-                for (int p2 = 0; p2 < NP; p2++)
-                  ldsm_x4(b[q2][p2][0], b[q2][p2][1], b[q2][p2][2], b[q2][p2][3],
-                          adR + q2 * rpl + koR + 256u * p2);
-              }
-            }
-#pragma unroll
-            for (int pq = 0; pq < 3; pq++)
-#pragma unroll
-              for (int mt = 0; mt < MT; mt++)
-#pragma unroll
-                for (int nt = 0; nt < NT; nt++)
-                  if (live[mt][nt])
-                    mma_tf32_k8(acc[mt][nt], a[PA[pq]][mt], b[PB[pq]][nt >> 1][2 * (nt & 1)],
-                                b[PB[pq]][nt >> 1][2 * (nt & 1) + 1]);
-          }
-        }
-      } else {
-      // slice products, smallest first: (3,1) (2,2) (1,3) (2,1) (1,2) (1,1)
-      // (BF16); (2,1) (1,2) (1,1) (TF32)
-      if (BF) {
-        constexpr int PA[6] = {2, 1, 0, 1, 0, 0};
-        constexpr int PB[6] = {0, 1, 2, 0, 1, 0};
-        for (int kk = 0; kk < s; kk += 16) {
-          const uint32_t koL = 16u * (uint32_t)((kk >> 3) * Mp), koR = 16u * (uint32_t)((kk >> 3) * Np);
-          if (s - kk <= 8) {  // one k piece left: m16n8k8
-            uint32_t a[3][2], b[3][2];
-#pragma unroll
-            for (int q3 = 0; q3 < 3; q3++) {
-              ldsm_x2(a[q3][0], a[q3][1], adL + q3 * lpl + koL);
-              ldsm_x2(b[q3][0], b[q3][1], adR2 + q3 * rpl + koR);
-            }
-            if (two) {
-#pragma unroll
-              for (int pq = 0; pq < 6; pq++) {
-                mma_bf16_k8(acc[0][0], a[PA[pq]][0], a[PA[pq]][1], b[PB[pq]][0]);
-                mma_bf16_k8(acc[0][1], a[PA[pq]][0], a[PA[pq]][1], b[PB[pq]][1]);
-              }
-            } else {
-#pragma unroll
-              for (int pq = 0; pq < 6; pq++)
-                mma_bf16_k8(acc[0][0], a[PA[pq]][0], a[PA[pq]][1], b[PB[pq]][0]);
-            }
-          } else {
-            uint32_t a[3][4], b[3][4];
-#pragma unroll
-            for (int q3 = 0; q3 < 3; q3++) {
-              ldsm_x4(a[q3][0], a[q3][1], a[q3][2], a[q3][3], adL + q3 * lpl + koL);
-              ldsm_x4(b[q3][0], b[q3][1], b[q3][2], b[q3][3], adR + q3 * rpl + koR);
-            }
-            if (two) {
-#pragma unroll
-              for (int pq = 0; pq < 6; pq++) {
-                mma_bf16_k16(acc[0][0], a[PA[pq]], b[PB[pq]][0], b[PB[pq]][1]);
-                mma_bf16_k16(acc[0][1], a[PA[pq]], b[PB[pq]][2], b[PB[pq]][3]);
-              }
-            } else {
-#pragma unroll
-              for (int pq = 0; pq < 6; pq++)
-                mma_bf16_k16(acc[0][0], a[PA[pq]], b[PB[pq]][0], b[PB[pq]][1]);
-            }
-          }
-        }
-      } else {
-        constexpr int PA[3] = {1, 0, 0};
-        constexpr int PB[3] = {0, 1, 0};
-        for (int kk = 0; kk < s; kk += 8) {
-          const uint32_t koL = 16u * (uint32_t)((kk >> 2) * Mp), koR = 16u * (uint32_t)((kk >> 2) * Np);
-          uint32_t a[2][4], b[2][4];
-          if (s - kk <= 4) {  // one k piece left: the other half is zero
-#pragma unroll
-            for (int q2 = 0; q2 < 2; q2++) {
-              ldsm_x2(a[q2][0], a[q2][1], adL + q2 * lpl + koL);
-              ldsm_x2(b[q2][0], b[q2][2], adR2 + q2 * rpl + koR);
-              a[q2][2] = a[q2][3] = b[q2][1] = b[q2][3] = 0u;
-            }
-          } else {
-#pragma unroll
-            for (int q2 = 0; q2 < 2; q2++) {
-              ldsm_x4(a[q2][0], a[q2][1], a[q2][2], a[q2][3], adL + q2 * lpl + koL);
-              ldsm_x4(b[q2][0], b[q2][1], b[q2][2], b[q2][3], adR + q2 * rpl + koR);
-            }
-          }
-          if (two) {
-#pragma unroll
-            for (int pq = 0; pq < 3; pq++) {
-              mma_tf32_k8(acc[0][0], a[PA[pq]], b[PB[pq]][0], b[PB[pq]][1]);
-              mma_tf32_k8(acc[0][1], a[PA[pq]], b[PB[pq]][2], b[PB[pq]][3]);
-            }
-          } else {
-#pragma unroll
-            for (int pq = 0; pq < 3; pq++)
-              mma_tf32_k8(acc[0][0], a[PA[pq]], b[PB[pq]][0], b[PB[pq]][1]);
-          }
-        }
-      }
-      }
-      // every kFold products (and after the last): fold the FP32 partial sum
-      // into the compensated running sum
-      if ((q % kFold) == kFold - 1 || q == cur.np - 1) {
-#pragma unroll
-        for (int mt = 0; mt < MT; mt++)
+        if (fold) {
 #pragma unroll
           for (int nt = 0; nt < NT; nt++)
 #pragma unroll
             for (int x = 0; x < 4; x++) {
-              two_sum_acc(hi[mt][nt][x], lo[mt][nt][x], acc[mt][nt][x]);
-              acc[mt][nt][x] = 0.f;
+              two_sum_acc(hi[nt][x], lo[nt][x], acc[nt][x]);
+              acc[nt][x] = 0.f;
             }
-      }
-    }
-    if (failed) break;
-
-    const int64_t gb = cur.gb;
-    const int cin = ws.c_cin[gb];
-    const double *cinv = (cin >= 0) ? Cin.vals + Cin.blk_off[cin] : nullptr;
-    double *out = C.vals + C.blk_off[gb];
-    double *hblk = (C.host_vals && st->nnz_c <= C.host_cap) ? C.host_vals + C.blk_off[gb] : nullptr;
-#pragma unroll
-    for (int mt = 0; mt < MT; mt++)
-#pragma unroll
-    for (int nt = 0; nt < NT; nt++)
-#pragma unroll
-      for (int x = 0; x < 4; x++) {
-        const int rr = mt * 16 + g + ((x >> 1) << 3);
-        const int cc = nt * 8 + 2 * t + (x & 1);
-        if (rr < Mp && cc < Np) {
-          const int row = tr ? cc : rr, col = tr ? rr : cc;
-          const int64_t e = (int64_t)col * m + row;
-          // FP32 -> FP64 is exact; hi + lo rounded once in FP64
-          double v = (double)hi[mt][nt][x] + (double)lo[mt][nt][x];
-          if (!plain) {
-            v = alpha * v;
-            if (cinv) v = fma(beta, cinv[e], v);
-          }
-          out[e] = v;
-          if (hblk) hblk[e] = v;
+        }
+      };
+#pragma unroll 1
+      for (int o = 0; o < end; o += 4) {
+        Raw f0, f1;
+        load(f0, o);
+        const bool d0 = w.pieces[o] & kSbFold;
+        if (o + 2 < end) {
+          load(f1, o + 2);
+          const bool d1 = w.pieces[o + 2] & kSbFold;
+          mma(f0, d0);
+          mma(f1, d1);
+        } else {
+          mma(f0, d0);
         }
       }
-
-    // the next block (already begun if the ring ran into it)
-    if (!have_nxt) {
-      take(nxt);
-      nxt_issued = 0;
     }
-    cur = nxt;
-    cur_issued = nxt_issued;
-    have_nxt = false;
-    __syncwarp();  // every lane is past its reads of the slots about to be refilled
-    while (cur_issued < cur.np && (int)(u_issue - u_done) < STAGES - 1) issue(cur, cur_issued++);
   }
-  if (failed && lane == 0) atomicOr(const_cast<int32_t *>(&st->error), 1);
-  // copies still in flight into this warp's slots (none unless a wait gave up)
-  for (uint32_t u = u_done; u < u_issue; u++)
-    if (!mbar_wait(bar0 + 8 * (u % STAGES), (u / STAGES) & 1u)) break;
+  // the tile as it lies in C: row + rows of the tile * column
+  __syncwarp();
+  const int ld = swap ? tr : tl;
+#pragma unroll
+  for (int nt = 0; nt < NT; nt++)
+#pragma unroll
+    for (int x = 0; x < (TILE == kHalf ? 2 : 4); x++) {
+      const int u = g + (x >> 1) * 8, v = nt * 8 + 2 * t + (x & 1);
+      if (u < tl && v < tr) w.tile[swap ? u * ld + v : v * ld + u] = make_float2(hi[nt][x], lo[nt][x]);
+    }
+  __syncwarp();
+}
+
+// sel: 0 every C block, 2 those beyond 16 x 16.
+template <int PREC>
+__global__ void __launch_bounds__(kSbWarps * 32, kSbBlocksPerSm)
+    k_numeric_split_blocks(DevMat A, DevMat B, DevOut C, DevMat Cin,
+                           const uint4 *__restrict__ a_left, const uint4 *__restrict__ b_right,
+                           double alpha, double beta, DevWs ws, const DevStatus *st,
+                           const int32_t *__restrict__ items, const int64_t *__restrict__ seg,
+                           int sel, unsigned long long *work) {
+  if (st->overflow) return;
+  constexpr bool BF = (PREC == BSM_PREC_SPLIT_BF16X3);
+  constexpr int VPP = BF ? 8 : 4;
+  constexpr int64_t kUnit = BF ? 3 : 2;
+  extern __shared__ __align__(16) unsigned char smem_sb[];
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+  SbWarp &w = reinterpret_cast<SbWarp *>(smem_sb)[warp];
+  int64_t wb = 0, we = st->nblk_c;
+  if (seg) wb = seg[0], we = seg[1];
+  double *hout = (C.host_vals && st->nnz_c <= C.host_cap) ? C.host_vals : nullptr;
+  const bool plain = (alpha == 1.0 && beta == 0.0);
+  // fewer at a time where that would leave warps without work
+  const int64_t share = (we - wb) / ((int64_t)gridDim.x * kSbWarps * 4);
+  const int grab = share >= kSbGrab ? kSbGrab : share < 1 ? 1 : (int)share;
+
+  for (;;) {
+    unsigned long long got = 0;
+    if (lane == 0) got = atomicAdd(work, (unsigned long long)grab);
+    const int64_t base = wb + (int64_t)__shfl_sync(0xffffffffu, got, 0);
+    if (base >= we) break;
+    const int count = we - base < grab ? (int)(we - base) : grab;
+    if (lane < count) {
+      const int64_t gb = items ? items[base + lane] : base + lane;
+      SbItem it;
+      const int64_t p0 = ws.prod_ptr[gb];
+      it.prods = ws.prods + p0;
+      it.np = (int)(ws.prod_ptr[gb + 1] - p0);
+      it.m = C.row_sizes[C.blk_row[gb]];
+      it.n = C.col_sizes[C.col_idx[gb]];
+      it.coff = C.blk_off[gb];
+      const int cin = ws.c_cin[gb];
+      it.cin = cin >= 0 ? Cin.blk_off[cin] : -1;
+      w.item[lane] = it;
+    }
+    __syncwarp();
+    // a block's first products and where their operands lie are loaded while the
+    // block before is computed
+    int2 pr = make_int2(-1, -1);
+    auto products = [&](int x) {
+      pr = make_int2(-1, -1);
+      if (x < count && lane < w.item[x].np) pr = __ldg(w.item[x].prods + lane);
+    };
+    const uint4 *a = nullptr, *b = nullptr;
+    int pc = 0;
+    auto operands = [&]() {
+      pc = 0;
+      if (pr.x >= 0) {
+        a = a_left + kUnit * A.blk_off[pr.x];
+        b = b_right + kUnit * B.blk_off[pr.y];
+        pc = (A.col_sizes[A.col_idx[pr.x]] + VPP - 1) / VPP;
+      }
+    };
+    products(0);
+    operands();
+    int64_t first = 0;  // where the staged values start in C, and how many there are
+    int held = 0;
+    auto flush = [&]() {
+      // from the start of the 128-byte line that they begin in
+      for (int e = lane - (int)(first & 15); e < held; e += 32)
+        if (e >= 0) {
+          const double v = w.stage[e];
+          __stcs(C.vals + first + e, v);
+          if (hout) __stcs(hout + first + e, v);
+        }
+      held = 0;
+      __syncwarp();
+    };
+    for (int x = 0; x < count; x++) {
+      const SbItem &it = w.item[x];
+      const int m = it.m, n = it.n;
+      const uint4 *ca = a, *cb = b;
+      const int cp = pc;
+      products(x + 1);
+      if (sel == 2 && m <= 16 && n <= 16) {
+        operands();
+        continue;
+      }
+      const bool staged = m * n <= kSbStage;
+      if (held > 0 && (!staged || held + m * n > kSbStage || it.coff != first + held)) flush();
+      if (held == 0) first = it.coff;
+      // the orientation with fewer MMA tiles
+      const bool swap = ((n + 15) >> 4) * ((m + 7) >> 3) < ((m + 15) >> 4) * ((n + 7) >> 3);
+      for (int m0 = 0; m0 < m; m0 += 16)
+        for (int n0 = 0; n0 < n; n0 += 16) {
+          const int tm = min(16, m - m0), tn = min(16, n - n0);
+          const int l0 = swap ? n0 : m0, tl = swap ? tn : tm, r0 = swap ? m0 : n0, tr = swap ? tm : tn;
+          if (tr > 8)
+            sb_tile<PREC, kTwo>(w, ca, cb, cp, it, l0, tl, r0, tr, swap, A, B, a_left, b_right, lane);
+          else if (tl > 8)
+            sb_tile<PREC, kOne>(w, ca, cb, cp, it, l0, tl, r0, tr, swap, A, B, a_left, b_right, lane);
+          else
+            sb_tile<PREC, kHalf>(w, ca, cb, cp, it, l0, tl, r0, tr, swap, A, B, a_left, b_right, lane);
+          if (m0 + 16 >= m && n0 + 16 >= n) operands();
+          const double *cinv = it.cin >= 0 ? Cin.vals + it.cin : nullptr;
+          const int dc = 32 / tm, dr = 32 - dc * tm;
+          int c = lane / tm, r = lane - c * tm;
+          for (int e = lane; e < tm * tn; e += 32) {
+            const float2 s = w.tile[e];
+            // FP32 -> FP64 is exact; hi + lo rounded once in FP64
+            double v = (double)s.x + (double)s.y;
+            const int64_t loc = (int64_t)(n0 + c) * m + m0 + r;
+            if (!plain) {
+              v = alpha * v;
+              if (cinv) v = fma(beta, cinv[loc], v);
+            }
+            if (staged) {
+              w.stage[held + (int)loc] = v;
+            } else {
+              __stcs(C.vals + it.coff + loc, v);
+              if (hout) __stcs(hout + it.coff + loc, v);
+            }
+            r += dr, c += dc;
+            if (r >= tm) r -= tm, c++;
+          }
+          __syncwarp();
+        }
+      if (staged) held += m * n;
+    }
+    if (held > 0) flush();
+    __syncwarp();  // the items are read before the next ones are written
+  }
 }
 
 // ---------------------------------------------------------------------------
 // Chunked kernel: the products of a C block concatenated along k. A warp
-// computes one C block at a time (or its transpose, as the pipelined kernel
+// computes one C block at a time (or its transpose, as the per-block kernel
 // chooses), for the C blocks whose MMA problem fits 16 x 16. The k pieces of
 // the block's products, in ascending k, are staged chunk by chunk into shared
 // memory. A chunk holds whole products, at most PCMAX 16-byte pieces of k, and
@@ -806,7 +624,8 @@ __global__ void __launch_bounds__(kCatWarps * 32)
   const unsigned char **meta_b = meta_a + kCatMeta;
   int *meta_k = reinterpret_cast<int *>(meta_b + kCatMeta);  // pieces of k
   const uint32_t sbase = (uint32_t)__cvta_generic_to_shared(wbase);
-  // ldmatrix lane roles (as in the pipelined kernel)
+  // which 8 x 8 piece (rows 0-7 or 8-15, k piece 0 or 1 of the step) this lane
+  // addresses in ldmatrix: "a" order for the left operand, "b" for the right one
   const int ra = (lane & 7) + ((lane >> 3) & 1) * 8, pa = lane >> 4;
   const int rb_ = (lane & 7) + (lane >> 4) * 8, pb = (lane >> 3) & 1;
   int64_t wb = 0, we = st->nblk_c;
@@ -829,7 +648,7 @@ __global__ void __launch_bounds__(kCatWarps * 32)
     const int tiles_t = ((n + 15) >> 4) * ((m + 7) >> 3);
     const bool tr = tiles_t < tiles_n;
     const int Mp = tr ? n : m, Np = tr ? m : n;
-    if (Mp > 16 || Np > 16) continue;  // the large-block instance of the pipelined kernel
+    if (Mp > 16 || Np > 16) continue;  // the per-block kernel's
     const bool two = Np > 8;
     const int64_t p0 = ws.prod_ptr[gb], p1 = ws.prod_ptr[gb + 1];
     // chunk plane strides of L (Mp rows) and R (Np rows)
@@ -1002,66 +821,20 @@ __global__ void __launch_bounds__(kCatWarps * 32)
   }
 }
 
-// The pipelined kernel's bounded barrier wait on its own: lane 0 completes the
-// phase (a plain arrive), unless never_complete; the warp then waits as the
-// kernel does and records in *flag whether the wait gave up.
-__global__ void k_wait_selftest(int never_complete, int32_t *flag) {
-  __shared__ __align__(8) unsigned long long bar_storage;
-  const uint32_t bar = (uint32_t)__cvta_generic_to_shared(&bar_storage);
-  const int lane = threadIdx.x & 31;
-  if (lane == 0) {
-    mbar_init(bar, 1);
-    mbar_init_fence();
-  }
-  __syncwarp();
-  if (lane == 0 && !never_complete)
-    asm volatile("mbarrier.arrive.shared::cta.b64 _, [%0];\n" ::"r"(bar) : "memory");
-  const bool ok = __all_sync(0xffffffffu, mbar_wait(bar, 0u));
-  if (lane == 0) *flag = ok ? 0 : 1;
-}
-
-cudaError_t launch_wait_selftest(int never_complete, int32_t *flag, cudaStream_t stream) {
-  k_wait_selftest<<<1, 32, 0, stream>>>(never_complete, flag);
-  return cudaGetLastError();
-}
-
-// [precision: BF16x3, TF32x2][0: the small-block instance, 1: the large-block one]
-static const void *const (&pipe_instances())[2][2] {
-  static const void *const inst[2][2] = {
-      {(const void *)k_numeric_split_pipe<BSM_PREC_SPLIT_BF16X3, 2, false>,
-       (const void *)k_numeric_split_pipe<BSM_PREC_SPLIT_BF16X3, 2, true>},
-      {(const void *)k_numeric_split_pipe<BSM_PREC_SPLIT_TF32X2, 2, false>,
-       (const void *)k_numeric_split_pipe<BSM_PREC_SPLIT_TF32X2, 2, true>}};
-  return inst;
-}
-
 cudaError_t launch_numeric_split(int precision, int sizes, DevMat A, DevMat B, DevOut C,
                                  DevMat Cin, const void *a_left, const void *b_right, double alpha,
                                  double beta, DevWs ws, const DevStatus *st, const int32_t *items,
-                                 const int64_t *seg, int smax, int nsm, unsigned long long *work,
+                                 const int64_t *seg, int nsm, unsigned long long *work,
                                  cudaStream_t stream) {
-  const int pi = precision == BSM_PREC_SPLIT_BF16X3 ? 0 : 1;
-  const bool big = sizes == 2;  // C blocks beyond 16x16: the large-block instance
-  constexpr int stages = kPipeStages;
-  const int warps = big ? kPipeWarpsBig : kPipeWarps;
-  const size_t smem = (size_t)warps * pipe_warp_bytes(precision, smax, stages, big ? 32 : 16);
-  const void *fn = pipe_instances()[pi][big ? 1 : 0];
-  int per_sm = 1;
-  cudaError_t e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, fn, warps * 32, smem);
-  if (e != cudaSuccess) return e;
-  const int grid = nsm * (per_sm > 0 ? per_sm : 1);
-  const int sel = sizes;  // 0 all, 1 small C blocks only, 2 large ones only
-#define BSM_SPLIT_PIPE(P, G)                                                                    \
-  k_numeric_split_pipe<P, stages, G><<<grid, warps * 32, smem, stream>>>(                       \
-      A, B, C, Cin, a_left, b_right, alpha, beta, ws, st, items, seg, smax, sel, work)
-  if (precision == BSM_PREC_SPLIT_BF16X3) {
-    if (big) BSM_SPLIT_PIPE(BSM_PREC_SPLIT_BF16X3, true);
-    else BSM_SPLIT_PIPE(BSM_PREC_SPLIT_BF16X3, false);
-  } else {
-    if (big) BSM_SPLIT_PIPE(BSM_PREC_SPLIT_TF32X2, true);
-    else BSM_SPLIT_PIPE(BSM_PREC_SPLIT_TF32X2, false);
-  }
-#undef BSM_SPLIT_PIPE
+  const size_t smem = kSbWarps * sizeof(SbWarp);
+  const int grid = nsm * kSbBlocksPerSm;
+  const uint4 *l = static_cast<const uint4 *>(a_left), *r = static_cast<const uint4 *>(b_right);
+  if (precision == BSM_PREC_SPLIT_BF16X3)
+    k_numeric_split_blocks<BSM_PREC_SPLIT_BF16X3><<<grid, kSbWarps * 32, smem, stream>>>(
+        A, B, C, Cin, l, r, alpha, beta, ws, st, items, seg, sizes, work);
+  else
+    k_numeric_split_blocks<BSM_PREC_SPLIT_TF32X2><<<grid, kSbWarps * 32, smem, stream>>>(
+        A, B, C, Cin, l, r, alpha, beta, ws, st, items, seg, sizes, work);
   return cudaGetLastError();
 }
 
@@ -1124,19 +897,16 @@ cudaError_t numeric_split_init() {
       if (e != cudaSuccess) return e;
     }
   }
-  // the largest slot layout of each instance (k up to 32), and the whole
-  // shared memory of an SM for the carveout (the rings decide occupancy)
-  for (int pi = 0; pi < 2; pi++)
-    for (int big = 0; big < 2; big++) {
-      const int prec = pi == 0 ? BSM_PREC_SPLIT_BF16X3 : BSM_PREC_SPLIT_TF32X2;
-      const int bytes = big ? kPipeWarpsBig * pipe_warp_bytes(prec, 32, kPipeStages, 32)
-                            : kPipeWarps * pipe_warp_bytes(prec, 32, kPipeStages, 16);
-      const void *fn = pipe_instances()[pi][big];
-      cudaError_t e = cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, bytes);
-      if (e == cudaSuccess)
-        e = cudaFuncSetAttribute(fn, cudaFuncAttributePreferredSharedMemoryCarveout, 100);
-      if (e != cudaSuccess) return e;
-    }
+  // the per-block kernel's operands come through L1: no more shared memory than its own
+  for (const void *fn : {(const void *)k_numeric_split_blocks<BSM_PREC_SPLIT_BF16X3>,
+                         (const void *)k_numeric_split_blocks<BSM_PREC_SPLIT_TF32X2>}) {
+    cudaError_t e = cudaFuncSetAttribute(fn, cudaFuncAttributePreferredSharedMemoryCarveout,
+                                         kSbCarveout);
+    if (e == cudaSuccess)
+      e = cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                               (int)(kSbWarps * sizeof(SbWarp)));
+    if (e != cudaSuccess) return e;
+  }
   return cudaSuccess;
 }
 

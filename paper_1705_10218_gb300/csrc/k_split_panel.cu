@@ -1316,4 +1316,26 @@ cudaError_t numeric_split_panel_init() {
   return cudaSuccess;
 }
 
+// The kernel's bounded barrier wait on its own: lane 0 completes the phase (a plain
+// arrive), unless never_complete; the warp then waits as the kernel does and records
+// in *flag whether the wait gave up.
+__global__ void k_wait_selftest(int never_complete, int32_t *flag) {
+  __shared__ __align__(8) unsigned long long bar_storage;
+  const uint32_t bar = (uint32_t)__cvta_generic_to_shared(&bar_storage);
+  const int lane = threadIdx.x & 31;
+  if (lane == 0) {
+    pb_init(bar, 1);
+    asm volatile("fence.mbarrier_init.release.cluster;\n" ::: "memory");
+  }
+  __syncwarp();
+  if (lane == 0 && !never_complete) pb_arrive(bar);
+  const bool ok = __all_sync(0xffffffffu, pb_wait(bar, 0u));
+  if (lane == 0) *flag = ok ? 0 : 1;
+}
+
+cudaError_t launch_wait_selftest(int never_complete, int32_t *flag, cudaStream_t stream) {
+  k_wait_selftest<<<1, 32, 0, stream>>>(never_complete, flag);
+  return cudaGetLastError();
+}
+
 }  // namespace bsm
