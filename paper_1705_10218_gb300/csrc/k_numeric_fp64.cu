@@ -1219,9 +1219,16 @@ cudaError_t launch_numeric_fp64(int variant, DevMat A, DevMat B, DevOut C, DevMa
     case kFp64G8: {
       const int mr = max_m <= 4 ? 4 : max_m <= 6 ? 6 : 8;
       const int gs = max_n <= 4 ? 4 : max_n <= 6 ? 6 : 8;
-#define BSM_G8(R, G)                                                                           \
-  k_numeric_fp64_g8<R, G><<<grid, kG8Warps * 32, g8_smem_bytes(), stream>>>(                   \
-      A, B, C, Cin, alpha, beta, ws, st, items, seg, work)
+// the shared memory is opted into here, for the one instance (it loads its code)
+#define BSM_G8(R, G)                                                                             \
+  do {                                                                                           \
+    const cudaError_t e = cudaFuncSetAttribute(                                                  \
+        k_numeric_fp64_g8<R, G>, cudaFuncAttributeMaxDynamicSharedMemorySize,                    \
+        (int)g8_smem_bytes());                                                                   \
+    if (e != cudaSuccess) return e;                                                              \
+    k_numeric_fp64_g8<R, G><<<grid, kG8Warps * 32, g8_smem_bytes(), stream>>>(                   \
+        A, B, C, Cin, alpha, beta, ws, st, items, seg, work);                                    \
+  } while (0)
       if (mr == 4) {
         if (gs == 4) BSM_G8(4, 4); else if (gs == 6) BSM_G8(4, 6); else BSM_G8(4, 8);
       } else if (mr == 6) {
@@ -1273,15 +1280,6 @@ cudaError_t numeric_fp64_init() {
   if (e != cudaSuccess) return e;
   // its operands come through L1: no more shared memory than its own
   e = cudaFuncSetAttribute(k_numeric_fp64_dg, cudaFuncAttributePreferredSharedMemoryCarveout, 50);
-  if (e != cudaSuccess) return e;
-#define BSM_G8(R, G)                                                                      \
-  if (e == cudaSuccess)                                                                   \
-  e = cudaFuncSetAttribute(k_numeric_fp64_g8<R, G>, cudaFuncAttributeMaxDynamicSharedMemorySize, \
-                           (int)g8_smem_bytes())
-  BSM_G8(4, 4); BSM_G8(4, 6); BSM_G8(4, 8);
-  BSM_G8(6, 4); BSM_G8(6, 6); BSM_G8(6, 8);
-  BSM_G8(8, 4); BSM_G8(8, 6); BSM_G8(8, 8);
-#undef BSM_G8
   if (e != cudaSuccess) return e;
   e = cudaFuncSetAttribute(k_numeric_fp64_pk<12>, cudaFuncAttributeMaxDynamicSharedMemorySize,
                            (int)pk_smem_bytes());
