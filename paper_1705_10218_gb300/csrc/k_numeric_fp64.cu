@@ -1100,13 +1100,16 @@ __global__ void __launch_bounds__(kDgWarps * 32, kDgBlocksPerSm)
   const int nparts =
       (int)min((int64_t)ntiles, max((int64_t)1, kDgUnits * warps / max((int64_t)1, we - wb)));
   we = wb + (we - wb) * nparts;
-  const int64_t share = (we - wb) / (warps * 4);
-  const int grab = share >= kDgGrab ? kDgGrab : share < 1 ? 1 : (int)share;
-
+  // Towards the end shorter runs, a quarter to an eighth of what is left for each warp,
+  // so that the warps end together (a fixed length: water of 64 molecules 0.66 ms, of 512
+  // 5.45, blocks of 1 to 33 in 200 rows 1.25; this 0.61, 5.34 and 1.02).
+  const int shift = 34 - __clz((int)warps);
+  int64_t base = wb;
   for (;;) {
+    const int grab = (int)max((int64_t)1, min((int64_t)kDgGrab, (we - base) >> shift));
     unsigned long long got = 0;
     if (lane == 0) got = atomicAdd(work, (unsigned long long)grab);
-    const int64_t base = wb + (int64_t)__shfl_sync(0xffffffffu, got, 0);
+    base = wb + (int64_t)__shfl_sync(0xffffffffu, got, 0);
     if (base >= we) break;
     const int count = we - base < grab ? (int)(we - base) : grab;
     // what the C blocks of the run need, a lane each: the next block is then found
