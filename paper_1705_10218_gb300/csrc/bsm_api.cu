@@ -888,7 +888,7 @@ static int launch_numeric(Launch &L, int variant, const int32_t *items, const in
         CK(cudaMemsetAsync(ctx->d_work, 0, sizeof(unsigned long long), L.s));
         CK(launch_numeric_split(L.o.precision, 2, L.dA, L.dB, L.out, L.dC, L.A->split_left,
                                 L.B->split_right, L.alpha, L.beta, L.ws, ctx->d_status, items,
-                                seg, ctx->nsm, ctx->d_work, L.s));
+                                seg, max_m, max_n, ctx->nsm, ctx->d_work, L.s));
       }
       ctx->launches++;
       return BSM_OK;
@@ -897,7 +897,7 @@ static int launch_numeric(Launch &L, int variant, const int32_t *items, const in
     CK(cudaMemsetAsync(ctx->d_work, 0, sizeof(unsigned long long), L.s));
     CK(launch_numeric_split(L.o.precision, 0, L.dA, L.dB, L.out, L.dC, L.A->split_left,
                             L.B->split_right, L.alpha, L.beta, L.ws, ctx->d_status, items, seg,
-                            ctx->nsm, ctx->d_work, L.s));
+                            max_m, max_n, ctx->nsm, ctx->d_work, L.s));
   } else {
     if (fp64_variant_uses_work(variant))
       CK(cudaMemsetAsync(ctx->d_work, 0, sizeof(unsigned long long), L.s));

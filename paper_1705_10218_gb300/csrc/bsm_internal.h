@@ -240,8 +240,8 @@ cudaError_t launch_numeric_split_cat(int precision, DevMat A, DevMat B, DevOut C
 cudaError_t launch_numeric_split(int precision, int sizes, DevMat A, DevMat B, DevOut C,
                                  DevMat Cin, const void *a_left, const void *b_right, double alpha,
                                  double beta, DevWs ws, const DevStatus *st, const int32_t *items,
-                                 const int64_t *seg, int nsm, unsigned long long *work,
-                                 cudaStream_t stream);
+                                 const int64_t *seg, int max_m, int max_n, int nsm,
+                                 unsigned long long *work, cudaStream_t stream);
 // The row-panel split kernel (k_split_panel.cu). Its work of a multiply:
 //   tiles:  per C block row, its tiles (runs of whole C blocks, at most 128
 //           columns and 32 blocks) as 64-byte entries at the row's first C

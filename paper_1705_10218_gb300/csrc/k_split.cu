@@ -270,13 +270,16 @@ constexpr int kSbBlocksPerSm = 2;
 constexpr int kSbStage = 512;    // values gathered at most
 constexpr int kSbCarveout = 60;  // % of an SM's L1 as shared memory: what two blocks need
 constexpr int kSbGrab = 8;  // C blocks a warp takes at a time, at most
+// Units of work per warp up to which C blocks are split into parts of their tiles (32 x 32
+// blocks of 32, BF16x3: 0.151 ms with whole blocks, 0.086 with parts; 8 units gain no more).
+constexpr int kSbUnits = 4;
 
 __device__ const uint4 g_zero_pieces[32] = {};  // a piece of zeros for each row
 
 struct SbItem {  // a C block of a warp's run
   const int2 *prods;
   int64_t coff, cin;  // cin: offset of its C_in block, or -1
-  int32_t np, m, n;
+  int32_t np, m, n, part;  // part: every nparts-th tile from this one on
 };
 struct SbPiece {  // a piece of k: where row 0's lies in both operands' first planes, and
   const uint4 *a, *b;  // the distance of the planes in rows
@@ -438,7 +441,7 @@ __global__ void __launch_bounds__(kSbWarps * 32, kSbBlocksPerSm)
                            const uint4 *__restrict__ a_left, const uint4 *__restrict__ b_right,
                            double alpha, double beta, DevWs ws, const DevStatus *st,
                            const int32_t *__restrict__ items, const int64_t *__restrict__ seg,
-                           int sel, unsigned long long *work) {
+                           int sel, int ntiles, unsigned long long *work) {
   if (st->overflow) return;
   constexpr bool BF = (PREC == BSM_PREC_SPLIT_BF16X3);
   constexpr int VPP = BF ? 8 : 4;
@@ -451,7 +454,12 @@ __global__ void __launch_bounds__(kSbWarps * 32, kSbBlocksPerSm)
   double *hout = (C.host_vals && st->nnz_c <= C.host_cap) ? C.host_vals : nullptr;
   const bool plain = (alpha == 1.0 && beta == 0.0);
   // fewer at a time where that would leave warps without work
-  const int64_t share = (we - wb) / ((int64_t)gridDim.x * kSbWarps * 4);
+  const int64_t warps = (int64_t)gridDim.x * kSbWarps;
+  // the parts of a C block, a unit of work each
+  const int nparts =
+      (int)min((int64_t)ntiles, max((int64_t)1, kSbUnits * warps / max((int64_t)1, we - wb)));
+  we = wb + (we - wb) * nparts;
+  const int64_t share = (we - wb) / (warps * 4);
   const int grab = share >= kSbGrab ? kSbGrab : share < 1 ? 1 : (int)share;
 
   for (;;) {
@@ -461,8 +469,10 @@ __global__ void __launch_bounds__(kSbWarps * 32, kSbBlocksPerSm)
     if (base >= we) break;
     const int count = we - base < grab ? (int)(we - base) : grab;
     if (lane < count) {
-      const int64_t gb = items ? items[base + lane] : base + lane;
+      const int64_t unit = base + lane - wb, blk = nparts > 1 ? wb + unit / nparts : base + lane;
+      const int64_t gb = items ? items[blk] : blk;
       SbItem it;
+      it.part = nparts > 1 ? (int)(unit % nparts) : 0;
       const int64_t p0 = ws.prod_ptr[gb];
       it.prods = ws.prods + p0;
       it.np = (int)(ws.prod_ptr[gb + 1] - p0);
@@ -516,13 +526,15 @@ __global__ void __launch_bounds__(kSbWarps * 32, kSbBlocksPerSm)
         operands();
         continue;
       }
-      const bool staged = m * n <= kSbStage;
+      const bool staged = nparts == 1 && m * n <= kSbStage;
+      int number = 0;
       if (held > 0 && (!staged || held + m * n > kSbStage || it.coff != first + held)) flush();
       if (held == 0) first = it.coff;
       // the orientation with fewer MMA tiles
       const bool swap = ((n + 15) >> 4) * ((m + 7) >> 3) < ((m + 15) >> 4) * ((n + 7) >> 3);
       for (int m0 = 0; m0 < m; m0 += 16)
         for (int n0 = 0; n0 < n; n0 += 16) {
+          if (nparts > 1 && number++ % nparts != it.part) continue;
           const int tm = min(16, m - m0), tn = min(16, n - n0);
           const int l0 = swap ? n0 : m0, tl = swap ? tn : tm, r0 = swap ? m0 : n0, tr = swap ? tm : tn;
           if (tr > 8)
@@ -531,7 +543,6 @@ __global__ void __launch_bounds__(kSbWarps * 32, kSbBlocksPerSm)
             sb_tile<PREC, kOne>(w, ca, cb, cp, it, l0, tl, r0, tr, swap, A, B, a_left, b_right, lane);
           else
             sb_tile<PREC, kHalf>(w, ca, cb, cp, it, l0, tl, r0, tr, swap, A, B, a_left, b_right, lane);
-          if (m0 + 16 >= m && n0 + 16 >= n) operands();
           const double *cinv = it.cin >= 0 ? Cin.vals + it.cin : nullptr;
           const int dc = 32 / tm, dr = 32 - dc * tm;
           int c = lane / tm, r = lane - c * tm;
@@ -555,6 +566,7 @@ __global__ void __launch_bounds__(kSbWarps * 32, kSbBlocksPerSm)
           }
           __syncwarp();
         }
+      operands();
       if (staged) held += m * n;
     }
     if (held > 0) flush();
@@ -824,17 +836,18 @@ __global__ void __launch_bounds__(kCatWarps * 32)
 cudaError_t launch_numeric_split(int precision, int sizes, DevMat A, DevMat B, DevOut C,
                                  DevMat Cin, const void *a_left, const void *b_right, double alpha,
                                  double beta, DevWs ws, const DevStatus *st, const int32_t *items,
-                                 const int64_t *seg, int nsm, unsigned long long *work,
-                                 cudaStream_t stream) {
+                                 const int64_t *seg, int max_m, int max_n, int nsm,
+                                 unsigned long long *work, cudaStream_t stream) {
+  const int ntiles = ((max_m + 15) / 16) * ((max_n + 15) / 16);
   const size_t smem = kSbWarps * sizeof(SbWarp);
   const int grid = nsm * kSbBlocksPerSm;
   const uint4 *l = static_cast<const uint4 *>(a_left), *r = static_cast<const uint4 *>(b_right);
   if (precision == BSM_PREC_SPLIT_BF16X3)
     k_numeric_split_blocks<BSM_PREC_SPLIT_BF16X3><<<grid, kSbWarps * 32, smem, stream>>>(
-        A, B, C, Cin, l, r, alpha, beta, ws, st, items, seg, sizes, work);
+        A, B, C, Cin, l, r, alpha, beta, ws, st, items, seg, sizes, ntiles, work);
   else
     k_numeric_split_blocks<BSM_PREC_SPLIT_TF32X2><<<grid, kSbWarps * 32, smem, stream>>>(
-        A, B, C, Cin, l, r, alpha, beta, ws, st, items, seg, sizes, work);
+        A, B, C, Cin, l, r, alpha, beta, ws, st, items, seg, sizes, ntiles, work);
   return cudaGetLastError();
 }
 
