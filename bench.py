@@ -55,6 +55,9 @@ FP64_KERNELS = {"t16b2": (0, "k_numeric_fp64_t16"), "t16b3": (1, "k_numeric_fp64
                 "t32": (2, "k_numeric_fp64_t32"), "pk12": (3, "k_numeric_fp64_pk"),
                 "pk16": (4, "k_numeric_fp64_pk"), "g8": (5, "k_numeric_fp64_g8")}
 FP64_BY_NUMBER = {v[0]: k for k, v in FP64_KERNELS.items()}
+# The default FP64 multiply is reported as pk12 and runs as its form on the tensor
+# cores: 43 products of FP16 digit pairs for one FP64 product.
+DIGIT_KERNEL, DIGIT_PAIRS = "k_numeric_fp64_dg", 43
 # DRAM bytes (read + write) per launch of a kernel, from one ncu capture
 # (dram__bytes_read.sum + dram__bytes_write.sum, profiles/): valid only while
 # the code that decides it is unchanged -- the kernel's own source section and,
@@ -65,14 +68,14 @@ MEASURED_TRAFFIC = {
     ("pk12", "water2048"): dict(
         sections=[("paper_1705_10218_gb300/csrc/k_numeric_fp64.cu",
                    ("// pk\n", "cudaError_t launch_numeric_fp64("),
-                   "7bbcdcfe0e18d9a1b4f6759ea308f217cc9b13f32aaa2edbd5433183548b5194"),
+                   "d2f677421bba82e40c8a281c2384355575f55598d2d185672d3a3d378381dd67"),
                   ("paper_1705_10218_gb300/csrc/k_classes.cu",
                    ("// Work in a row order.", "}  // namespace bsm"),
                    "b173af39936271e55c6a2623c0b1222afaca8a97ab34ff8f9a0ec78e9ecdf01b"),
                   ("paper_1705_10218_gb300/csrc/bsm_api.cu",
                    ("static void bfs_row_order(", "static uint64_t next_order_id("),
                    "113dd9175f43cb3ea209f7d880be5023dd9fd7acdf547fa5077ea74319814288")],
-        bytes=2.983e9 + 1.559e9),
+        bytes=6.80e9 + 1.68e9),
 }
 
 
@@ -859,10 +862,13 @@ def main():
     # replay the phases are not timed separately: the whole multiply is used.
     if prof.multiplies > 0:
         num_ms = prof.ms_numeric / prof.multiplies
-        kname = (FP64_KERNELS[FP64_BY_NUMBER[prof.last_fp64_kernel]][1] if args.precision == "fp64"
+        digits = args.precision == "fp64" and fk is None and FP64_BY_NUMBER[prof.last_fp64_kernel] == "pk12"
+        kname = (DIGIT_KERNEL if digits else
+                 FP64_KERNELS[FP64_BY_NUMBER[prof.last_fp64_kernel]][1] if args.precision == "fp64"
                  else SPLIT_KERNEL_SYMBOLS.get(prof.last_split_kernel, "k_numeric_split_blocks"))
     else:
         num_ms = total_ms / args.steps
+        digits = False
         kname = "whole multiply (CUDA graph replay)"
     phase = {"norms": round(prof.ms_norms / max(prof.multiplies, 1), 4),
              "symbolic": round(prof.ms_symbolic / max(prof.multiplies, 1), 4),
@@ -887,6 +893,12 @@ def main():
                 "kernel": kname, "peak_source": fp64_src,
                 "algorithmic": "2*m*n*k over kept products per launch", "phase_ms": phase,
                 "phase_rates": phase_rates}
+        if digits:  # on the tensor cores: against their measured rate
+            peak, src = measured_peak("bf16_tflops", 1900.0)
+            roof.update(bound="tensor", achieved=round(DIGIT_PAIRS * achieved / 1e3, 2), peak=peak,
+                        unit="TFLOP/s", frac=round(DIGIT_PAIRS * achieved / 1e3 / peak, 4), peak_source=src,
+                        algorithmic=f"{DIGIT_PAIRS} FP16 digit pairs x 2*m*n*k over kept products per launch",
+                        fp64_gflops=round(achieved, 2), fp64_pipe_peak_gflops=round(fp64_peak, 1))
     else:
         # compulsory bytes of the numeric kernel: C written once (FP64) and the
         # operand slices read once (A = B: left and right layouts)

@@ -300,10 +300,12 @@ __global__ void __launch_bounds__(kSWarps * 32, MINB)
 // at 25 GB/s of its 193.
 // Measured, 20000 atoms, 2.2 M C blocks of 6, numeric phase with a second
 // destination in host memory: 26.1 -> 3.40 ms, bound by the link (637 MB); without
-// one 1.40 -> 1.37, bound by the FP64 pipe (0.68 without its instructions): the
+// one 1.40 -> 1.33, bound by the FP64 pipe (0.68 without its instructions): the
 // multiplication by alpha, on the few lanes of one group at a time, moved to the
-// stores, where it is on all lanes. 16 warps per SM with runs of 30 blocks: 24 warps
-// with runs of 15 took 0.15 ms more, 32 0.5 (the groups idle at a run's end).
+// stores, where it is on all lanes and not there for alpha = 1 (another alpha: 1.40 ->
+// 1.48; as exponent arithmetic for powers of two no less). 16 warps per SM with runs of
+// 30 blocks: 24 warps with runs of 15 took 0.15 ms more, 32 0.5 (the groups idle at a
+// run's end).
 // A C block of more than MR rows or GS columns (only when the kernel is forced on
 // larger blocks) is done in column and row chunks by its group and stored directly.
 // ----------------------------------------------------------------------------
@@ -451,12 +453,16 @@ __global__ void __launch_bounds__(kG8Warps * 32, kG8BlocksPerSm)
             p++;
           }
           if (p >= it.np && cl < it.n) {  // the block is complete
+            double *to = stage + it.at + cl * it.m;
+            if (late) {
 #pragma unroll
-            for (int r = 0; r < MR; r++)
-              if (r < it.m) {
-                const int loc = cl * it.m + r;
-                stage[it.at + loc] = late ? acc[r] : value(cinv, r, loc);
-              }
+              for (int r = 0; r < MR; r++)
+                if (r < it.m) to[r] = acc[r];
+            } else {
+#pragma unroll
+              for (int r = 0; r < MR; r++)
+                if (r < it.m) to[r] = value(cinv, r, cl * it.m + r);
+            }
           }
         }
       }
@@ -472,6 +478,11 @@ __global__ void __launch_bounds__(kG8Warps * 32, kG8BlocksPerSm)
       taken += __popc(heads);
     }
     __syncwarp();
+    if (late && alpha != 1.0) {  // a loop of its own: no FP64 instruction without it
+      const int all = __shfl_sync(0xffffffffu, own.at + mn, count - 1);
+      for (int e = lane; e < all; e += 32) stage[e] *= alpha;
+      __syncwarp();
+    }
     while (gather && starts) {  // blocks x to y - 1, which follow one another in C
       const int x = __ffs(starts) - 1;
       starts &= starts - 1;
@@ -482,8 +493,7 @@ __global__ void __launch_bounds__(kG8Warps * 32, kG8BlocksPerSm)
       // from the start of the 128-byte line that they begin in
       for (int e = lane - (int)(first & 15); e < total; e += 32)
         if (e >= 0) {
-          double v = stage[at + e];
-          if (late && alpha != 1.0) v *= alpha;
+          const double v = stage[at + e];
           __stcs(C.vals + first + e, v);
           if (hout) __stcs(hout + first + e, v);
         }

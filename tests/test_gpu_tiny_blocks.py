@@ -38,3 +38,30 @@ def test_g8_runs_and_host_copy(gpu_ctx, bsm_lib, top, alpha, with_c, launch):
     assert np.array_equal(host[:len(got)], got)
     for M in (dA, dB, dC):
         M.destroy()
+
+
+@pytest.mark.parametrize("alpha", [-1.0, 2.0 ** -520, -2.0 ** 40, 1.7, -0.0])
+def test_g8_alpha(gpu_ctx, bsm_lib, alpha):
+    """alpha at the stores (with results that are denormal, zeros, infinities and values
+    that are not numbers): the bits are those of a multiplication of the sums."""
+    rng = np.random.default_rng(9)
+    rs = rng.choice([1, 3, 5], 30)
+    A = synth.random_blocks(rng, rs, rs, 0.4, kind="normal")
+    off = H.block_list_offsets(A)
+    for b in range(0, len(A.blk_row), 5):
+        A.values[off[b]:off[b + 1]] *= 2.0 ** -260
+    A.values[off[7]] = np.inf
+    A.values[off[9]] = np.nan
+    A.values[off[11]:off[12]] = 0.0
+    out = []
+    dA = gpu_ctx.from_blocks(A)
+    for a in (1.0, alpha):
+        dC = gpu_ctx.empty(A.row_sizes, A.col_sizes)
+        gpu_ctx.multiply(a, dA, dA, 0.0, dC, 0.0, fp64_kernel=bsm_lib.BSM_FP64_G8, blocking=True)
+        out.append(dC.values())
+        dC.destroy()
+    dA.destroy()
+    with np.errstate(all="ignore"):
+        want = out[0] * alpha
+    assert np.array_equal(out[1], want, equal_nan=True)
+    assert np.array_equal(np.signbit(out[1])[~np.isnan(want)], np.signbit(want)[~np.isnan(want)])
