@@ -1428,8 +1428,8 @@ int bsm_ctx_create(int device, bsm_ctx *out) {
   }
   if (rc == BSM_OK) {
     rc = dev_alloc(&ctx->cls_counts, kMaxClasses);
-    if (rc == BSM_OK) rc = dev_alloc(&ctx->dg.range, 2);
-    if (rc == BSM_OK) rc = dev_alloc(&ctx->d_ticket, 1);
+    if (rc == BSM_OK) rc = dev_alloc(&ctx->dg.range, 3);  // and the ticket
+    ctx->d_ticket = reinterpret_cast<int32_t *>(ctx->dg.range + 2);
     if (rc == BSM_OK && (e = cudaMemsetAsync(ctx->d_ticket, 0, sizeof(int32_t), ctx->stream)) != cudaSuccess)
       rc = cuda_fail(e, "cudaMemset");
     if (rc == BSM_OK) rc = dev_alloc(&ctx->cls_cursor, kMaxClasses);
@@ -1494,7 +1494,6 @@ int bsm_ctx_destroy(bsm_ctx ctx) {
   dev_free(ctx->cls_items);
   dev_free(ctx->ord_start);
   dev_free(ctx->d_pk_tab);
-  dev_free(ctx->d_ticket);
   dev_free(ctx->dg.range);
   for (DigitSide *d : {&ctx->dg.a, &ctx->dg.b}) {
     dev_free(d->units);
@@ -1870,10 +1869,8 @@ int bsm_mat_create(bsm_ctx ctx, int32_t nbrows, const int32_t *row_sizes, int32_
   };
   // first scalar row / column of each block row / column (32-bit: the digit
   // kernel, their only reader, takes matrices of less than 2^31 of them)
-  std::vector<int32_t> h_row_first, h_col_first;
-  auto firsts = [](const std::vector<int32_t> &sizes, std::vector<int32_t> &first) {
+  auto firsts = [](const std::vector<int32_t> &sizes, int32_t *first) {
     int64_t at = 0;
-    first.resize(sizes.size() + 1);
     for (size_t i = 0; i < sizes.size(); i++) first[i] = (int32_t)at, at += sizes[i];
     first[sizes.size()] = (int32_t)at;
     return at;
@@ -1885,24 +1882,26 @@ int bsm_mat_create(bsm_ctx ctx, int32_t nbrows, const int32_t *row_sizes, int32_
   };
   M->digit_rate[0] = most(M->h_col_sizes);
   M->digit_rate[1] = most(M->h_row_sizes);
-  M->scalar_rows = firsts(M->h_row_sizes, h_row_first);
-  M->scalar_cols = firsts(M->h_col_sizes, h_col_first);
-  if ((rc = dev_alloc(&M->row_sizes, nbrows)) || (rc = dev_alloc(&M->col_sizes, nbcols)) ||
-      (rc = dev_alloc(&M->row_cls, nbrows)) || (rc = dev_alloc(&M->col_cls, nbcols)) ||
-      (rc = dev_alloc(&M->row_first, nbrows + 1)) || (rc = dev_alloc(&M->col_first, nbcols + 1)))
-    return fail(rc);
-  cudaStream_t s = ctx->stream;
-  auto cp = [&](void *dst, const void *src, size_t bytes) -> cudaError_t {
-    return bytes ? cudaMemcpyAsync(dst, src, bytes, cudaMemcpyHostToDevice, s) : cudaSuccess;
-  };
-  cudaError_t e;
-  if ((e = cp(M->row_sizes, row_sizes, (size_t)nbrows * 4)) != cudaSuccess ||
-      (e = cp(M->col_sizes, col_sizes, (size_t)nbcols * 4)) != cudaSuccess ||
-      (e = cp(M->row_cls, h_row_cls.data(), (size_t)nbrows * 4)) != cudaSuccess ||
-      (e = cp(M->col_cls, h_col_cls.data(), (size_t)nbcols * 4)) != cudaSuccess ||
-      (e = cp(M->row_first, h_row_first.data(), ((size_t)nbrows + 1) * 4)) != cudaSuccess ||
-      (e = cp(M->col_first, h_col_first.data(), ((size_t)nbcols + 1) * 4)) != cudaSuccess)
-    return fail(cuda_fail(e, "bsm_mat_create copy"));
+  // sizes, kinds and first scalars of the block rows, then of the block columns: one
+  // buffer and one copy (each costs a matrix as much as its launches)
+  const size_t nr = (size_t)nbrows, nc = (size_t)nbcols;
+  std::vector<int32_t> h(3 * nr + 3 * nc + 2);
+  std::copy(M->h_row_sizes.begin(), M->h_row_sizes.end(), h.begin());
+  std::copy(h_row_cls.begin(), h_row_cls.end(), h.begin() + nr);
+  M->scalar_rows = firsts(M->h_row_sizes, h.data() + 2 * nr);
+  int32_t *hc = h.data() + 3 * nr + 1;
+  std::copy(M->h_col_sizes.begin(), M->h_col_sizes.end(), hc);
+  std::copy(h_col_cls.begin(), h_col_cls.end(), hc + nc);
+  M->scalar_cols = firsts(M->h_col_sizes, hc + 2 * nc);
+  if ((rc = dev_alloc(&M->row_sizes, (int64_t)h.size()))) return fail(rc);
+  M->row_cls = M->row_sizes + nr;
+  M->row_first = M->row_sizes + 2 * nr;
+  M->col_sizes = M->row_sizes + 3 * nr + 1;
+  M->col_cls = M->col_sizes + nc;
+  M->col_first = M->col_sizes + 2 * nc;
+  const cudaError_t e = cudaMemcpyAsync(M->row_sizes, h.data(), h.size() * sizeof(int32_t),
+                                        cudaMemcpyHostToDevice, ctx->stream);
+  if (e != cudaSuccess) return fail(cuda_fail(e, "bsm_mat_create copy"));
   if ((rc = upload_contents(M, nblocks, blk_row, blk_col, values, true))) return fail(rc);
   *out = M;
   return BSM_OK;
@@ -1949,12 +1948,7 @@ int bsm_mat_destroy(bsm_mat m) {
   m->back.release();
   cache_free(m->split_left);
   cache_free(m->split_right);
-  dev_free(m->row_sizes);
-  dev_free(m->col_sizes);
-  dev_free(m->row_cls);
-  dev_free(m->col_cls);
-  dev_free(m->row_first);
-  dev_free(m->col_first);
+  dev_free(m->row_sizes);  // and the other arrays of block rows and columns, behind it
   dev_free(m->row_order);
   if (m->ev_use) cudaEventDestroy(m->ev_use);
   // captured multiplies may name this matrix's buffers
