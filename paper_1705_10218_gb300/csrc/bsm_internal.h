@@ -109,7 +109,13 @@ struct DevStatus {
 constexpr int kDigits = 8;
 constexpr int kDigitZeros = 64;
 constexpr uint32_t kDigitOutside = 1u << 31;
-constexpr int kDigitRange = 11;
+// How far a row may lie below its block's class. Wider keeps more C blocks on the tensor
+// cores and fewer bits of such a row; at 12 the error of every element against the sum of
+// its absolute products is no larger than at 9, 10 or 11 (where FP64 FMAs take more C blocks)
+// on blocks of 1 to 33, sign iterates, water and amorphous systems, and below the FP64
+// kernel's: sign iterates 0.4, 2.2 and 0.8e-15, 2.4, 3.0 and 4.4e-15 there. Two sign iterations
+// of 192 water molecules: 18.6 ms at 9, 15.3 at 11, 14.4 at 12, 13 and 15.
+constexpr int kDigitRange = 12;
 constexpr int kDigitMaxRows = 128;
 constexpr int kDigitMaxOctets = 0xFFFF;
 constexpr int kDigitMaxClass = 60;
