@@ -859,7 +859,7 @@ static int stage_a(Launch &L, bool record) {
   // with few rows the count pass's last thread block does the scan
   const bool fused = L.A->nbr <= kFusedScanRows;
   CK(launch_symbolic_count(L.dA, L.dB, L.dC, L.use_cin ? 1 : 0, L.eps, L.ws, L.out, ctx->d_status,
-                           fused ? ctx->d_ticket : nullptr, ctx->nsm * 6, L.s));
+                           fused ? ctx->d_ticket : nullptr, ctx->nsm, L.s));
   ctx->launches++;
   if (!fused) {
     CK(launch_symbolic_scan(L.A->nbr, L.ws, L.out, ctx->d_status, L.s));

@@ -11,7 +11,6 @@ namespace bsm {
 
 // Block columns handled per pass of the per-row bitmap in the symbolic phase.
 constexpr int kWindowCols = 65536;
-constexpr int kSymThreads = 256;
 // Largest output tile one warp accumulates in registers (32 x 32 scalars).
 constexpr int kTile = 32;
 
@@ -154,7 +153,7 @@ cudaError_t launch_block_norms_scales(const int32_t *row_sizes, const int32_t *c
 // where the scan's own thread block would take as long as its launch).
 constexpr int32_t kFusedScanRows = 2048;
 cudaError_t launch_symbolic_count(DevMat A, DevMat B, DevMat Cin, int use_cin, double eps,
-                                  DevWs ws, DevOut C, DevStatus *st, int32_t *ticket, int grid,
+                                  DevWs ws, DevOut C, DevStatus *st, int32_t *ticket, int nsm,
                                   cudaStream_t stream);
 
 cudaError_t launch_symbolic_scan(int32_t nbr, DevWs ws, DevOut C, DevStatus *st,

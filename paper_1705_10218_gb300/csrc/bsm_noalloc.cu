@@ -295,7 +295,7 @@ extern "C" int bsm_multiply_noalloc(double alpha, const bsm_dev_csr *A, const bs
                                      B->values, hdr_b, norms_b, normsf_b, nullptr, nullptr, nullptr,
                                      nullptr, nsm, s)) != cudaSuccess)
     return noalloc_cuda_fail(e);
-  if ((e = launch_symbolic_count(dA, dB, none, 0, eps, ws, out, st, nullptr, nsm * 6, s)) != cudaSuccess)
+  if ((e = launch_symbolic_count(dA, dB, none, 0, eps, ws, out, st, nullptr, nsm, s)) != cudaSuccess)
     return noalloc_cuda_fail(e);
   if ((e = launch_symbolic_scan(A->nbr, ws, out, st, s)) != cudaSuccess)
     return noalloc_cuda_fail(e);

@@ -397,10 +397,10 @@ __device__ void symbolic_scan(int32_t nbr, const DevWs &ws, const DevOut &C, Dev
 // ----------------------------------------------------------------------------
 // Count pass: one thread block per C block row (grid-stride).
 // ----------------------------------------------------------------------------
-__global__ void __launch_bounds__(kSymThreads) k_symbolic_count(DevMat A, DevMat B, DevMat Cin,
-                                                                int use_cin, double eps,
-                                                                DevWs ws, DevOut C, DevStatus *st,
-                                                                int32_t *ticket) {
+template <int THREADS>
+__global__ void __launch_bounds__(THREADS)
+    k_symbolic_count(DevMat A, DevMat B, DevMat Cin, int use_cin, double eps, DevWs ws, DevOut C,
+                     DevStatus *st, int32_t *ticket) {
   extern __shared__ uint32_t smem_bits[];
   const int nbc = B.nbc;
   const bool whole = nbc <= kWindowCols;
@@ -449,13 +449,24 @@ __global__ void __launch_bounds__(kSymThreads) k_symbolic_count(DevMat A, DevMat
   }
 }
 
+// Threads of a thread block, which takes a row at a time: a row is a chain of loads for
+// every warp, so few rows (up to three per SM) get 16 warps each, more rows 8 and twice the
+// thread blocks per SM. Count and fill with digits, 96 rows 78 -> 60 us, 192 rows 113 -> 91,
+// 64 rows of 64 blocks of 32 106 -> 85; 32 warps a row 93 and 89 for the last two.
+static int sym_threads(int nbr, int nsm) { return nbr <= 3 * nsm ? 512 : 256; }
+
 cudaError_t launch_symbolic_count(DevMat A, DevMat B, DevMat Cin, int use_cin, double eps,
-                                  DevWs ws, DevOut C, DevStatus *st, int32_t *ticket, int grid,
+                                  DevWs ws, DevOut C, DevStatus *st, int32_t *ticket, int nsm,
                                   cudaStream_t stream) {
   const int nwords = (min(B.nbc, kWindowCols) + 31) / 32;
   const size_t smem = (size_t)max(nwords, 1) * sizeof(uint32_t);
+  const int threads = sym_threads(A.nbr, nsm);
+  int grid = nsm * 6;
   if (ticket) grid = min(grid, max(A.nbr, 1));  // fewer to wait for
-  k_symbolic_count<<<grid, kSymThreads, smem, stream>>>(A, B, Cin, use_cin, eps, ws, C, st, ticket);
+  if (threads == 512)
+    k_symbolic_count<512><<<grid, 512, smem, stream>>>(A, B, Cin, use_cin, eps, ws, C, st, ticket);
+  else
+    k_symbolic_count<256><<<grid, 256, smem, stream>>>(A, B, Cin, use_cin, eps, ws, C, st, ticket);
   return cudaGetLastError();
 }
 
@@ -504,10 +515,10 @@ __device__ __forceinline__ int bit_rank(const uint32_t *bitmap, const int32_t *w
 // ----------------------------------------------------------------------------
 // Fill pass: one thread block per C block row (grid-stride).
 // ----------------------------------------------------------------------------
-__global__ void __launch_bounds__(kSymThreads) k_symbolic_fill(DevMat A, DevMat B, DevMat Cin,
-                                                               int use_cin, double eps, DevWs ws,
-                                                               DevOut C, const DevStatus *st,
-                                                               int mask_words, Digits dg) {
+template <int THREADS>
+__global__ void __launch_bounds__(THREADS)
+    k_symbolic_fill(DevMat A, DevMat B, DevMat Cin, int use_cin, double eps, DevWs ws, DevOut C,
+                    const DevStatus *st, int mask_words, Digits dg) {
   if (st->overflow) return;
   extern __shared__ uint32_t smem_bits[];
   const int nbc = B.nbc;
@@ -728,7 +739,11 @@ __global__ void __launch_bounds__(kSymThreads) k_symbolic_fill(DevMat A, DevMat 
     __syncthreads();
     int32_t *seg = reinterpret_cast<int32_t *>(smem_bits) + warp * kDigitMaxRows;
     const bool same = A.vals == B.vals;
-    const int64_t w0 = (int64_t)blockIdx.x * nwarps + warp, nw = (int64_t)gridDim.x * nwarps;
+    // few rows: from the last thread block on, which has none, and one block of each, so
+    // that few blocks are on as many SMs; else consecutive blocks in a thread block
+    const int64_t w0 = THREADS == 512 ? (int64_t)warp * gridDim.x + (gridDim.x - 1 - blockIdx.x)
+                                      : (int64_t)blockIdx.x * nwarps + warp;
+    const int64_t nw = (int64_t)gridDim.x * nwarps;
     digits_of(A, &dg.a, same ? &dg.b : nullptr, seg, w0, nw, lane);
     if (!same) digits_of(B, nullptr, &dg.b, seg, w0, nw, lane);
   }
@@ -740,16 +755,17 @@ cudaError_t launch_symbolic_fill(DevMat A, DevMat B, DevMat Cin, int use_cin, do
   const int nwords = (min(B.nbc, kWindowCols) + 31) / 32;
   const int mw = (mask_words > 0 && mask_words < kMaskWords) ? mask_words : kMaskWords;
   size_t smem = ((size_t)max(nwords, 1) * 2 + mw) * sizeof(uint32_t);
-  if (digits) smem = max(smem, sizeof(int32_t) * kDigitMaxRows * (kSymThreads / 32));
+  const int threads = sym_threads(A.nbr, nsm);
+  if (digits) smem = max(smem, sizeof(int32_t) * kDigitMaxRows * (threads / 32));
   // one wave of resident blocks (rows taken in a grid stride): more resident
   // blocks hide more of each row's load latency, a second wave only adds a tail
   int per_sm = 0;
-  cudaError_t e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k_symbolic_fill,
-                                                                kSymThreads, smem);
+  const auto fill = threads == 512 ? k_symbolic_fill<512> : k_symbolic_fill<256>;
+  cudaError_t e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, fill, threads, smem);
   if (e != cudaSuccess) return e;
   const int grid = nsm * (per_sm > 0 ? per_sm : 1);
-  k_symbolic_fill<<<grid, kSymThreads, smem, stream>>>(A, B, Cin, use_cin, eps, ws, C, st, mw,
-                                                       digits ? *digits : Digits{});
+  fill<<<grid, threads, smem, stream>>>(A, B, Cin, use_cin, eps, ws, C, st, mw,
+                                        digits ? *digits : Digits{});
   return cudaGetLastError();
 }
 

@@ -76,3 +76,22 @@ def test_parts_of_blocks(gpu_ctx, n, sizes, launch):
     assert np.array_equal(got, H.to_dense(A) @ H.to_dense(B))
     for M in (dA, dB, dC):
         M.destroy()
+
+
+# rows: one; the most that get the wide thread blocks, one more; past the fused scan
+@pytest.mark.parametrize("eps", [0.0, 30.0])
+@pytest.mark.parametrize("rows", [1, 455, 456, 457, 2048, 2049])
+def test_rows_of_the_symbolic_phase(gpu_ctx, oracle_mod, rows, eps):
+    rng = np.random.default_rng(rows)
+    rs, ks, cs = rng.integers(1, 4, rows), rng.integers(1, 4, 70), rng.integers(1, 4, 40)
+    A = synth.random_blocks(rng, rs, ks, 0.3, kind="int", shuffle=True)
+    B = synth.random_blocks(rng, ks, cs, 0.3, kind="int", shuffle=True)
+    ref = oracle_mod.multiply(A, B, eps=eps)
+    dA, dB = gpu_ctx.from_blocks(A), gpu_ctx.from_blocks(B)
+    dC = gpu_ctx.empty(A.row_sizes, B.col_sizes)
+    st = gpu_ctx.multiply(1.0, dA, dB, 0.0, dC, eps, stats=True)
+    r, c = dC.pattern()
+    assert np.array_equal(r, ref.blk_row) and np.array_equal(c, ref.blk_col)
+    assert st.kept == ref.kept and st.flops == ref.flops and np.array_equal(dC.values(), ref.values)
+    for M in (dA, dB, dC):
+        M.destroy()
