@@ -68,7 +68,7 @@ MEASURED_TRAFFIC = {
     ("pk12", "water2048"): dict(
         sections=[("paper_1705_10218_gb300/csrc/k_numeric_fp64.cu",
                    ("// pk\n", "cudaError_t launch_numeric_fp64("),
-                   "d2f677421bba82e40c8a281c2384355575f55598d2d185672d3a3d378381dd67"),
+                   "c4d0a2d33d0541f245f25dabd7b17608518a0df277e5ea3ac09dc06495b99449"),
                   ("paper_1705_10218_gb300/csrc/k_classes.cu",
                    ("// Work in a row order.", "}  // namespace bsm"),
                    "b173af39936271e55c6a2623c0b1222afaca8a97ab34ff8f9a0ec78e9ecdf01b"),

@@ -861,8 +861,8 @@ __global__ void __launch_bounds__(kPkWarps * 32, 2)
 // Why: the FP64 pipe does 2 FMA per clock and SM, mma.sync on FP16 1024, and 43
 // digit pairs stand for one product. (FP8 and INT8 mma.sync are emulated or slow on
 // this part: 3.8 and 16 clocks per m16n8k32 and SM, FP16 m16n8k16 2.0.) Numeric
-// phase, packed kernel -> this one: water of 2048 molecules 47.7 -> 21.4 ms,
-// amorphous of 1024 atoms 67.9 -> 22.5, 64 x 64 full blocks of 32 15.7 -> 2.0. What
+// phase, packed kernel -> this one: water of 2048 molecules 47.7 -> 21.2 ms,
+// amorphous of 1024 atoms 67.9 -> 21.9, 64 x 64 full blocks of 32 15.7 -> 2.0. What
 // bounds it: the MMA pipe (0.49 of the clocks of the first) and the instructions beside
 // it, which do not hide behind the MMAs whatever the number of warps (with 16, 20 and 24
 // per SM 21.4, 21.9 and 22.2 ms): left out one at a time, the digits' conversion is
