@@ -134,8 +134,9 @@ typedef struct {
                           8 x 8, else T16_B2.
                           The form on the tensor cores multiplies 62-bit integer
                           images of the operands (on a scale per scalar row of A and
-                          column of B) exactly, digit by digit, and rounds to FP64
-                          once per 144 values of k; C blocks with an operand that such
+                          column of B) exactly, digit by digit, and rounds the sum
+                          to FP64 once (the sums of products of one magnitude, in
+                          steps of 2^8, each); C blocks with an operand that such
                           an image would hold less exactly than FP64 does (infinities,
                           NaN, rows of widely different size in one block) are left to
                           the packed kernel. It takes device memory for the images,

@@ -294,8 +294,7 @@ struct bsm_server_s {
 };
 
 static void drop_result(bsm_server s, Request *r) {
-  s->pinned.put(r->res_row);
-  s->pinned.put(r->res_col);
+  s->pinned.put(r->res_row);  // and res_col, in the same block
   s->pinned.put(r->res_val);
   r->res_row = r->res_col = nullptr;
   r->res_val = nullptr;
@@ -311,8 +310,8 @@ static int split_result(bsm_server s, Request *r, int32_t r0, int32_t r1, const 
   const int64_t b1 = std::lower_bound(rows, rows + nblk, r1) - rows;
   r->nblk = b1 - b0;
   r->nnz = voff[b1] - voff[b0];
-  r->res_row = static_cast<int32_t *>(s->pinned.get(4 * (size_t)r->nblk));
-  r->res_col = static_cast<int32_t *>(s->pinned.get(4 * (size_t)r->nblk));
+  r->res_row = static_cast<int32_t *>(s->pinned.get(8 * (size_t)r->nblk));
+  r->res_col = r->res_row ? r->res_row + r->nblk : nullptr;
   r->res_val = static_cast<double *>(s->pinned.get(8 * (size_t)r->nnz));
   if (!r->res_row || !r->res_col || !r->res_val) return BSM_ERR_NOMEM;
   for (int64_t b = b0; b < b1; b++) {  // block-diagonal: the columns lie in [r0, r1) too
@@ -389,8 +388,9 @@ static void run_batch(bsm_server s, Slot &sl, const std::vector<Request *> &batc
   double *vals = nullptr;
   const bool direct = rc == BSM_OK && hv && nnz <= hv_cap;  // values already in host memory
   if (rc == BSM_OK) {
-    rows = static_cast<int32_t *>(s->pinned.get(4 * (size_t)nblk));
-    cols = static_cast<int32_t *>(s->pinned.get(4 * (size_t)nblk));
+    // one block for both: a new page-locked block takes as long as a small multiply
+    rows = static_cast<int32_t *>(s->pinned.get(8 * (size_t)nblk));
+    cols = rows ? rows + nblk : nullptr;
     if (direct) {
       vals = hv;
       hv = nullptr;
@@ -417,7 +417,6 @@ static void run_batch(bsm_server s, Slot &sl, const std::vector<Request *> &batc
       rc = split_result(s, batch[p], row0[p], row0[p + 1], rows, cols, vals, nblk, voff);
   }
   s->pinned.put(rows);
-  s->pinned.put(cols);
   s->pinned.put(vals);
   s->pinned.put(hv);
   if (A) bsm_mat_destroy(A);
