@@ -2299,6 +2299,12 @@ int mat_create_diag(bsm_ctx ctx, int nparts, const DiagPart *parts, bsm_mat *out
   return BSM_OK;
 }
 
+int reserve_staging(bsm_ctx ctx, size_t bytes) {
+  if (!ctx) return BSM_ERR_INVALID_ARG;
+  const int rc = ctx_set_device(ctx);
+  return rc ? rc : stage_reserve(ctx, bytes);
+}
+
 int set_slice_gate(bsm_ctx ctx, SliceGate gate, void *arg) {
   if (!ctx) return BSM_ERR_INVALID_ARG;
   if (gate && !ctx->ev_gate) {

@@ -329,5 +329,7 @@ int mat_create_diag(bsm_ctx ctx, int nparts, const DiagPart *parts, bsm_mat *out
 // large multiply's next slice there while small multiplies run). nullptr: none.
 using SliceGate = void (*)(void *arg);
 int set_slice_gate(bsm_ctx ctx, SliceGate gate, void *arg);
+// Page-locked staging for uploads of block lists, ahead of the first one.
+int reserve_staging(bsm_ctx ctx, size_t bytes);
 
 }  // namespace bsm

@@ -29,6 +29,7 @@
 // request into the batch's matrix. Results go to page-locked host memory (the
 // multiply stores the values there directly when they fit) and wait there
 // until taken or released.
+#include <cstdlib>
 #include <cuda_runtime.h>
 
 #include <algorithm>
@@ -60,7 +61,8 @@ enum { kQueued = 0, kRunning = 1, kDone = 2, kFailed = 3 };
 struct Request {
   int64_t id = 0;
   std::vector<int32_t> sizes, brow, bcol;  // blocks sorted by (row, col)
-  double *vals = nullptr;  // page-locked copy of the values, in block order
+  double *vals = nullptr;  // copy of the values, in block order, page-locked or (heap) not
+  bool heap = false;
   const double *in_vals = nullptr;  // what the lane uploads: vals, or the caller's (borrowed)
   int64_t nvals = 0;
   double eps = 0;
@@ -130,6 +132,7 @@ double est_run_ms(int64_t macs, int precision) {
 // a result can be handed to the caller without a copy. Freed blocks are kept
 // for reuse (cudaHostAlloc is slow), up to kPinnedCap bytes.
 constexpr size_t kPinnedCap = 16ull << 30;
+constexpr size_t kHeapInput = 8u << 20;
 constexpr int64_t kHostValuesCap = 128ll << 20;  // values (1 GiB) a lane's multiply stores directly
 
 struct PinnedPool {
@@ -144,7 +147,8 @@ struct PinnedPool {
     const size_t step = (size_t)1 << (p - 3);
     return (b + step - 1) & ~(step - 1);
   }
-  void *get(size_t bytes) {
+  // at_hand: only a block that is there already (else null)
+  void *get(size_t bytes, bool at_hand = false) {
     const size_t cls = size_class(bytes);
     std::lock_guard<std::mutex> lk(mu);
     auto it = free_blocks.find(cls);
@@ -155,6 +159,7 @@ struct PinnedPool {
       return p;
     }
     void *p = nullptr;
+    if (at_hand) return p;
     if (cudaHostAlloc(&p, cls, cudaHostAllocDefault) != cudaSuccess) {
       cudaGetLastError();
       return nullptr;
@@ -293,6 +298,15 @@ struct bsm_server_s {
   bool stop = false;
 };
 
+static void drop_input(bsm_server s, Request *r) {
+  if (r->heap)
+    free(r->vals);
+  else
+    s->pinned.put(r->vals);
+  r->vals = nullptr;
+  r->heap = false;
+}
+
 static void drop_result(bsm_server s, Request *r) {
   s->pinned.put(r->res_row);  // and res_col, in the same block
   s->pinned.put(r->res_val);
@@ -424,8 +438,7 @@ static void run_batch(bsm_server s, Slot &sl, const std::vector<Request *> &batc
   const double t = now_ms();
   for (Request *r : batch) {
     if (rc != BSM_OK) drop_result(s, r);
-    s->pinned.put(r->vals);  // the host copy of the input is no longer needed
-    r->vals = nullptr;
+    drop_input(s, r);  // the host copy of the input is no longer needed
     r->in_vals = nullptr;  // a borrowed input is no longer read
     r->err = rc;
     r->t_done = t;
@@ -489,8 +502,10 @@ static void worker_loop(bsm_server s, int lane) {
     }
     int64_t held = 0;
     const double t = now_ms();
+    std::vector<size_t> heap;  // inputs that found no page-locked block
     for (Request *r : batch) {
       held += r->footprint;
+      if (r->heap) heap.push_back(8 * (size_t)std::max<int64_t>(r->nvals, 1));
       r->state = kRunning;
       r->slot = lane;
       r->t_start = t;
@@ -516,12 +531,17 @@ static void worker_loop(bsm_server s, int lane) {
     s->completed += (int64_t)batch.size();
     batch.clear();
     s->cv.notify_all();  // a head that waited for memory may fit now
+    if (!heap.empty()) {  // the next inputs of these sizes find one
+      lk.unlock();
+      for (size_t b : heap) s->pinned.put(s->pinned.get(b));
+      lk.lock();
+    }
   }
 }
 
 static void forget(bsm_server s, Request *r) {
   drop_result(s, r);
-  s->pinned.put(r->vals);
+  drop_input(s, r);
   delete r;
 }
 
@@ -550,6 +570,9 @@ int bsm_server_create(int device, const bsm_server_opts *opts, bsm_server *out) 
   for (Slot &sl : s->slots) {
     int rc = bsm_ctx_create(device, &sl.ctx);
     if (rc == BSM_OK) rc = bsm::set_slice_gate(sl.ctx, slice_gate, s);
+    // a lane's first small requests find their staging there: growing it frees the old
+    // one, which waits for every stream of the device
+    if (rc == BSM_OK) rc = bsm::reserve_staging(sl.ctx, 1 << 20);
     if (rc == BSM_OK &&
         cudaStreamCreateWithPriority(&sl.hi, cudaStreamNonBlocking, greatest) != cudaSuccess) {
       cudaGetLastError();
@@ -621,7 +644,14 @@ static int submit_request(bsm_server s, int32_t nbrows, const int32_t *sizes, in
   if (borrow) {
     r->in_vals = values;
   } else {
-    r->vals = static_cast<double *>(s->pinned.get(8 * (size_t)std::max<int64_t>(nv, 1)));
+    // a small copy goes to the heap rather than wait for a new page-locked block, which
+    // may wait for a lane that is allocating a large result's (tens of milliseconds)
+    const size_t bytes = 8 * (size_t)std::max<int64_t>(nv, 1);
+    r->vals = static_cast<double *>(s->pinned.get(bytes, bytes <= kHeapInput));
+    if (!r->vals && bytes <= kHeapInput) {
+      r->vals = static_cast<double *>(malloc(bytes));
+      r->heap = r->vals != nullptr;
+    }
     if (!r->vals) {
       delete r;
       return BSM_ERR_NOMEM;
