@@ -132,13 +132,16 @@ typedef struct {
                           on the tensor cores (below), or where C blocks have fewer
                           than 4 products on average, G8 when C's blocks are at most
                           8 x 8, else T16_B2.
-                          The form on the tensor cores multiplies 62-bit integer
-                          images of the operands (on a scale per scalar row of A and
-                          column of B) exactly, digit by digit, and rounds the sum
-                          to FP64 once (the sums of products of one magnitude, in
-                          steps of 2^8, each); C blocks with an operand that such
-                          an image would hold less exactly than FP64 does (infinities,
-                          NaN, rows of widely different size in one block) are left to
+                          The form on the tensor cores holds the operands as 62-bit integers
+                          (on a scale per scalar row of A and column of B) and adds their
+                          products up in exact integers, 43 of 64 digit pairs of each, then
+                          rounds to FP64 (once for the products of one magnitude, in
+                          steps of 2^8). What that loses is bounded for every element:
+                          C blocks with an element where it may be more than (4 sqrt(N) - 2)
+                          2^-53 of the sum of its absolute products (N terms; FP64 FMAs
+                          lose up to N 2^-53 of it), and those with an operand that such an
+                          image does not hold (infinities, NaN, scales beyond 2^+-300, rows
+                          of widely different size in one block) are left to
                           the packed kernel. It takes device memory for the images,
                           about 1.6 times the operands' values each, kept with the
                           context; without that memory PK12 runs */

@@ -905,7 +905,7 @@ static int launch_numeric(Launch &L, int variant, const int32_t *items, const in
     ctx->last_fp64 = variant == kFp64Dg ? (int)kFp64Pk12 : variant;
     Digits dg = ctx->dg;
     dg.list = L.ws.cnt;  // the fill pass's counters, free by now
-    if (variant == kFp64Dg) CK(cudaMemsetAsync(dg.range, 0, 2 * sizeof(int64_t), L.s));
+    if (variant == kFp64Dg) CK(cudaMemsetAsync(dg.range, 0, digit_state_bytes(ctx->nsm), L.s));
     L.host_written = L.host_written && fp64_variant_writes_host(variant);
     CK(launch_numeric_fp64(variant, L.dA, L.dB, L.out, L.dC, L.alpha, L.beta, L.ws,
                            ctx->d_status, items, seg,
@@ -1428,8 +1428,9 @@ int bsm_ctx_create(int device, bsm_ctx *out) {
   }
   if (rc == BSM_OK) {
     rc = dev_alloc(&ctx->cls_counts, kMaxClasses);
-    if (rc == BSM_OK) rc = dev_alloc(&ctx->dg.range, 3);  // and the ticket
-    ctx->d_ticket = reinterpret_cast<int32_t *>(ctx->dg.range + 2);
+    if (rc == BSM_OK) rc = dev_alloc(&ctx->dg.range, digit_state_bytes(ctx->nsm) / 8 + 2);
+    ctx->dg.marks = reinterpret_cast<uint32_t *>(ctx->dg.range + 2);
+    ctx->d_ticket = reinterpret_cast<int32_t *>(ctx->dg.range + digit_state_bytes(ctx->nsm) / 8 + 1);
     if (rc == BSM_OK && (e = cudaMemsetAsync(ctx->d_ticket, 0, sizeof(int32_t), ctx->stream)) != cudaSuccess)
       rc = cuda_fail(e, "cudaMemset");
     if (rc == BSM_OK) rc = dev_alloc(&ctx->cls_cursor, kMaxClasses);

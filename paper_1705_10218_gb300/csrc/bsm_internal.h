@@ -97,23 +97,26 @@ struct DevStatus {
 // left operand; its columns as the rows of a right one) is ceil(s / 8) octets of
 // 4 units for each row, row after row: as much as its FP64 values, with k up to a
 // multiple of 8. Block b's units start at kDigitZeros + (blk_off[b] * mul >> 6) +
-// b * pad; the units before are zeros. meta[b]: {first unit, octets | class << 16 |
-// kDigitOutside}. A block is outside when a digit representation would lose more
-// than FP64 does: a value that is not finite, a scale beyond 2^+-300, a row (column)
-// of the block whose largest value is below 2^-kDigitRange of the scale less the
-// class (it would keep less than 62 - kDigitRange bits), or more than kDigitMaxRows
-// rows or kDigitMaxOctets octets; the C blocks it contributes to are computed by
-// FP64 FMAs.
+// b * pad; the units before are zeros. meta[b]: the first unit, and the fields below
+// (octets in the low 16 bits).
+// What is lost: half a unit of X for each value, and the digit pairs (i, j) with
+// i + j > 8 of each product. Values far below the scale keep few bits of their own, so
+// the digit kernel bounds both for every element of C against the sum of its absolute
+// products, and leaves the C blocks that have an element below the bound to FP64 FMAs
+// (dg_enough in k_numeric_fp64.cu). Left to them at once are the C blocks that an
+// "outside" block contributes to: one with a value that is not finite, a scale beyond
+// 2^+-300, a row (column) whose largest value is below 2^-kDigitRange of the scale less
+// the class, or more than kDigitMaxRows rows or kDigitMaxOctets octets.
 // ---------------------------------------------------------------------------
 constexpr int kDigits = 8;
 constexpr int kDigitZeros = 64;
 constexpr uint32_t kDigitOutside = 1u << 31;
-// How far a row may lie below its block's class. Wider keeps more C blocks on the tensor
-// cores and fewer bits of such a row; at 12 the error of every element against the sum of
-// its absolute products is no larger than at 9, 10 or 11 (where FP64 FMAs take more C blocks)
-// on blocks of 1 to 33, sign iterates, water and amorphous systems, and below the FP64
-// kernel's: sign iterates 0.4, 2.2 and 0.8e-15, 2.4, 3.0 and 4.4e-15 there. Two sign iterations
-// of 192 water molecules: 18.6 ms at 9, 15.3 at 11, 14.4 at 12, 13 and 15.
+// fields of meta[b].y: the class; by how many bits (0 to 7) every row of the block stays
+// below its scale less the class; the zeros that fill up the last octet
+constexpr int kDigitClassAt = 16, kDigitGapAt = 24, kDigitPadAt = 27;
+// How far a row may lie below its block's class before all C blocks of the block are FP64
+// FMAs'. A wider range keeps more C blocks on the tensor cores: two sign iterations of 192
+// water molecules 18.6 ms at 9, 15.3 at 11, 14.4 at 12, 13 and 15.
 constexpr int kDigitRange = 12;
 constexpr int kDigitMaxRows = 128;
 constexpr int kDigitMaxOctets = 0xFFFF;
@@ -132,10 +135,13 @@ struct DigitSide {
 struct Digits {
   DigitSide a, b;
   // C blocks that the digit kernel leaves to the packed one: their number
-  // (range[0] = 0, range[1]) and list
+  // (range[0] = 0, range[1]) and list, and a bit for each that several warps share and that
+  // is in it (behind the range: digit_state_bytes of both, zero before a launch)
   int64_t *range;
+  uint32_t *marks;
   int32_t *list;
 };
+int64_t digit_state_bytes(int nsm);
 
 // ---- launchers (each enqueues on `stream`, returns cudaGetLastError()) ----
 // The norms, and the largest exponent fields of every scalar row (column) into

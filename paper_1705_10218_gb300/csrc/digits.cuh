@@ -61,7 +61,7 @@ __device__ __forceinline__ void digit_layout(const double *__restrict__ x, int r
   const int32_t *expo = o.expo + first;
   uint4 *units = o.units + base;
   bool outside = rows > kDigitMaxRows || octets > kDigitMaxOctets;
-  int cls = 0;
+  int cls = 0, gap = 0;
   if (!outside) {
     // the largest exponent field of each row of the block
     for (int r = lane; r < rows; r += 32) seg[r] = 0;
@@ -81,6 +81,7 @@ __device__ __forceinline__ void digit_layout(const double *__restrict__ x, int r
     }
     room = __reduce_min_sync(0xffffffffu, room);
     cls = room >> 3;
+    gap = room & 7;
     for (int r = lane; r < rows; r += 32)
       outside |= seg[r] && seg[r] < expo[r] - 8 * cls - kDigitRange;
     outside = __any_sync(0xffffffffu, outside);
@@ -97,8 +98,11 @@ __device__ __forceinline__ void digit_layout(const double *__restrict__ x, int r
   }
   outside = __any_sync(0xffffffffu, outside);
   if (lane == 0)
-    o.meta[b] = make_uint2((uint32_t)base, (uint32_t)octets | (uint32_t)cls << 16 |
-                                               (outside ? kDigitOutside : 0u));
+    o.meta[b] = make_uint2((uint32_t)base,
+                           outside ? kDigitOutside
+                                   : (uint32_t)octets | (uint32_t)cls << kDigitClassAt |
+                                         (uint32_t)gap << kDigitGapAt |
+                                         (uint32_t)(8 * octets - s) << kDigitPadAt);
 }
 
 // The digits of M as a left and / or right operand, one warp per block.

@@ -850,19 +850,24 @@ __global__ void __launch_bounds__(kPkWarps * 32, 2)
 // operands that are small integers, so every term is exact) into one FP32
 // accumulator per element and diagonal. With at most 144 values of k between two
 // reads its sums stay below 2^24, where FP32 numbers are exact integers. A read
-// adds the diagonals up in 64-bit integers, and the whole sum is rounded to FP64 once;
-// what is lost besides is half a unit of 2^-62 of each row's scale and the diagonals
-// from kDgDiag on (2^-70 of the largest product of the row and column).
+// adds the diagonals up in 64-bit integers, and the whole sum (of the products of one
+// class) is rounded to FP64 once. What is lost besides is half a unit of 2^-62 of each
+// row's scale and the diagonals from kDgDiag on (2^-67.4 of the product of the scales for
+// each value of k): dg_enough says for which C blocks that is no more than FP64 FMAs lose.
 // Measured against long double, relative Frobenius error of C (and the worst of C's
-// blocks): water of 128 molecules 4.5e-17 (7.5e-17), the packed kernel 4.7e-16
+// blocks): water of 128 molecules 4.5e-17 (1.4e-16), the packed kernel 4.7e-16
 // (7.9e-16); amorphous of 200 atoms 4.6e-17 (7.3e-17), packed 1.0e-15 (1.7e-15); rows of
-// unlike scales in blocks of 1 to 33 5.9e-17 (4.4e-16), packed 4.0e-16 (9.6e-15).
+// unlike scales in blocks of 1 to 33 5.9e-17 (4.4e-16), packed 4.0e-16 (9.6e-15). Largest
+// error of an element against the sum of its absolute products: ragged blocks 2.7e-16, sign
+// iterates of 64 water molecules 2.4, 2.7 and 4.3e-15, water 1.0e-16, amorphous 1.0e-16;
+// packed 5.1e-16; 2.4, 3.0 and 4.4e-15; 2.0e-15; 3.1e-15.
 //
 // Why: the FP64 pipe does 2 FMA per clock and SM, mma.sync on FP16 1024, and 43
 // digit pairs stand for one product. (FP8 and INT8 mma.sync are emulated or slow on
 // this part: 3.8 and 16 clocks per m16n8k32 and SM, FP16 m16n8k16 2.0.) Numeric
-// phase, packed kernel -> this one: water of 2048 molecules 47.7 -> 21.2 ms,
-// amorphous of 1024 atoms 67.9 -> 21.9, 64 x 64 full blocks of 32 15.7 -> 2.0. What
+// phase, packed kernel -> this one: water of 2048 molecules 47.7 -> 23.4 ms (21.3 without
+// dg_enough, 0.8 of it the packed kernel's on the 8% of the C blocks that it leaves),
+// amorphous of 1024 atoms 67.9 -> 22.8 (22.0), 64 x 64 full blocks of 32 15.7 -> 2.0. What
 // bounds it: the MMA pipe (0.49 of the clocks of the first) and the instructions beside
 // it, which do not hide behind the MMAs whatever the number of warps (with 16, 20 and 24
 // per SM 21.4, 21.9 and 22.2 ms): left out one at a time, the digits' conversion is
@@ -931,6 +936,13 @@ __device__ __forceinline__ double dg_scaled(double v, int e) {
   return v * __hiloint2double((1023 + half) << 20, 0) * __hiloint2double((1023 + e - half) << 20, 0);
 }
 
+// Fields of a block's metadata: its class, its gap, its values of k.
+__device__ __forceinline__ int dg_class(uint2 x) { return (int)(x.y >> kDigitClassAt & 0xFF); }
+__device__ __forceinline__ int dg_gap(uint2 x) { return (int)(x.y >> kDigitGapAt & 7); }
+__device__ __forceinline__ int dg_length(uint2 x) {
+  return 8 * (int)(x.y & 0xFFFF) - (int)(x.y >> kDigitPadAt & 7);
+}
+
 // A word of a unit (digits 2 i and 2 i + 1 of two values) as the two MMA registers.
 __device__ __forceinline__ uint32_t dg_even(uint32_t w) { return digit_half2(w, 0x4140); }
 __device__ __forceinline__ uint32_t dg_odd(uint32_t w) { return digit_half2(w, 0x4342); }
@@ -991,7 +1003,7 @@ __device__ __forceinline__ int dg_tile(const Digits &dg, const int2 *__restrict_
   for (int pb = 0;;) {
     const uint2 xa = ma, xb = mb;  // lane p: product p of the batch
     const bool in = pb + lane < np;
-    const int cls = (int)(xa.y >> 16 & 0xFF) + (int)(xb.y >> 16 & 0xFF);
+    const int cls = dg_class(xa) + dg_class(xb);
     pb += 32;
     if (pb < np) {  // the next batch's metadata, on its way during this one
       ma = mb = make_uint2(0, 0);
@@ -1080,15 +1092,154 @@ __device__ __forceinline__ int dg_tile(const Digits &dg, const int2 *__restrict_
   }
 }
 
+// Whether the digits hold enough of a C block. A product's value of k loses at most
+// 2^-63 (2^-gb + 2^-ga) + 2^-67.4 in units of W, the product of the row's and the
+// column's scale less the classes (half a unit of X each, beside values below 2^-ga or
+// 2^-gb of the scale, and the digit pairs beyond kDgDiag). The sum of that over the C block
+// may be at most (4 sqrt(N) - 2) 2^-53 of the element's sum of absolute products, N the
+// block's number of values of k. That is no more than (N + 2) 2^-53, where FP64 FMAs have
+// N 2^-53 in the worst case; and the losses being independent, what is lost of elements at
+// this very limit is about what FP64 FMAs lose (normal values of one size; root mean
+// square in units of 2^-53 of that sum, the rounding of the result with it, where FP64 has
+// 0.4 to 0.5: N = 5 0.31, 13 0.37, 50 0.33, 200 0.20), of most elements far less.
+// The sum of absolute products is bounded from below by the two top digits t of both
+// values (2^14 of the scale): t_a t_b less the digits' rounding, added up by one MMA for
+// every 16 k. Any part of the products will do, so those of the largest scales go first and
+// it ends when every element has enough, mostly after the first one or two. C blocks that
+// have not enough with all of theirs are left to the packed kernel.
+// 2^-ga + 2^-gb
+__device__ __forceinline__ float dg_sizes(uint2 a, uint2 b) {
+  return __int_as_float((127 - dg_gap(a)) << 23) + __int_as_float((127 - dg_gap(b)) << 23);
+}
+// the weight of products whose classes add up to d more than the least (2 and more: at most this)
+__device__ __forceinline__ float dg_weight(int d) {
+  return d == 0 ? 1.0f : d == 1 ? 0x1p-8f : 0x1p-16f;
+}
+
+// What the sums of t_a t_b have to reach; infinity where an operand block is outside.
+// least: the least sum of two classes.
+__device__ __forceinline__ float dg_need(const Digits &dg, const int2 *__restrict__ prods, int np,
+                                         uint2 ma, uint2 mb, int &least, int lane) {
+  auto loss = [&](uint2 a, uint2 b) {
+    return (float)dg_length(a) * (0x1p18f * dg_sizes(a, b) + 12400.0f);
+  };
+  // the lane's products: their least class and their loss at its weight
+  int cls = 1 << 10, n = 0;
+  float sum = 0.0f;
+  uint32_t flags = ma.y | mb.y;
+  if (lane < np) {
+    cls = dg_class(ma) + dg_class(mb);
+    n = dg_length(ma);
+    sum = loss(ma, mb);
+  }
+  for (int p = lane + 32; p < np; p += 32) {
+    const int2 q = __ldg(prods + p);
+    const uint2 a = __ldg(dg.a.meta + q.x), b = __ldg(dg.b.meta + q.y);
+    const int c = dg_class(a) + dg_class(b), now = min(c, cls);
+    sum = sum * dg_weight(cls - now) + loss(a, b) * dg_weight(c - now);
+    cls = now;
+    n += dg_length(a);
+    flags |= a.y | b.y;
+  }
+  if (__any_sync(0xffffffffu, flags & kDigitOutside)) return INFINITY;
+  least = __reduce_min_sync(0xffffffffu, cls);
+  n = __reduce_add_sync(0xffffffffu, n);
+  sum *= dg_weight(cls - least);
+#pragma unroll
+  for (int d = 16; d; d >>= 1) sum += __shfl_xor_sync(0xffffffffu, sum, d);
+  // t carries 11 bits, the sums 24, the root and the quotient 20: 1% covers them
+  return __fdividef(1.01f * sum, 4.0f * (float)n * rsqrtf((float)n) - 2.0f);
+}
+
+__device__ __forceinline__ uint32_t dg_top(uint32_t w) {  // |256 d_0 + d_1| of two values
+  uint32_t h = dg_even(w);
+  asm("fma.rn.f16x2 %0, %0, %1, %2;\n" : "+r"(h) : "r"(0x5C005C00u), "r"(dg_odd(w)));
+  return h & 0x7FFF7FFFu;
+}
+
+// Whether each element of a tile reaches `need`: rows from r0 of A and columns from c0 of
+// B, tm x tn of up to 16 x 16 (the left side's registers serve both halves of the columns).
+__device__ __forceinline__ bool dg_enough(const Digits &dg, const int2 *__restrict__ prods, int np,
+                                          uint2 ma, uint2 mb, int m, int n, int r0, int c0, int tm,
+                                          int tn, float need, int least, int lane) {
+  const int g = lane >> 2, t = lane & 3;
+  // rows and columns past the last one: the last one again, so that every sum is an element's
+  const uint4 *__restrict__ ua = dg.a.units + min(g, tm - 1) * 4 + t;
+  const uint4 *__restrict__ ub = dg.b.units + min(g, tn - 1) * 4 + t;
+  const int low = (min(g + 8, tm - 1) - min(g, tm - 1)) * 4;
+  const int right = (min(g + 8, tn - 1) - min(g, tn - 1)) * 4;
+  float sum[2][4] = {};
+  for (int pb = 0;;) {
+    const int above = dg_class(ma) + dg_class(mb) - least;
+    uint32_t key = pb + lane < np && above <= 1
+                       ? (uint32_t)(8 * above + dg_gap(ma) + dg_gap(mb)) << 5 | lane
+                       : ~0u;
+#pragma unroll 1
+    for (;;) {
+      const uint32_t best = __reduce_min_sync(0xffffffffu, key);
+      if (best == ~0u) break;
+      const int p = best & 31;
+      if (lane == p) key = ~0u;
+      const uint2 xa = make_uint2(__shfl_sync(0xffffffffu, ma.x, p), __shfl_sync(0xffffffffu, ma.y, p));
+      const uint2 xb = make_uint2(__shfl_sync(0xffffffffu, mb.x, p), __shfl_sync(0xffffffffu, mb.y, p));
+      const int octets = (int)(xa.y & 0xFFFF);
+      float acc[2][4] = {};
+#pragma unroll 1
+      for (int o = 0; o < octets; o += 2) {
+        uint32_t a[2], a8[2], b[2], b8[2];
+#pragma unroll
+        for (int h = 0; h < 2; h++) {
+          const bool in = o + h < octets;  // else zeros
+          const uint4 *pa = ua + (in ? xa.x + (uint32_t)(4 * r0 + (o + h) * 4 * m) : 0u);
+          const uint4 *pb = ub + (in ? xb.x + (uint32_t)(4 * c0 + (o + h) * 4 * n) : 0u);
+          a[h] = __ldg(&pa->x);
+          a8[h] = __ldg(&pa[low].x);
+          b[h] = __ldg(&pb->x);
+          if (tn > 8) b8[h] = __ldg(&pb[right].x);
+        }
+        const uint32_t x0 = dg_top(a[0]), x1 = dg_top(a8[0]), x2 = dg_top(a[1]), x3 = dg_top(a8[1]);
+        dg_mma(acc[0], x0, x1, x2, x3, dg_top(b[0]), dg_top(b[1]));
+        if (tn > 8) dg_mma(acc[1], x0, x1, x2, x3, dg_top(b8[0]), dg_top(b8[1]));
+      }
+      const float w = dg_weight(dg_class(xa) + dg_class(xb) - least);
+      // t may be 0.503 above the value: what that adds at most
+      need += w * (float)dg_length(xa) * (8260.0f * dg_sizes(xa, xb) + 0.3f);
+      bool enough = true;
+#pragma unroll
+      for (int e = 0; e < 4; e++) {
+        sum[0][e] += w * acc[0][e];
+        sum[1][e] += w * acc[1][e];
+        enough = enough && sum[0][e] >= need && (tn <= 8 || sum[1][e] >= need);
+      }
+      if (__all_sync(0xffffffffu, enough)) return true;
+    }
+    pb += 32;
+    if (pb >= np) return false;
+    ma = mb = make_uint2(0, 0);
+    if (pb + lane < np) {
+      const int2 pr = __ldg(prods + pb + lane);
+      ma = __ldg(dg.a.meta + pr.x);
+      mb = __ldg(dg.b.meta + pr.y);
+    }
+  }
+}
+
 struct DgItem {  // a C block of a warp's run
   const int2 *prods;
   int64_t coff;
   int32_t gblk, np, m, n, cin, fa, fb;
   int32_t part, nparts;  // the part of its tiles that is to be done
+  int32_t at;            // its number in the work range
 };
+// words of the bits in dg.marks: a bit for each C block that is split into parts
+constexpr int dg_mark_words(int warps) { return (kDgUnits * warps / 2 + 31) / 32; }
+int64_t digit_state_bytes(int nsm) {
+  return 2 * sizeof(int64_t) + 4 * (int64_t)dg_mark_words(nsm * kDgBlocksPerSm * kDgWarps);
+}
 
-// C blocks without products (C_in only) and those with an operand block outside
-// go to dg.list, for the packed kernel.
+// C blocks without products (C_in only), with an operand block outside or with too little
+// of the digits go to dg.list, for the packed kernel (whose values replace those that other
+// parts of such a block have stored).
 __global__ void __launch_bounds__(kDgWarps * 32, kDgBlocksPerSm)
     k_numeric_fp64_dg(DevMat A, DevMat B, DevOut C, DevMat Cin, double alpha, double beta,
                       DevWs ws, const DevStatus *st, const int32_t *items, const int64_t *seg,
@@ -1130,6 +1281,7 @@ __global__ void __launch_bounds__(kDgWarps * 32, kDgBlocksPerSm)
       it.part = nparts > 1 ? (int)(unit % nparts) : 0;
       it.nparts = nparts;
       it.gblk = items ? items[blk] : (int)blk;
+      it.at = (int)(blk - wb);
       const int64_t pp = ws.prod_ptr[it.gblk];
       it.prods = ws.prods + pp;
       it.np = (int)(ws.prod_ptr[it.gblk + 1] - pp);
@@ -1164,20 +1316,32 @@ __global__ void __launch_bounds__(kDgWarps * 32, kDgBlocksPerSm)
       const DgItem &it = item[x];
       products(x + 1);
       const int np = it.np;
-      uint32_t flags = ma.y | mb.y;
-      for (int p = lane + 32; p < np; p += 32) {
-        const int2 q = __ldg(it.prods + p);
-        flags |= dg.a.meta[q.x].y | dg.b.meta[q.y].y;
+      const int m = it.m, n = it.n;
+      const uint2 ka = ma, kb = mb;
+      int at = 0;  // the tile's number
+      int least;
+      const float need = np > 0 ? dg_need(dg, it.prods, np, ka, kb, least, lane) : INFINITY;
+      bool held = need < INFINITY;
+      bool first = it.part == 0;  // that finds out
+      if (held) {
+        for (int r0 = 0; r0 < m && held; r0 += 16)
+          for (int c0 = 0; c0 < n && held; c0 += 16) {
+            if (it.nparts > 1 && at++ % it.nparts != it.part) continue;
+            held = dg_enough(dg, it.prods, np, ka, kb, m, n, r0, c0, min(16, m - r0),
+                             min(16, n - c0), need, least, lane);
+          }
+        at = 0;
+        if (!held && it.nparts > 1 && lane == 0) {
+          const uint32_t bit = 1u << (it.at & 31);
+          first = !(atomicOr(dg.marks + (it.at >> 5), bit) & bit);
+        }
       }
-      if (np == 0 || __any_sync(0xffffffffu, flags & kDigitOutside)) {
-        if (lane == 0 && it.part == 0)
+      if (!held) {
+        if (lane == 0 && first)
           dg.list[atomicAdd(reinterpret_cast<unsigned long long *>(dg.range + 1), 1ull)] = it.gblk;
         metadata();
         continue;
       }
-      const int m = it.m, n = it.n;
-      const uint2 ka = ma, kb = mb;
-      int at = 0;  // the tile's number
       for (int r0 = 0; r0 < m; r0 += 16) {
         for (int c0 = 0; c0 < n; c0 += 8) {
           if (it.nparts > 1 && at++ % it.nparts != it.part) continue;
