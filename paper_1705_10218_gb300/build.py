@@ -34,6 +34,11 @@ def sources() -> list[str]:
     return sorted(glob.glob(os.path.join(CSRC, "*.cu")) + glob.glob(os.path.join(CSRC, "*.cpp")))
 
 
+def headers() -> list[str]:
+    return sorted(glob.glob(os.path.join(CSRC, "*.h")) + glob.glob(os.path.join(CSRC, "*.cuh")) +
+                  [os.path.join(ROOT, "include", "bsm.h")])
+
+
 def _stale(lib: str, deps: list[str]) -> bool:
     if not os.path.exists(lib):
         return True
@@ -42,8 +47,7 @@ def _stale(lib: str, deps: list[str]) -> bool:
 
 
 def build(force: bool = False, verbose: bool = False) -> str:
-    deps = sources() + glob.glob(os.path.join(CSRC, "*.h")) + [os.path.join(ROOT, "include", "bsm.h")]
-    if not force and not _stale(LIB, deps):
+    if not force and not _stale(LIB, sources() + headers()):
         return LIB
     nvcc = _nvcc()
     os.makedirs(BUILD, exist_ok=True)
