@@ -615,13 +615,16 @@ static bool digit_entries(bsm_ctx ctx, bsm_mat A, bsm_mat B, cudaStream_t s) {
     sides[x]->pad = by_value ? 0 : pad;
     const int64_t n = kDigitZeros + (M->nnz * sides[x]->mul >> 6) + M->nblk * sides[x]->pad + 1;
     if (n >= (int64_t)UINT32_MAX) return false;
-    const void *old = sides[x]->units;
-    if (!digit_grow(ctx, sides[x]->units, ctx->cap_dg_units[x], n) ||
-        !digit_grow(ctx, sides[x]->meta, ctx->cap_dg_meta[x], M->nblk))
-      return false;
-    if (sides[x]->units != old &&
-        cudaMemsetAsync(sides[x]->units, 0x80, kDigitZeros * sizeof(uint4), s) != cudaSuccess)
-      return false;
+    // the zeros at its start belong to a new buffer, whatever else fails and wherever it lies
+    if (ctx->cap_dg_units[x] < n) {
+      if (!digit_grow(ctx, sides[x]->units, ctx->cap_dg_units[x], n)) return false;
+      if (cudaMemsetAsync(sides[x]->units, 0x80, kDigitZeros * sizeof(uint4), s) != cudaSuccess) {
+        dev_free(sides[x]->units);
+        ctx->cap_dg_units[x] = 0;
+        return false;
+      }
+    }
+    if (!digit_grow(ctx, sides[x]->meta, ctx->cap_dg_meta[x], M->nblk)) return false;
   }
   return true;
 }
