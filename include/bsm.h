@@ -144,7 +144,8 @@ typedef struct {
                           of widely different size in one block) are left to
                           the packed kernel. It takes device memory for the images,
                           about 1.6 times the operands' values each, kept with the
-                          context; without that memory PK12 runs */
+                          context and given back when an allocation of any context of the
+                          process on that device fails; without that memory PK12 runs */
   double *host_values; /* NULL, or page-locked host memory (cudaHostAlloc /
                           cudaHostRegister, device-mapped) of host_cap doubles that also
                           receives the result's values, in bsm_mat_get_values order,

@@ -20,6 +20,7 @@
 #include <cstring>
 #include <map>
 #include <mutex>
+#include <optional>
 #include <string>
 #include <new>
 #include <numeric>
@@ -164,16 +165,15 @@ void cache_free(void *p) {
   }
 }
 
-// The context of the call that runs on this thread: an allocation that fails
-// takes back its digit workspace (which a multiply can do without) and retries.
-thread_local bsm_ctx t_ctx = nullptr;
-bool digit_reclaim(bsm_ctx ctx);
+// An allocation that fails takes back the digit workspaces of the device's contexts
+// (which a multiply can do without) and retries.
+bool digits_reclaim();
 
 cudaError_t cache_alloc_reclaim(void **p, size_t bytes) {
   cudaError_t e = cache_alloc(p, bytes);
-  if (e == cudaErrorMemoryAllocation && t_ctx) {
+  if (e == cudaErrorMemoryAllocation) {
     cudaGetLastError();
-    if (digit_reclaim(t_ctx)) e = cache_alloc(p, bytes);
+    if (digits_reclaim()) e = cache_alloc(p, bytes);
   }
   return e;
 }
@@ -320,6 +320,8 @@ struct bsm_ctx_s {
   // scales), for the FP64 products on the tensor cores; capacities in elements
   Digits dg{};
   int64_t cap_dg_units[2] = {0, 0}, cap_dg_meta[2] = {0, 0}, cap_dg_expo[2] = {0, 0};
+  bsm_ctx next_ctx = nullptr;  // in the list of all contexts
+  std::mutex dg_mu;  // held while a multiply that uses them is enqueued, or while they are freed
   int32_t *cls_counts = nullptr, *cls_cursor = nullptr;  // [kMaxClasses]
   int64_t *cls_segs = nullptr;   // [2 * kMaxClasses]
   // captured multiplies (opts.graph), keyed by every kernel argument
@@ -370,7 +372,6 @@ static int prof_collect(bsm_ctx ctx, int s) {
 }
 
 static int ctx_set_device(bsm_ctx ctx) {
-  t_ctx = ctx;
   CK(cudaSetDevice(ctx->device));
   return BSM_OK;
 }
@@ -555,38 +556,75 @@ static int enqueue_norms(bsm_ctx ctx, bsm_mat M, cudaStream_t s, int32_t *rexp =
   return BSM_OK;
 }
 
-// The digit workspace. digit_reclaim: gives it back. digit_scales: the scale arrays of A's rows and B's
-// columns; digit_entries: the entries and block metadata. Both return false
-// (and leave the FP64 kernels to the multiply) where the operands have more
-// values or rows than the 32-bit indices reach, or the memory is not there.
+// The digit workspace. digits_reclaim: gives those of all contexts back. digit_scales: the
+// scale arrays of A's rows and B's columns; digit_entries: the entries and block metadata.
+// Both return false (and leave the FP64 kernels to the multiply) where the operands have
+// more values or rows than the 32-bit indices reach, or the memory is not there.
 namespace {
-// Frees the entries and metadata (not the scales, which are small) once the
-// work that uses them is done; true if there were any.
-bool digit_reclaim(bsm_ctx ctx) {
-  DigitSide *sides[2] = {&ctx->dg.a, &ctx->dg.b};
-  bool any = false;
-  for (int x = 0; x < 2; x++) any = any || sides[x]->units || sides[x]->meta;
-  if (!any || cudaStreamSynchronize(ctx->stream) != cudaSuccess) return false;
-  for (int x = 0; x < 2; x++) {
-    dev_free(sides[x]->units);
-    dev_free(sides[x]->meta);
-    ctx->cap_dg_units[x] = ctx->cap_dg_meta[x] = 0;
+std::mutex g_ctx_mu;  // of the list; taken before a context's dg_mu
+bsm_ctx g_ctxs = nullptr;  // every context, by next_ctx
+// The context whose digits the multiply that runs on this thread holds.
+thread_local bsm_ctx t_digits = nullptr;
+
+// Holds a context's digits while a multiply that uses them is enqueued; if that fails, until
+// what was enqueued is done.
+struct DigitHold {
+  bsm_ctx ctx;
+  cudaStream_t s;
+  bool done = false;
+  DigitHold(bsm_ctx c, cudaStream_t st) : ctx(c), s(st) {
+    ctx->dg_mu.lock();
+    t_digits = ctx;
   }
-  return true;
+  ~DigitHold() {
+    if (!done) cudaStreamSynchronize(s);
+    t_digits = nullptr;
+    ctx->dg_mu.unlock();
+  }
+  DigitHold(const DigitHold &) = delete;
+  DigitHold &operator=(const DigitHold &) = delete;
+};
+
+// Frees the entries and metadata (not the scales, which are small) of the device's contexts
+// once the work that uses them is done, except those that a multiply is being enqueued on;
+// true if there were any. Any multiply's work is followed by its context's stream.
+bool digits_reclaim() {
+  int dev = -1;
+  if (cudaGetDevice(&dev) != cudaSuccess) return false;
+  std::lock_guard<std::mutex> list(g_ctx_mu);
+  bool any = false;
+  for (bsm_ctx c = g_ctxs; c; c = c->next_ctx) {
+    if (c->device != dev || c == t_digits) continue;
+    std::unique_lock<std::mutex> lock(c->dg_mu, std::try_to_lock);
+    if (!lock.owns_lock()) continue;
+    DigitSide *sides[2] = {&c->dg.a, &c->dg.b};
+    bool here = false;
+    for (int x = 0; x < 2; x++) here = here || sides[x]->units || sides[x]->meta;
+    if (!here || cudaStreamSynchronize(c->stream) != cudaSuccess) continue;
+    for (int x = 0; x < 2; x++) {
+      dev_free(sides[x]->units);
+      dev_free(sides[x]->meta);
+      c->cap_dg_units[x] = c->cap_dg_meta[x] = 0;
+    }
+    any = true;
+  }
+  return any;
 }
 }  // namespace
 
+// Digits take nothing back from other contexts.
 template <class T>
 static bool digit_grow(bsm_ctx ctx, T *&p, int64_t &cap, int64_t n) {
   if (cap >= n) return true;
   if (p && cudaStreamSynchronize(ctx->stream) != cudaSuccess) return false;
   dev_free(p);
   cap = 0;
-  const bsm_ctx c = t_ctx;
-  t_ctx = nullptr;  // the digits take nothing back from themselves
-  const int rc = dev_alloc(&p, n + n / 8 + 64);
-  t_ctx = c;
-  if (rc) return false;
+  void *q = nullptr;
+  if (cache_alloc(&q, (size_t)(n + n / 8 + 64) * sizeof(T)) != cudaSuccess) {
+    cudaGetLastError();
+    return false;
+  }
+  p = static_cast<T *>(q);
   cap = n + n / 8 + 64;
   return true;
 }
@@ -1234,7 +1272,11 @@ static int run_multiply(bsm_ctx ctx, double alpha, bsm_mat A, bsm_mat B, double 
   auto wants_digits = [&]() {
     return o.autotune || !ctx->tune.empty() || fp64_default(ctx, C, true) == kFp64Dg;
   };
-  L.scales = !L.split && !o.fp64_kernel && (sync_sizes || wants_digits()) && digit_scales(ctx, A, B);
+  std::optional<DigitHold> hold;
+  if (!L.split && !o.fp64_kernel && (sync_sizes || wants_digits())) {
+    hold.emplace(ctx, L.s);
+    L.scales = digit_scales(ctx, A, B);
+  }
   if (!sync_sizes) L.dg = L.scales && digit_entries(ctx, A, B, L.s);
   const bool use_graph = o.graph && !sync_sizes;
   L.prof = ctx->prof && !use_graph;
@@ -1318,6 +1360,7 @@ static int run_multiply(bsm_ctx ctx, double alpha, bsm_mat A, bsm_mat B, double 
   CK(cudaEventRecord(ctx->slot_ev[slot], L.s));
   CK(cudaEventRecord(ctx->ev_last, L.s));
   if (L.s != ctx->stream) CK(cudaStreamWaitEvent(ctx->stream, ctx->ev_last, 0));
+  if (hold) hold->done = true;
   return BSM_OK;
 }
 
@@ -1392,7 +1435,6 @@ const char *bsm_last_cuda_error(void) { return g_cuda_err; }
 int bsm_ctx_create(int device, bsm_ctx *out) {
   if (!out) return BSM_ERR_INVALID_ARG;
   *out = nullptr;
-  t_ctx = nullptr;
   int ndev = 0;
   CK(cudaGetDeviceCount(&ndev));
   if (device < 0 || device >= ndev) return BSM_ERR_INVALID_ARG;
@@ -1465,6 +1507,11 @@ int bsm_ctx_create(int device, bsm_ctx *out) {
     bsm_ctx_destroy(ctx);
     return rc;
   }
+  {
+    std::lock_guard<std::mutex> list(g_ctx_mu);
+    ctx->next_ctx = g_ctxs;
+    g_ctxs = ctx;
+  }
   *out = ctx;
   return BSM_OK;
 }
@@ -1473,6 +1520,14 @@ int bsm_mat_destroy(bsm_mat m);
 
 int bsm_ctx_destroy(bsm_ctx ctx) {
   if (!ctx) return BSM_ERR_INVALID_ARG;
+  {
+    std::lock_guard<std::mutex> list(g_ctx_mu);
+    for (bsm_ctx *c = &g_ctxs; *c; c = &(*c)->next_ctx)
+      if (*c == ctx) {
+        *c = ctx->next_ctx;
+        break;
+      }
+  }
   cudaSetDevice(ctx->device);
   if (ctx->stream) cudaStreamSynchronize(ctx->stream);
   if (ctx->up_stream) cudaStreamSynchronize(ctx->up_stream);

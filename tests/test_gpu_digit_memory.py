@@ -78,3 +78,66 @@ def test_each_buffer_of_the_workspace_refused_in_turn(bsm_lib):
     # without all of it the packed kernel, bit for bit; in the end the digits
     assert out["same"][0] and not out["same"][-1]
     assert max(out["off"]) <= 1e-15
+
+
+# What a second context can have before and after the first one has taken digits.
+TWO = r"""
+A = banded(8000, 9)
+with Context(0) as one, Context(0) as two:
+    dA, dC = one.from_blocks(A), one.empty(A.row_sizes, A.col_sizes)
+    want = [multiply(one, dA, dC, BSM_FP64_PK12) for _ in range(2)][1]  # both of C's buffers
+    room, off = [], []
+    for _ in range(2):
+        held = ballast(two, 256 << 10)
+        for m in held:
+            m.destroy()
+        room.append(len(held))
+        off.append(H.rel_frobenius(multiply(one, dA, dC), want))
+print(json.dumps(dict(room=room, off=off)))
+"""
+
+
+def test_another_context_gets_the_memory_of_the_digits(bsm_lib):
+    out = child(TWO, 48 << 20)
+    # all of it: the workspace is twice 64 bytes a value, 20 pieces of 256 KiB each
+    assert out["room"][1] >= out["room"][0] - 1
+    assert max(out["off"]) <= 1e-15
+
+
+# Two threads, each with a context of its own, at the cap: one takes the other's digits
+# back whenever its matrices need the room.
+THREADS = r"""
+import threading
+bad = []
+
+def work(seed):
+    rng = np.random.default_rng(seed)
+    with Context(0) as ctx:
+        for n in [2000, 4000, 3000, 6000, 1000, 5000] * 6:
+            A = banded(n, 9)
+            A.values[:] = rng.standard_normal(len(A.values))
+            try:
+                dA, dC = ctx.from_blocks(A), ctx.empty(A.row_sizes, A.col_sizes)
+                want = multiply(ctx, dA, dC, BSM_FP64_PK12)
+                for _ in range(3):
+                    off = H.rel_frobenius(multiply(ctx, dA, dC), want)
+                    if not off <= 1e-15:
+                        bad.append((seed, n, off))
+            except BsmError as e:
+                if e.name != "NOMEM":
+                    bad.append((seed, n, e.name))
+            dA.destroy()
+            dC.destroy()
+
+threads = [threading.Thread(target=work, args=(s,)) for s in (1, 2)]
+for t in threads:
+    t.start()
+for t in threads:
+    t.join()
+print(json.dumps(bad))
+"""
+
+
+@pytest.mark.parametrize("cap", [28, 36, 48])
+def test_threads_take_digits_from_each_other(bsm_lib, cap):
+    assert child(THREADS, cap << 20) == []
