@@ -28,6 +28,7 @@
 //   dg:  the products on the tensor cores, from digits of the operands (below).
 // All take an optional work list (C block indices, e.g. one shape class) and
 // its [begin, end) range in device memory.
+#include <algorithm>
 #include <cstdlib>
 
 #include "bsm_internal.h"
@@ -1382,6 +1383,12 @@ __global__ void __launch_bounds__(kDgWarps * 32, kDgBlocksPerSm)
   }
 }
 
+// The tiles of a C block of m x n, at most (block sizes may be anything below 2^31).
+static int tiles_of(int m, int n, int tm, int tn) {
+  const int64_t t = (((int64_t)m + tm - 1) / tm) * (((int64_t)n + tn - 1) / tn);
+  return (int)std::min<int64_t>(t, INT32_MAX);
+}
+
 cudaError_t launch_numeric_fp64(int variant, DevMat A, DevMat B, DevOut C, DevMat Cin,
                                 double alpha, double beta, DevWs ws, const DevStatus *st,
                                 const int32_t *items, const int64_t *seg, int grid,
@@ -1390,8 +1397,7 @@ cudaError_t launch_numeric_fp64(int variant, DevMat A, DevMat B, DevOut C, DevMa
   switch (variant) {
     case kFp64Dg:
       k_numeric_fp64_dg<<<grid, kDgWarps * 32, 0, stream>>>(
-          A, B, C, Cin, alpha, beta, ws, st, items, seg, work, *digits,
-          ((max_m + 15) / 16) * ((max_n + 7) / 8));
+          A, B, C, Cin, alpha, beta, ws, st, items, seg, work, *digits, tiles_of(max_m, max_n, 16, 8));
       break;
     case kFp64G8: {
       const int mr = max_m <= 4 ? 4 : max_m <= 6 ? 6 : 8;
@@ -1431,7 +1437,7 @@ cudaError_t launch_numeric_fp64(int variant, DevMat A, DevMat B, DevOut C, DevMa
       // digits: the blocks that the digit kernel left, tile by tile
       k_numeric_fp64_pk<12><<<grid, kPkWarps * 32, pk_smem_bytes(), stream>>>(
           A, B, C, Cin, alpha, beta, ws, st, items, seg, work,
-          digits ? ((max_m + kPkTile - 1) / kPkTile) * ((max_n + kPkTile - 1) / kPkTile) : 0);
+          digits ? tiles_of(max_m, max_n, kPkTile, kPkTile) : 0);
       break;
     case kFp64Pk16:
       k_numeric_fp64_pk<16><<<grid, kPkWarps * 32, pk_smem_bytes(), stream>>>(
