@@ -147,16 +147,20 @@ struct PinnedPool {
     const size_t step = (size_t)1 << (p - 3);
     return (b + step - 1) & ~(step - 1);
   }
-  // at_hand: only a block that is there already (else null)
+  // at_hand: only a block that is there already (else null). The lock covers the lists
+  // alone: page-locking a large block takes tens of milliseconds, for which nobody else
+  // has to wait.
   void *get(size_t bytes, bool at_hand = false) {
     const size_t cls = size_class(bytes);
-    std::lock_guard<std::mutex> lk(mu);
-    auto it = free_blocks.find(cls);
-    if (it != free_blocks.end()) {
-      void *p = it->second;
-      free_blocks.erase(it);
-      cached -= cls;
-      return p;
+    {
+      std::lock_guard<std::mutex> lk(mu);
+      auto it = free_blocks.find(cls);
+      if (it != free_blocks.end()) {
+        void *p = it->second;
+        free_blocks.erase(it);
+        cached -= cls;
+        return p;
+      }
     }
     void *p = nullptr;
     if (at_hand) return p;
@@ -164,21 +168,24 @@ struct PinnedPool {
       cudaGetLastError();
       return nullptr;
     }
+    std::lock_guard<std::mutex> lk(mu);
     block_size[p] = cls;
     return p;
   }
   void put(void *p) {
     if (!p) return;
-    std::lock_guard<std::mutex> lk(mu);
-    auto it = block_size.find(p);
-    if (it == block_size.end()) return;
-    if (cached + it->second <= kPinnedCap) {
-      free_blocks.emplace(it->second, p);
-      cached += it->second;
-    } else {
+    {
+      std::lock_guard<std::mutex> lk(mu);
+      auto it = block_size.find(p);
+      if (it == block_size.end()) return;
+      if (cached + it->second <= kPinnedCap) {
+        free_blocks.emplace(it->second, p);
+        cached += it->second;
+        return;
+      }
       block_size.erase(it);
-      cudaFreeHost(p);
     }
+    cudaFreeHost(p);
   }
   void clear() {
     std::lock_guard<std::mutex> lk(mu);
@@ -533,7 +540,9 @@ static void worker_loop(bsm_server s, int lane) {
     s->cv.notify_all();  // a head that waited for memory may fit now
     if (!heap.empty()) {  // the next inputs of these sizes find one
       lk.unlock();
-      for (size_t b : heap) s->pinned.put(s->pinned.get(b));
+      std::vector<void *> blocks;
+      for (size_t b : heap) blocks.push_back(s->pinned.get(b));
+      for (void *p : blocks) s->pinned.put(p);
       lk.lock();
     }
   }
@@ -644,8 +653,10 @@ static int submit_request(bsm_server s, int32_t nbrows, const int32_t *sizes, in
   if (borrow) {
     r->in_vals = values;
   } else {
-    // a small copy goes to the heap rather than wait for a new page-locked block, which
-    // may wait for a lane that is allocating a large result's (tens of milliseconds)
+    // a small copy takes a page-locked block only if one is at hand, else the heap: a new
+    // block may wait for a lane that is page-locking a large result's (1 GiB: 35 ms). The
+    // heap does too if it has to grow meanwhile (the kernel's lock on the address space),
+    // so the lane leaves a block for every input that found none.
     const size_t bytes = 8 * (size_t)std::max<int64_t>(nv, 1);
     r->vals = static_cast<double *>(s->pinned.get(bytes, bytes <= kHeapInput));
     if (!r->vals && bytes <= kHeapInput) {
