@@ -137,9 +137,9 @@ typedef struct {
                           products up in exact integers, 43 of 64 digit pairs of each, then
                           rounds to FP64 (once for the products of one magnitude, in
                           steps of 2^8). What that loses is bounded for every element:
-                          C blocks with an element where it may be more than (4 sqrt(N) - 2)
-                          2^-53 of the sum of its absolute products (N terms; FP64 FMAs
-                          lose up to N 2^-53 of it), and those with an operand that such an
+                          C blocks with an element where it may be more than 3 sqrt(N) 2^-53
+                          of the sum of its absolute products (N terms; FP64 FMAs lose up
+                          to N 2^-53 of it), and those with an operand that such an
                           image does not hold (infinities, NaN, scales beyond 2^+-300, rows
                           of widely different size in one block) are left to
                           the packed kernel. It takes device memory for the images,

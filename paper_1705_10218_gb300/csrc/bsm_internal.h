@@ -97,8 +97,7 @@ struct DevStatus {
 // left operand; its columns as the rows of a right one) is ceil(s / 8) octets of
 // 4 units for each row, row after row: as much as its FP64 values, with k up to a
 // multiple of 8. Block b's units start at kDigitZeros + (blk_off[b] * mul >> 6) +
-// b * pad; the units before are zeros. meta[b]: the first unit, and the fields below
-// (octets in the low 16 bits).
+// b * pad; the units before are zeros. meta[b]: the first unit, and the fields below.
 // What is lost: half a unit of X for each value, and the digit pairs (i, j) with
 // i + j > 8 of each product. Values far below the scale keep few bits of their own, so
 // the digit kernel bounds both for every element of C against the sum of its absolute
@@ -111,15 +110,16 @@ struct DevStatus {
 constexpr int kDigits = 8;
 constexpr int kDigitZeros = 64;
 constexpr uint32_t kDigitOutside = 1u << 31;
-// fields of meta[b].y: the class; by how many bits (0 to 7) every row of the block stays
-// below its scale less the class; the zeros that fill up the last octet
-constexpr int kDigitClassAt = 16, kDigitGapAt = 24, kDigitPadAt = 27;
+// fields of meta[b].y: the octets (13 bits), the zeros that fill up the last one (3), the
+// class (6), and the largest sum of a row's absolute values, in units of its scale less the
+// class (7, digit_sum_of)
+constexpr int kDigitPadAt = 13, kDigitClassAt = 16, kDigitSumAt = 22;
 // How far a row may lie below its block's class before all C blocks of the block are FP64
 // FMAs'. A wider range keeps more C blocks on the tensor cores: two sign iterations of 192
 // water molecules 18.6 ms at 9, 15.3 at 11, 14.4 at 12, 13 and 15.
 constexpr int kDigitRange = 12;
 constexpr int kDigitMaxRows = 128;
-constexpr int kDigitMaxOctets = 0xFFFF;
+constexpr int kDigitMaxOctets = 0x1FFF;
 constexpr int kDigitMaxClass = 60;
 // exponent fields (of the row's largest value) that have a scale
 constexpr int kDigitExpLo = 722, kDigitExpHi = 1322;

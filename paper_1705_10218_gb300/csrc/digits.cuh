@@ -31,6 +31,22 @@ __device__ __forceinline__ uint64_t digit_word(double x, int field) {
   return (b < 0 ? (uint64_t)0 - f : f) + bias;
 }
 
+// |X| in units of 2^48, rounded up.
+__device__ __forceinline__ int digit_top(uint64_t word) {
+  const int64_t x = (int64_t)(word - 0x8080808080808080ull);
+  return (int)((uint64_t)((x < 0 ? -x : x) + ((1ll << 48) - 1)) >> 48);
+}
+
+// A sum of these (below 2^30) over 2^14 in 7 bits: rounded up to two bits behind the leading
+// one, as an FP32 number's exponent (2^-15, which stands for less too, to 2^16) and mantissa.
+__device__ __forceinline__ uint32_t digit_sum_code(uint32_t sum) {
+  const float f = fmaxf(__uint2float_ru(sum) * 0x1p-14f, 0x1p-15f);
+  return ((__float_as_uint(f) + (1u << 21) - 1) >> 21) - (112u << 2);
+}
+__device__ __forceinline__ float digit_sum_of(uint32_t code) {
+  return __uint_as_float((code + (112u << 2)) << 21);
+}
+
 __device__ __forceinline__ int digit_field(double x) {
   const int f = (int)(((uint32_t)__double2hiint(x) >> 20) & 0x7FF);
   return f ? f : (x != 0.0 ? 1 : 0);
@@ -53,7 +69,7 @@ __device__ __forceinline__ uint4 digit_unit(uint64_t x, uint64_t y) {
 }
 
 // One layout of a block: element (r, k) at r * rs + k * ks, `rows` rows, k up to s
-// (rs = 1, ks = rows; or rs = s, ks = 1). seg: kDigitMaxRows words of the warp's own.
+// (rs = 1, ks = rows; or rs = s, ks = 1). seg: 2 kDigitMaxRows words of the warp's own.
 __device__ __forceinline__ void digit_layout(const double *__restrict__ x, int rows, int s, int rs,
                                              int ks, const DigitSide &o, int64_t first, int64_t b,
                                              int64_t base, int32_t *seg, int lane) {
@@ -61,10 +77,12 @@ __device__ __forceinline__ void digit_layout(const double *__restrict__ x, int r
   const int32_t *expo = o.expo + first;
   uint4 *units = o.units + base;
   bool outside = rows > kDigitMaxRows || octets > kDigitMaxOctets;
-  int cls = 0, gap = 0;
+  int cls = 0;
+  uint32_t most = 0;  // the largest sum of a row's absolute values, in 2^-14 of its scale
   if (!outside) {
     // the largest exponent field of each row of the block
-    for (int r = lane; r < rows; r += 32) seg[r] = 0;
+    int32_t *sum = seg + kDigitMaxRows;
+    for (int r = lane; r < rows; r += 32) seg[r] = sum[r] = 0;
     __syncwarp();
     const int len = rows * s;
     for (int z = lane; z < len; z += 32) {  // in the order of the values
@@ -81,7 +99,6 @@ __device__ __forceinline__ void digit_layout(const double *__restrict__ x, int r
     }
     room = __reduce_min_sync(0xffffffffu, room);
     cls = room >> 3;
-    gap = room & 7;
     for (int r = lane; r < rows; r += 32)
       outside |= seg[r] && seg[r] < expo[r] - 8 * cls - kDigitRange;
     outside = __any_sync(0xffffffffu, outside);
@@ -92,17 +109,21 @@ __device__ __forceinline__ void digit_layout(const double *__restrict__ x, int r
       const double v0 = (2 * q < s) ? __ldg(p) : 0.0;
       const double v1 = (2 * q + 1 < s) ? __ldg(p + ks) : 0.0;
       const int field = seg[r] ? expo[r] - 8 * cls : 0;
-      units[((q >> 2) * rows + r) * 4 + (q & 3)] = digit_unit(digit_word(v0, field), digit_word(v1, field));
+      const uint64_t w0 = digit_word(v0, field), w1 = digit_word(v1, field);
+      units[((q >> 2) * rows + r) * 4 + (q & 3)] = digit_unit(w0, w1);
+      atomicAdd(&sum[r], digit_top(w0) + digit_top(w1));
     }
     __syncwarp();
+    for (int r = lane; r < rows; r += 32) most = max(most, (uint32_t)sum[r]);
+    most = __reduce_max_sync(0xffffffffu, most);
   }
   outside = __any_sync(0xffffffffu, outside);
   if (lane == 0)
     o.meta[b] = make_uint2((uint32_t)base,
                            outside ? kDigitOutside
-                                   : (uint32_t)octets | (uint32_t)cls << kDigitClassAt |
-                                         (uint32_t)gap << kDigitGapAt |
-                                         (uint32_t)(8 * octets - s) << kDigitPadAt);
+                                   : (uint32_t)octets | (uint32_t)(8 * octets - s) << kDigitPadAt |
+                                         (uint32_t)cls << kDigitClassAt |
+                                         digit_sum_code(most) << kDigitSumAt);
 }
 
 // The digits of M as a left and / or right operand, one warp per block.

@@ -860,15 +860,15 @@ __global__ void __launch_bounds__(kPkWarps * 32, 2)
 // (7.9e-16); amorphous of 200 atoms 4.6e-17 (7.3e-17), packed 1.0e-15 (1.7e-15); rows of
 // unlike scales in blocks of 1 to 33 5.9e-17 (4.4e-16), packed 4.0e-16 (9.6e-15). Largest
 // error of an element against the sum of its absolute products: ragged blocks 2.7e-16, sign
-// iterates of 64 water molecules 2.4, 2.7 and 4.3e-15, water 1.0e-16, amorphous 1.0e-16;
+// iterates of 64 water molecules 0.4, 2.4 and 0.8e-15, water 1.0e-16, amorphous 1.0e-16;
 // packed 5.1e-16; 2.4, 3.0 and 4.4e-15; 2.0e-15; 3.1e-15.
 //
 // Why: the FP64 pipe does 2 FMA per clock and SM, mma.sync on FP16 1024, and 43
 // digit pairs stand for one product. (FP8 and INT8 mma.sync are emulated or slow on
 // this part: 3.8 and 16 clocks per m16n8k32 and SM, FP16 m16n8k16 2.0.) Numeric
-// phase, packed kernel -> this one: water of 2048 molecules 47.7 -> 23.4 ms (21.3 without
-// dg_enough, 0.8 of it the packed kernel's on the 8% of the C blocks that it leaves),
-// amorphous of 1024 atoms 67.9 -> 22.8 (22.0), 64 x 64 full blocks of 32 15.7 -> 2.0. What
+// phase, packed kernel -> this one: water of 2048 molecules 47.7 -> 23.3 ms (21.3 without
+// dg_enough; 0.8 is the packed kernel's on the 8% of the C blocks that it leaves),
+// amorphous of 1024 atoms 67.9 -> 22.7 (22.0), 64 x 64 full blocks of 32 15.7 -> 2.0. What
 // bounds it: the MMA pipe (0.49 of the clocks of the first) and the instructions beside
 // it, which do not hide behind the MMAs whatever the number of warps (with 16, 20 and 24
 // per SM 21.4, 21.9 and 22.2 ms): left out one at a time, the digits' conversion is
@@ -937,12 +937,13 @@ __device__ __forceinline__ double dg_scaled(double v, int e) {
   return v * __hiloint2double((1023 + half) << 20, 0) * __hiloint2double((1023 + e - half) << 20, 0);
 }
 
-// Fields of a block's metadata: its class, its gap, its values of k.
-__device__ __forceinline__ int dg_class(uint2 x) { return (int)(x.y >> kDigitClassAt & 0xFF); }
-__device__ __forceinline__ int dg_gap(uint2 x) { return (int)(x.y >> kDigitGapAt & 7); }
+// Fields of a block's metadata: octets, values of k, class, sum of a row.
+__device__ __forceinline__ int dg_octets(uint2 x) { return (int)(x.y & kDigitMaxOctets); }
 __device__ __forceinline__ int dg_length(uint2 x) {
-  return 8 * (int)(x.y & 0xFFFF) - (int)(x.y >> kDigitPadAt & 7);
+  return 8 * dg_octets(x) - (int)(x.y >> kDigitPadAt & 7);
 }
+__device__ __forceinline__ int dg_class(uint2 x) { return (int)(x.y >> kDigitClassAt & 0x3F); }
+__device__ __forceinline__ uint32_t dg_sum_code(uint2 x) { return x.y >> kDigitSumAt & 0x7F; }
 
 // A word of a unit (digits 2 i and 2 i + 1 of two values) as the two MMA registers.
 __device__ __forceinline__ uint32_t dg_even(uint32_t w) { return digit_half2(w, 0x4140); }
@@ -1023,7 +1024,7 @@ __device__ __forceinline__ int dg_tile(const Digits &dg, const int2 *__restrict_
       const bool mine = in && cls == now;
       todo &= ~__ballot_sync(0xffffffffu, mine);
       // its octets' end, and its units less its first slot's
-      const int octets = mine ? (int)(xa.y & 0xFFFF) : 0;
+      const int octets = mine ? dg_octets(xa) : 0;
       int incl = octets;
 #pragma unroll
       for (int d = 1; d < 32; d <<= 1) {
@@ -1093,24 +1094,24 @@ __device__ __forceinline__ int dg_tile(const Digits &dg, const int2 *__restrict_
   }
 }
 
-// Whether the digits hold enough of a C block. A product's value of k loses at most
-// 2^-63 (2^-gb + 2^-ga) + 2^-67.4 in units of W, the product of the row's and the
-// column's scale less the classes (half a unit of X each, beside values below 2^-ga or
-// 2^-gb of the scale, and the digit pairs beyond kDgDiag). The sum of that over the C block
-// may be at most (4 sqrt(N) - 2) 2^-53 of the element's sum of absolute products, N the
-// block's number of values of k. That is no more than (N + 2) 2^-53, where FP64 FMAs have
-// N 2^-53 in the worst case; and the losses being independent, what is lost of elements at
-// this very limit is about what FP64 FMAs lose (normal values of one size; root mean
-// square in units of 2^-53 of that sum, the rounding of the result with it, where FP64 has
-// 0.4 to 0.5: N = 5 0.31, 13 0.37, 50 0.33, 200 0.20), of most elements far less.
+// Whether the digits hold enough of a C block. A product of s values of k loses at most
+// 2^-63 (sa + sb) + 2^-67.4 s in units of W, the product of the row's and the column's scale
+// less the classes: half a unit of X for each value of one side beside the other side's
+// values, whose absolute sum over k is at most sa (sb) of the scale, and the digit pairs
+// beyond kDgDiag. Over the C block, N values of k in all, the first may come to sqrt(N) 2^-53
+// of the element's sum of absolute products, the second to 3 sqrt(N) 2^-53 (of both, the
+// fractions of their limits to 1). FP64 FMAs lose up to N 2^-53 of that sum. What they lose of
+// ordinary elements is 0.4 2^-53 of it where terms are alike, as the second, being a sum of
+// many independent parts, at its limit; and 0.3 sqrt(N) 2^-53 where one term is most of the sum,
+// as where the first comes near its limit.
 // The sum of absolute products is bounded from below by the two top digits t of both
 // values (2^14 of the scale): t_a t_b less the digits' rounding, added up by one MMA for
 // every 16 k. Any part of the products will do, so those of the largest scales go first and
 // it ends when every element has enough, mostly after the first one or two. C blocks that
 // have not enough with all of theirs are left to the packed kernel.
-// 2^-ga + 2^-gb
-__device__ __forceinline__ float dg_sizes(uint2 a, uint2 b) {
-  return __int_as_float((127 - dg_gap(a)) << 23) + __int_as_float((127 - dg_gap(b)) << 23);
+// sa + sb
+__device__ __forceinline__ float dg_sums(uint2 a, uint2 b) {
+  return digit_sum_of(dg_sum_code(a)) + digit_sum_of(dg_sum_code(b));
 }
 // the weight of products whose classes add up to d more than the least (2 and more: at most this)
 __device__ __forceinline__ float dg_weight(int d) {
@@ -1122,7 +1123,7 @@ __device__ __forceinline__ float dg_weight(int d) {
 __device__ __forceinline__ float dg_need(const Digits &dg, const int2 *__restrict__ prods, int np,
                                          uint2 ma, uint2 mb, int &least, int lane) {
   auto loss = [&](uint2 a, uint2 b) {
-    return (float)dg_length(a) * (0x1p18f * dg_sizes(a, b) + 12400.0f);
+    return 3 * 0x1p18f * dg_sums(a, b) + 12400.0f * (float)dg_length(a);
   };
   // the lane's products: their least class and their loss at its weight
   int cls = 1 << 10, n = 0;
@@ -1149,7 +1150,7 @@ __device__ __forceinline__ float dg_need(const Digits &dg, const int2 *__restric
 #pragma unroll
   for (int d = 16; d; d >>= 1) sum += __shfl_xor_sync(0xffffffffu, sum, d);
   // t carries 11 bits, the sums 24, the root and the quotient 20: 1% covers them
-  return __fdividef(1.01f * sum, 4.0f * (float)n * rsqrtf((float)n) - 2.0f);
+  return 1.01f / 3.0f * sum * rsqrtf((float)n);
 }
 
 __device__ __forceinline__ uint32_t dg_top(uint32_t w) {  // |256 d_0 + d_1| of two values
@@ -1157,6 +1158,11 @@ __device__ __forceinline__ uint32_t dg_top(uint32_t w) {  // |256 d_0 + d_1| of 
   asm("fma.rn.f16x2 %0, %0, %1, %2;\n" : "+r"(h) : "r"(0x5C005C00u), "r"(dg_odd(w)));
   return h & 0x7FFF7FFFu;
 }
+
+// Products that are looked at before a tile may be given up: operands whose values cancel
+// along k by 2^-10 to 2^10 (water of 512 molecules, every C block left to the packed kernel)
+// 14.2 ms with all products looked at, 13.1 so, 12.2 for the packed kernel alone.
+constexpr int kDgLook = 3;
 
 // Whether each element of a tile reaches `need`: rows from r0 of A and columns from c0 of
 // B, tm x tn of up to 16 x 16 (the left side's registers serve both halves of the columns).
@@ -1170,10 +1176,11 @@ __device__ __forceinline__ bool dg_enough(const Digits &dg, const int2 *__restri
   const int low = (min(g + 8, tm - 1) - min(g, tm - 1)) * 4;
   const int right = (min(g + 8, tn - 1) - min(g, tn - 1)) * 4;
   float sum[2][4] = {};
+  int seen = 0;
   for (int pb = 0;;) {
     const int above = dg_class(ma) + dg_class(mb) - least;
     uint32_t key = pb + lane < np && above <= 1
-                       ? (uint32_t)(8 * above + dg_gap(ma) + dg_gap(mb)) << 5 | lane
+                       ? (32 * above + 254 - dg_sum_code(ma) - dg_sum_code(mb)) << 5 | lane
                        : ~0u;
 #pragma unroll 1
     for (;;) {
@@ -1183,7 +1190,7 @@ __device__ __forceinline__ bool dg_enough(const Digits &dg, const int2 *__restri
       if (lane == p) key = ~0u;
       const uint2 xa = make_uint2(__shfl_sync(0xffffffffu, ma.x, p), __shfl_sync(0xffffffffu, ma.y, p));
       const uint2 xb = make_uint2(__shfl_sync(0xffffffffu, mb.x, p), __shfl_sync(0xffffffffu, mb.y, p));
-      const int octets = (int)(xa.y & 0xFFFF);
+      const int octets = dg_octets(xa);
       float acc[2][4] = {};
 #pragma unroll 1
       for (int o = 0; o < octets; o += 2) {
@@ -1204,15 +1211,18 @@ __device__ __forceinline__ bool dg_enough(const Digits &dg, const int2 *__restri
       }
       const float w = dg_weight(dg_class(xa) + dg_class(xb) - least);
       // t may be 0.503 above the value: what that adds at most
-      need += w * (float)dg_length(xa) * (8260.0f * dg_sizes(xa, xb) + 0.3f);
-      bool enough = true;
+      need += w * (8260.0f * dg_sums(xa, xb) + 0.3f * (float)dg_length(xa));
+      float some = INFINITY;  // the least sum of the lane's elements
 #pragma unroll
       for (int e = 0; e < 4; e++) {
         sum[0][e] += w * acc[0][e];
         sum[1][e] += w * acc[1][e];
-        enough = enough && sum[0][e] >= need && (tn <= 8 || sum[1][e] >= need);
+        some = fminf(some, tn <= 8 ? sum[0][e] : fminf(sum[0][e], sum[1][e]));
       }
-      if (__all_sync(0xffffffffu, enough)) return true;
+      if (__all_sync(0xffffffffu, some >= need)) return true;
+      // not with four times as much from each of the others, which are smaller: no use going on
+      if (++seen >= kDgLook &&
+          __any_sync(0xffffffffu, some * (float)(4 * np) < need * (float)seen)) return false;
     }
     pb += 32;
     if (pb >= np) return false;

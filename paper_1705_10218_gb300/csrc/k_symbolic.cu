@@ -737,7 +737,7 @@ __global__ void __launch_bounds__(THREADS)
   // work that fits between the latency-bound rows of other thread blocks
   if (dg.a.units) {
     __syncthreads();
-    int32_t *seg = reinterpret_cast<int32_t *>(smem_bits) + warp * kDigitMaxRows;
+    int32_t *seg = reinterpret_cast<int32_t *>(smem_bits) + warp * 2 * kDigitMaxRows;
     const bool same = A.vals == B.vals;
     // few rows: from the last thread block on, which has none, and one block of each, so
     // that few blocks are on as many SMs; else consecutive blocks in a thread block
@@ -756,7 +756,7 @@ cudaError_t launch_symbolic_fill(DevMat A, DevMat B, DevMat Cin, int use_cin, do
   const int mw = (mask_words > 0 && mask_words < kMaskWords) ? mask_words : kMaskWords;
   size_t smem = ((size_t)max(nwords, 1) * 2 + mw) * sizeof(uint32_t);
   const int threads = sym_threads(A.nbr, nsm);
-  if (digits) smem = max(smem, sizeof(int32_t) * kDigitMaxRows * (threads / 32));
+  if (digits) smem = max(smem, sizeof(int32_t) * 2 * kDigitMaxRows * (threads / 32));
   // one wave of resident blocks (rows taken in a grid stride): more resident
   // blocks hide more of each row's load latency, a second wave only adds a tail
   int per_sm = 0;
