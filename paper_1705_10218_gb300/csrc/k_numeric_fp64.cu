@@ -299,14 +299,16 @@ __global__ void __launch_bounds__(kSWarps * 32, MINB)
 // covers 256 contiguous bytes. A lane's own columns would be 8 bytes apart from
 // every other store, which the link to host memory (the second destination) takes
 // at 25 GB/s of its 193.
-// Measured, 20000 atoms, 2.2 M C blocks of 6, numeric phase with a second
-// destination in host memory: 26.1 -> 3.40 ms, bound by the link (637 MB); without
-// one 1.40 -> 1.33, bound by the FP64 pipe (0.68 without its instructions): the
-// multiplication by alpha, on the few lanes of one group at a time, moved to the
-// stores, where it is on all lanes and not there for alpha = 1 (another alpha: 1.40 ->
-// 1.48; as exponent arithmetic for powers of two no less). 16 warps per SM with runs of
-// 30 blocks: 24 warps with runs of 15 took 0.15 ms more, 32 0.5 (the groups idle at a
-// run's end).
+// Measured, 20000 atoms, 2.2 M C blocks of 6, numeric phase with a second destination in
+// host memory: 26.1 -> 3.40 ms, bound by the link (637 MB); without one 1.40 -> 1.32, bound
+// by the FP64 pipe (0.68 without its instructions), if nothing is left to do at the stores
+// (alpha = 1, no C_in). 16 warps per SM with runs of 30 blocks: 24 warps with runs of 15 took
+// 0.15 ms more, 32 0.5 (the groups idle at a run's end).
+// g8_direct has no runs: each group stores its blocks itself, in the iteration that closes
+// them. It is the faster one without a second destination where the stores have work or the
+// blocks are up to 4 x 4 (gathered -> direct, blocks of 4, 6, 8): alpha other than 1 0.59 ->
+// 0.51, 1.47 -> 1.40, 1.73 -> 1.62 ms; with C_in 0.74 -> 0.63, 1.77 -> 1.60, 1.99 -> 1.82; plain
+// 0.53 -> 0.52, but 1.32 -> 1.40, 1.58 -> 1.62. Both give the same bits.
 // A C block of more than MR rows or GS columns (only when the kernel is forced on
 // larger blocks) is done in column and row chunks by its group and stored directly.
 // ----------------------------------------------------------------------------
@@ -500,6 +502,104 @@ __global__ void __launch_bounds__(kG8Warps * 32, kG8BlocksPerSm)
         }
     }
     __syncwarp();
+  }
+}
+
+// The groups of a warp are independent streams: each takes kG8Grab C blocks at a time from
+// the work counter and walks their products one step per loop iteration, closing a C block
+// (epilogue, next block's metadata) in the iteration that ends it, so a group whose block
+// has more products does not hold the other groups at a loop exit. The latency of each C
+// block's chain of dependent loads is hidden by the many independent blocks in flight.
+constexpr int kG8DirectBlocksPerSm = 4;
+constexpr int kG8Grab = 16;  // C blocks per group and grab
+
+template <int MR, int GS>
+__global__ void __launch_bounds__(kG8Warps * 32, kG8DirectBlocksPerSm)
+    k_numeric_fp64_g8_direct(DevMat A, DevMat B, DevOut C, DevMat Cin, double alpha, double beta,
+                             DevWs ws, const DevStatus *st, const int32_t *items,
+                             const int64_t *seg, unsigned long long *work) {
+  if (st->overflow) return;
+  const int lane = threadIdx.x & 31;
+  const int grp = lane / GS, cl = lane - grp * GS;
+  if (grp >= 32 / GS) return;  // lanes past the last whole group
+  const unsigned gmask = ((1u << GS) - 1u) << (GS * grp);
+  int64_t wb, we;
+  work_range(st, seg, wb, we);
+
+  // the group's current grab [w, wend) and C block (group-uniform state)
+  int64_t w = 0, wend = 0, p = 0, p1 = 0, cbase = 0;
+  int m = 0, n = 0;
+  const double *cinv = nullptr;
+  double acc[MR];
+  auto next_block = [&]() -> bool {
+    if (w >= wend) {
+      unsigned long long got = 0;
+      if (cl == 0) got = atomicAdd(work, (unsigned long long)kG8Grab);
+      w = wb + (int64_t)__shfl_sync(gmask, got, GS * grp);
+      wend = (w + kG8Grab < we) ? w + kG8Grab : we;
+      if (w >= we) return false;
+    }
+    const int64_t g = items ? items[w] : w;
+    w++;
+    m = C.row_sizes[C.blk_row[g]];
+    n = C.col_sizes[C.col_idx[g]];
+    p = ws.prod_ptr[g];
+    p1 = ws.prod_ptr[g + 1];
+    const int cin = ws.c_cin[g];
+    cinv = (cin >= 0) ? Cin.vals + Cin.blk_off[cin] : nullptr;
+    cbase = C.blk_off[g];
+#pragma unroll
+    for (int r = 0; r < MR; r++) acc[r] = 0.0;
+    return true;
+  };
+  // rows [r0, r0 + MR) of column c of product q, added to acc
+  auto product = [&](int64_t q, int c, int r0) {
+    const int2 pr = ws.prods[q];
+    const double *Ab = A.vals + A.blk_off[pr.x] + r0;
+    const int s = A.col_sizes[A.col_idx[pr.x]];
+    const double *Bb = B.vals + B.blk_off[pr.y] + (int64_t)c * s;
+    for (int kk = 0; kk < s; kk++) {
+      const double bv = __ldg(Bb + kk);
+      const double *a = Ab + (int64_t)kk * m;
+#pragma unroll
+      for (int r = 0; r < MR; r++)
+        if (r0 + r < m) acc[r] = fma(__ldg(a + r), bv, acc[r]);
+    }
+  };
+  // C_ij = beta * C_in_ij + alpha * S_ij for rows [r0, r0 + MR) of column c
+  auto store = [&](int c, int r0) {
+#pragma unroll
+    for (int r = 0; r < MR; r++) {
+      if (r0 + r < m) {
+        const int64_t loc = (int64_t)c * m + r0 + r;
+        double v = alpha * acc[r];
+        if (cinv) v = fma(beta, cinv[loc], v);
+        C.vals[cbase + loc] = v;
+      }
+    }
+  };
+
+  bool have = next_block();
+  while (have) {
+    if (m > MR || n > GS) {  // column and row chunks, the products once per chunk
+      for (int c = cl; c < n; c += GS)
+        for (int r0 = 0; r0 < m; r0 += MR) {
+#pragma unroll
+          for (int r = 0; r < MR; r++) acc[r] = 0.0;
+          for (int64_t q = p; q < p1; q++) product(q, c, r0);
+          store(c, r0);
+        }
+      have = next_block();
+      continue;
+    }
+    if (p < p1) {  // one product of the block (products in ascending k)
+      if (cl < n) product(p, cl, 0);
+      p++;
+    }
+    if (p >= p1) {  // the block is complete
+      if (cl < n) store(cl, 0);
+      have = next_block();
+    }
   }
 }
 
@@ -1412,9 +1512,16 @@ cudaError_t launch_numeric_fp64(int variant, DevMat A, DevMat B, DevOut C, DevMa
     case kFp64G8: {
       const int mr = max_m <= 4 ? 4 : max_m <= 6 ? 6 : 8;
       const int gs = max_n <= 4 ? 4 : max_n <= 6 ? 6 : 8;
+      const bool direct = !C.host_vals && (alpha != 1.0 || beta != 0.0 || (mr == 4 && gs == 4));
 // the shared memory is opted into here, for the one instance (it loads its code)
 #define BSM_G8(R, G)                                                                             \
   do {                                                                                           \
+    if (direct) {                                                                                \
+      k_numeric_fp64_g8_direct<R, G>                                                             \
+          <<<grid / kG8BlocksPerSm * kG8DirectBlocksPerSm, kG8Warps * 32, 0, stream>>>(          \
+              A, B, C, Cin, alpha, beta, ws, st, items, seg, work);                              \
+      break;                                                                                     \
+    }                                                                                            \
     const cudaError_t e = cudaFuncSetAttribute(                                                  \
         k_numeric_fp64_g8<R, G>, cudaFuncAttributeMaxDynamicSharedMemorySize,                    \
         (int)g8_smem_bytes());                                                                   \
