@@ -308,7 +308,8 @@ __global__ void __launch_bounds__(kSWarps * 32, MINB)
 // them. It is the faster one without a second destination where the stores have work or the
 // blocks are up to 4 x 4 (gathered -> direct, blocks of 4, 6, 8): alpha other than 1 0.59 ->
 // 0.51, 1.47 -> 1.40, 1.73 -> 1.62 ms; with C_in 0.74 -> 0.63, 1.77 -> 1.60, 1.99 -> 1.82; plain
-// 0.53 -> 0.52, but 1.32 -> 1.40, 1.58 -> 1.62. Both give the same bits.
+// 0.53 -> 0.52, but 1.32 -> 1.40, 1.58 -> 1.62. Both give the same bits. Larger blocks
+// (below) are the gathering kernel's: two to four times as fast.
 // A C block of more than MR rows or GS columns (only when the kernel is forced on
 // larger blocks) is done in column and row chunks by its group and stored directly.
 // ----------------------------------------------------------------------------
@@ -552,26 +553,26 @@ __global__ void __launch_bounds__(kG8Warps * 32, kG8DirectBlocksPerSm)
     for (int r = 0; r < MR; r++) acc[r] = 0.0;
     return true;
   };
-  // rows [r0, r0 + MR) of column c of product q, added to acc
-  auto product = [&](int64_t q, int c, int r0) {
+  // column cl of product q, added to acc
+  auto product = [&](int64_t q) {
     const int2 pr = ws.prods[q];
-    const double *Ab = A.vals + A.blk_off[pr.x] + r0;
+    const double *Ab = A.vals + A.blk_off[pr.x];
     const int s = A.col_sizes[A.col_idx[pr.x]];
-    const double *Bb = B.vals + B.blk_off[pr.y] + (int64_t)c * s;
+    const double *Bb = B.vals + B.blk_off[pr.y] + (int64_t)cl * s;
     for (int kk = 0; kk < s; kk++) {
       const double bv = __ldg(Bb + kk);
       const double *a = Ab + (int64_t)kk * m;
 #pragma unroll
       for (int r = 0; r < MR; r++)
-        if (r0 + r < m) acc[r] = fma(__ldg(a + r), bv, acc[r]);
+        if (r < m) acc[r] = fma(__ldg(a + r), bv, acc[r]);
     }
   };
-  // C_ij = beta * C_in_ij + alpha * S_ij for rows [r0, r0 + MR) of column c
-  auto store = [&](int c, int r0) {
+  // C_ij = beta * C_in_ij + alpha * S_ij
+  auto store = [&]() {
 #pragma unroll
     for (int r = 0; r < MR; r++) {
-      if (r0 + r < m) {
-        const int64_t loc = (int64_t)c * m + r0 + r;
+      if (r < m) {
+        const int64_t loc = (int64_t)cl * m + r;
         double v = alpha * acc[r];
         if (cinv) v = fma(beta, cinv[loc], v);
         C.vals[cbase + loc] = v;
@@ -581,23 +582,12 @@ __global__ void __launch_bounds__(kG8Warps * 32, kG8DirectBlocksPerSm)
 
   bool have = next_block();
   while (have) {
-    if (m > MR || n > GS) {  // column and row chunks, the products once per chunk
-      for (int c = cl; c < n; c += GS)
-        for (int r0 = 0; r0 < m; r0 += MR) {
-#pragma unroll
-          for (int r = 0; r < MR; r++) acc[r] = 0.0;
-          for (int64_t q = p; q < p1; q++) product(q, c, r0);
-          store(c, r0);
-        }
-      have = next_block();
-      continue;
-    }
     if (p < p1) {  // one product of the block (products in ascending k)
-      if (cl < n) product(p, cl, 0);
+      if (cl < n) product(p);
       p++;
     }
     if (p >= p1) {  // the block is complete
-      if (cl < n) store(cl, 0);
+      if (cl < n) store();
       have = next_block();
     }
   }
@@ -1512,7 +1502,8 @@ cudaError_t launch_numeric_fp64(int variant, DevMat A, DevMat B, DevOut C, DevMa
     case kFp64G8: {
       const int mr = max_m <= 4 ? 4 : max_m <= 6 ? 6 : 8;
       const int gs = max_n <= 4 ? 4 : max_n <= 6 ? 6 : 8;
-      const bool direct = !C.host_vals && (alpha != 1.0 || beta != 0.0 || (mr == 4 && gs == 4));
+      const bool direct = !C.host_vals && max_m <= 8 && max_n <= 8 &&
+                          (alpha != 1.0 || beta != 0.0 || (mr == 4 && gs == 4));
 // the shared memory is opted into here, for the one instance (it loads its code)
 #define BSM_G8(R, G)                                                                             \
   do {                                                                                           \
