@@ -254,9 +254,12 @@ __device__ __forceinline__ void ldsm_x2(uint32_t &r0, uint32_t &r1, uint32_t add
 // columns; a warp takes a tile of up to 16 x 16:
 //   kHalf: up to 8 x 8 (the lower half of the MMA's rows repeats the upper one);
 //   kOne:  up to 16 x 8;  kTwo: up to 16 x 16.
-// The blocks of a warp's run that follow one another in C are gathered and leave in
-// 256-byte stores, which the link to host memory needs (a block at a time: 141 of its
-// 193 GB/s).
+// With a second destination in host memory the blocks of a warp's run that follow one
+// another in C are gathered and leave in 256-byte stores, which the link needs (a block at a
+// time: 141 of its 193 GB/s). Without one (DIRECT) a tile goes from the registers into C:
+// numeric phase, gathered -> direct, water of 512 molecules 3.19 -> 3.05 ms, 10000 rows with about
+// one product for each C block of 6, 13, 16, 24 1.94 -> 1.64, 0.85 -> 0.78, 0.95 -> 0.78, 2.53 ->
+// 2.35 (the ring below 2.27, 0.75, 0.75, 3.27).
 //
 // Against one bulk copy per operand and product into a ring in shared memory and
 // ldmatrix, which cost 45 clocks of an SM per copy; numeric phase: water of 1024
@@ -284,6 +287,13 @@ struct SbItem {  // a C block of a warp's run
 struct SbPiece {  // a piece of k: where row 0's lies in both operands' first planes, and
   const uint4 *a, *b;  // the distance of the planes in rows
 };
+struct SbOut {  // a tile's element (0, 0) in C and in C_in (null: none), column-major, ld rows
+  double *c;
+  const double *cin;
+  double alpha, beta;
+  int ld;
+  bool plain;  // alpha = 1 and no C_in
+};
 struct SbWarp {  // a warp's shared memory
   float2 tile[16 * 16];  // hi and lo of a tile, column-major as in C
   double stage[kSbStage];  // values of finished blocks that follow one another in C
@@ -302,12 +312,13 @@ enum SbTile { kHalf, kOne, kTwo };
 
 // One tile, into w.tile: rows l0 to l0 + tl - 1 of L, r0 to r0 + tr - 1 of R (swap: L is
 // B). a, b, pc: where the operands of product `lane` start, and its pieces of k (0: none).
-template <int PREC, SbTile TILE>
+// DIRECT: into C (out) instead.
+template <int PREC, SbTile TILE, bool DIRECT>
 __device__ __forceinline__ void sb_tile(SbWarp &w, const uint4 *a, const uint4 *b, int pc,
                                         const SbItem &it, int l0, int tl, int r0, int tr, bool swap,
                                         const DevMat &A, const DevMat &B,
                                         const uint4 *__restrict__ a_left,
-                                        const uint4 *__restrict__ b_right, int lane) {
+                                        const uint4 *__restrict__ b_right, const SbOut &out, int lane) {
   constexpr bool BF = (PREC == BSM_PREC_SPLIT_BF16X3);
   constexpr int NSL = BF ? 3 : 2, NPQ = BF ? 6 : 3, VPP = BF ? 8 : 4;
   constexpr int64_t kUnit = BF ? 3 : 2;  // pieces per FP64 value of an operand's offset
@@ -421,6 +432,24 @@ __device__ __forceinline__ void sb_tile(SbWarp &w, const uint4 *a, const uint4 *
       }
     }
   }
+  if (DIRECT) {
+#pragma unroll
+    for (int nt = 0; nt < NT; nt++)
+#pragma unroll
+      for (int x = 0; x < (TILE == kHalf ? 2 : 4); x++) {
+        const int u = g + (x >> 1) * 8, v = nt * 8 + 2 * t + (x & 1);
+        if (u >= tl || v >= tr) continue;
+        const int64_t at = swap ? (int64_t)u * out.ld + v : (int64_t)v * out.ld + u;
+        // FP32 -> FP64 is exact; hi + lo rounded once in FP64
+        double y = (double)hi[nt][x] + (double)lo[nt][x];
+        if (!out.plain) {
+          y = out.alpha * y;
+          if (out.cin) y = fma(out.beta, out.cin[at], y);
+        }
+        __stcs(out.c + at, y);
+      }
+    return;
+  }
   // the tile as it lies in C: row + rows of the tile * column
   __syncwarp();
   const int ld = swap ? tr : tl;
@@ -434,8 +463,8 @@ __device__ __forceinline__ void sb_tile(SbWarp &w, const uint4 *a, const uint4 *
   __syncwarp();
 }
 
-// sel: 0 every C block, 2 those beyond 16 x 16.
-template <int PREC>
+// sel: 0 every C block, 2 those beyond 16 x 16. DIRECT: there is no second destination.
+template <int PREC, bool DIRECT>
 __global__ void __launch_bounds__(kSbWarps * 32, kSbBlocksPerSm)
     k_numeric_split_blocks(DevMat A, DevMat B, DevOut C, DevMat Cin,
                            const uint4 *__restrict__ a_left, const uint4 *__restrict__ b_right,
@@ -451,7 +480,7 @@ __global__ void __launch_bounds__(kSbWarps * 32, kSbBlocksPerSm)
   SbWarp &w = reinterpret_cast<SbWarp *>(smem_sb)[warp];
   int64_t wb = 0, we = st->nblk_c;
   if (seg) wb = seg[0], we = seg[1];
-  double *hout = (C.host_vals && st->nnz_c <= C.host_cap) ? C.host_vals : nullptr;
+  double *hout = (!DIRECT && C.host_vals && st->nnz_c <= C.host_cap) ? C.host_vals : nullptr;
   const bool plain = (alpha == 1.0 && beta == 0.0);
   // fewer at a time where that would leave warps without work
   const int64_t warps = (int64_t)gridDim.x * kSbWarps;
@@ -526,7 +555,7 @@ __global__ void __launch_bounds__(kSbWarps * 32, kSbBlocksPerSm)
         operands();
         continue;
       }
-      const bool staged = nparts == 1 && m * n <= kSbStage;
+      const bool staged = !DIRECT && nparts == 1 && m * n <= kSbStage;
       int number = 0;
       if (held > 0 && (!staged || held + m * n > kSbStage || it.coff != first + held)) flush();
       if (held == 0) first = it.coff;
@@ -537,13 +566,17 @@ __global__ void __launch_bounds__(kSbWarps * 32, kSbBlocksPerSm)
           if (nparts > 1 && number++ % nparts != it.part) continue;
           const int tm = min(16, m - m0), tn = min(16, n - n0);
           const int l0 = swap ? n0 : m0, tl = swap ? tn : tm, r0 = swap ? m0 : n0, tr = swap ? tm : tn;
-          if (tr > 8)
-            sb_tile<PREC, kTwo>(w, ca, cb, cp, it, l0, tl, r0, tr, swap, A, B, a_left, b_right, lane);
-          else if (tl > 8)
-            sb_tile<PREC, kOne>(w, ca, cb, cp, it, l0, tl, r0, tr, swap, A, B, a_left, b_right, lane);
-          else
-            sb_tile<PREC, kHalf>(w, ca, cb, cp, it, l0, tl, r0, tr, swap, A, B, a_left, b_right, lane);
           const double *cinv = it.cin >= 0 ? Cin.vals + it.cin : nullptr;
+          const int64_t corner = (int64_t)n0 * m + m0;
+          const SbOut out{C.vals + it.coff + corner,
+                          cinv ? cinv + corner : nullptr, alpha, beta, m, plain};
+          if (tr > 8)
+            sb_tile<PREC, kTwo, DIRECT>(w, ca, cb, cp, it, l0, tl, r0, tr, swap, A, B, a_left, b_right, out, lane);
+          else if (tl > 8)
+            sb_tile<PREC, kOne, DIRECT>(w, ca, cb, cp, it, l0, tl, r0, tr, swap, A, B, a_left, b_right, out, lane);
+          else
+            sb_tile<PREC, kHalf, DIRECT>(w, ca, cb, cp, it, l0, tl, r0, tr, swap, A, B, a_left, b_right, out, lane);
+          if (DIRECT) continue;
           const int dc = 32 / tm, dr = 32 - dc * tm;
           int c = lane / tm, r = lane - c * tm;
           for (int e = lane; e < tm * tn; e += 32) {
@@ -842,12 +875,18 @@ cudaError_t launch_numeric_split(int precision, int sizes, DevMat A, DevMat B, D
   const size_t smem = kSbWarps * sizeof(SbWarp);
   const int grid = nsm * kSbBlocksPerSm;
   const uint4 *l = static_cast<const uint4 *>(a_left), *r = static_cast<const uint4 *>(b_right);
-  if (precision == BSM_PREC_SPLIT_BF16X3)
-    k_numeric_split_blocks<BSM_PREC_SPLIT_BF16X3><<<grid, kSbWarps * 32, smem, stream>>>(
-        A, B, C, Cin, l, r, alpha, beta, ws, st, items, seg, sizes, ntiles, work);
-  else
-    k_numeric_split_blocks<BSM_PREC_SPLIT_TF32X2><<<grid, kSbWarps * 32, smem, stream>>>(
-        A, B, C, Cin, l, r, alpha, beta, ws, st, items, seg, sizes, ntiles, work);
+  const bool direct = !C.host_vals;
+#define BSM_SPLIT_BLOCKS(P, D)                                                            \
+  k_numeric_split_blocks<P, D><<<grid, kSbWarps * 32, smem, stream>>>(                    \
+      A, B, C, Cin, l, r, alpha, beta, ws, st, items, seg, sizes, ntiles, work)
+  if (precision == BSM_PREC_SPLIT_BF16X3) {
+    if (direct) BSM_SPLIT_BLOCKS(BSM_PREC_SPLIT_BF16X3, true);
+    else BSM_SPLIT_BLOCKS(BSM_PREC_SPLIT_BF16X3, false);
+  } else {
+    if (direct) BSM_SPLIT_BLOCKS(BSM_PREC_SPLIT_TF32X2, true);
+    else BSM_SPLIT_BLOCKS(BSM_PREC_SPLIT_TF32X2, false);
+  }
+#undef BSM_SPLIT_BLOCKS
   return cudaGetLastError();
 }
 
@@ -911,8 +950,10 @@ cudaError_t numeric_split_init() {
     }
   }
   // the per-block kernel's operands come through L1: no more shared memory than its own
-  for (const void *fn : {(const void *)k_numeric_split_blocks<BSM_PREC_SPLIT_BF16X3>,
-                         (const void *)k_numeric_split_blocks<BSM_PREC_SPLIT_TF32X2>}) {
+  for (const void *fn : {(const void *)k_numeric_split_blocks<BSM_PREC_SPLIT_BF16X3, false>,
+                         (const void *)k_numeric_split_blocks<BSM_PREC_SPLIT_BF16X3, true>,
+                         (const void *)k_numeric_split_blocks<BSM_PREC_SPLIT_TF32X2, false>,
+                         (const void *)k_numeric_split_blocks<BSM_PREC_SPLIT_TF32X2, true>}) {
     cudaError_t e = cudaFuncSetAttribute(fn, cudaFuncAttributePreferredSharedMemoryCarveout,
                                          kSbCarveout);
     if (e == cudaSuccess)
