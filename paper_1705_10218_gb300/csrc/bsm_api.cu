@@ -1939,8 +1939,9 @@ int bsm_mat_create(bsm_ctx ctx, int32_t nbrows, const int32_t *row_sizes, int32_
     for (int32_t v : sizes) r = std::max(r, (double)((v - 1) / 8 + 1) / v);
     return r;
   };
-  M->digit_rate[0] = most(M->h_col_sizes);
-  M->digit_rate[1] = most(M->h_row_sizes);
+  // of the distinct sizes, where these are known
+  M->digit_rate[0] = most(M->kinds_exact ? M->col_kinds : M->h_col_sizes);
+  M->digit_rate[1] = most(M->kinds_exact ? M->row_kinds : M->h_row_sizes);
   // sizes, kinds and first scalars of the block rows, then of the block columns: one
   // buffer and one copy (each costs a matrix as much as its launches)
   const size_t nr = (size_t)nbrows, nc = (size_t)nbcols;
