@@ -23,7 +23,7 @@ namespace bsm {
 // (sc may be null: no C_in). Launched with kSegWarps warps per block. A step takes
 // fewer blocks where 32 would leave warps without work: few large blocks are bound
 // by the length of a warp's walk, not by memory (3431 blocks of up to 33 x 33 on 9728
-// warps: 273 -> 26 us).
+// warps: 273 -> 26 us); but not so few that a step has next to nothing to copy.
 constexpr int kSegWarps = 8;
 
 __global__ void __launch_bounds__(kSegWarps * 32)
@@ -38,7 +38,9 @@ __global__ void __launch_bounds__(kSegWarps * 32)
   const int64_t n = st->nblk_c;
   const int64_t w0 = (blockIdx.x * (int64_t)blockDim.x + threadIdx.x) >> 5;
   const int64_t nw = ((int64_t)gridDim.x * blockDim.x) >> 5;
-  const int per = (int)min((int64_t)32, max((int64_t)1, (n + nw - 1) / nw));
+  // at least four values a lane, on average
+  const int64_t tiny = (128 * n + st->nnz_c - 1) / max((int64_t)1, st->nnz_c);
+  const int per = (int)min((int64_t)32, max(max((int64_t)1, tiny), (n + nw - 1) / nw));
   for (int64_t g0 = w0 * per; g0 < n; g0 += nw * per) {
     const int64_t g = g0 + lane;
     int len = 0;
