@@ -55,27 +55,45 @@ FP64_KERNELS = {"t16b2": (0, "k_numeric_fp64_t16"), "t16b3": (1, "k_numeric_fp64
                 "t32": (2, "k_numeric_fp64_t32"), "pk12": (3, "k_numeric_fp64_pk"),
                 "pk16": (4, "k_numeric_fp64_pk"), "g8": (5, "k_numeric_fp64_g8")}
 FP64_BY_NUMBER = {v[0]: k for k, v in FP64_KERNELS.items()}
-# The default FP64 multiply is reported as pk12 and runs as its form on the tensor
-# cores: 43 products of FP16 digit pairs for one FP64 product.
+# The default FP64 multiply, which the library reports as pk12, runs as its form on the
+# tensor cores ("dg" here): 43 products of FP16 digit pairs for one FP64 product.
 DIGIT_KERNEL, DIGIT_PAIRS = "k_numeric_fp64_dg", 43
+
+
+def fp64_kernel_run(number, forced, autotune):
+    """Name of the FP64 kernel that multiplies with the given choice ran on, from the number
+    that the library reports. A tuned choice may be either of the two reported as pk12."""
+    name = FP64_BY_NUMBER.get(number)
+    if name != "pk12" or forced is not None:
+        return name
+    return "dg or pk12" if autotune else "dg"
+
+
 # DRAM bytes (read + write) per launch of a kernel, from one ncu capture
 # (dram__bytes_read.sum + dram__bytes_write.sum, profiles/): valid only while
 # the code that decides it is unchanged -- the kernel's own source section and,
 # for the FP64 kernels, the row-order work list (SHA-256 of each section) --
 # for that variant (fp64 kernel name or split precision) and workload at its
 # default eps.
+_ROW_ORDER_SECTIONS = [
+    ("paper_1705_10218_gb300/csrc/k_classes.cu", ("// Work in a row order.", "}  // namespace bsm"),
+     "b173af39936271e55c6a2623c0b1222afaca8a97ab34ff8f9a0ec78e9ecdf01b"),
+    ("paper_1705_10218_gb300/csrc/bsm_api.cu",
+     ("static void bfs_row_order(", "static uint64_t next_order_id("),
+     "113dd9175f43cb3ea209f7d880be5023dd9fd7acdf547fa5077ea74319814288")]
 MEASURED_TRAFFIC = {
+    ("dg", "water2048"): dict(
+        sections=[("paper_1705_10218_gb300/csrc/k_numeric_fp64.cu",
+                   ("// dg: the FP64 products on the tensor cores", "cudaError_t launch_numeric_fp64("),
+                   "a38b9124b8716630a724c075c9410a362581da575162dff4106c94048ecca42b"),
+                  *_ROW_ORDER_SECTIONS],
+        bytes=6.73e9 + 1.52e9),
     ("pk12", "water2048"): dict(
         sections=[("paper_1705_10218_gb300/csrc/k_numeric_fp64.cu",
-                   ("// pk\n", "cudaError_t launch_numeric_fp64("),
-                   "c4d0a2d33d0541f245f25dabd7b17608518a0df277e5ea3ac09dc06495b99449"),
-                  ("paper_1705_10218_gb300/csrc/k_classes.cu",
-                   ("// Work in a row order.", "}  // namespace bsm"),
-                   "b173af39936271e55c6a2623c0b1222afaca8a97ab34ff8f9a0ec78e9ecdf01b"),
-                  ("paper_1705_10218_gb300/csrc/bsm_api.cu",
-                   ("static void bfs_row_order(", "static uint64_t next_order_id("),
-                   "113dd9175f43cb3ea209f7d880be5023dd9fd7acdf547fa5077ea74319814288")],
-        bytes=6.80e9 + 1.68e9),
+                   ("// pk\n", "// dg: the FP64 products on the tensor cores"),
+                   "f619bd7f598ccda899d4dfc97f413656fe8b68dc6d5a5c9a5a5ef8ad050aadca"),
+                  *_ROW_ORDER_SECTIONS],
+        bytes=2.99e9 + 1.56e9),
 }
 
 
@@ -862,9 +880,10 @@ def main():
     # replay the phases are not timed separately: the whole multiply is used.
     if prof.multiplies > 0:
         num_ms = prof.ms_numeric / prof.multiplies
-        digits = args.precision == "fp64" and fk is None and FP64_BY_NUMBER[prof.last_fp64_kernel] == "pk12"
-        kname = (DIGIT_KERNEL if digits else
-                 FP64_KERNELS[FP64_BY_NUMBER[prof.last_fp64_kernel]][1] if args.precision == "fp64"
+        run = fp64_kernel_run(prof.last_fp64_kernel, fk, args.autotune) if args.precision == "fp64" else None
+        digits = run == "dg"
+        kname = (DIGIT_KERNEL if digits else f"{DIGIT_KERNEL} or k_numeric_fp64_pk" if run == "dg or pk12" else
+                 FP64_KERNELS[run][1] if run
                  else SPLIT_KERNEL_SYMBOLS.get(prof.last_split_kernel, "k_numeric_split_blocks"))
     else:
         num_ms = total_ms / args.steps
@@ -887,7 +906,7 @@ def main():
                                                clocks)
         roof = {"bound": "alu", "achieved": round(achieved, 2), "peak": round(fp64_peak, 1),
                 "unit": "GFLOP/s", "frac": round(achieved / fp64_peak, 4),
-                "traffic": (measured_traffic(FP64_BY_NUMBER[prof.last_fp64_kernel], args.workload)
+                "traffic": (measured_traffic(run, args.workload)
                             if prof.multiplies > 0 and args.eps_percentile is None else None),
                 "traffic_unit": "DRAM bytes per launch (ncu dram__bytes_read.sum + write.sum)",
                 "kernel": kname, "peak_source": fp64_src,
@@ -1006,7 +1025,7 @@ def main():
                        "eps": eps, "precision": args.precision, "launch": args.launch,
                        "split_kernel": args.split_kernel,
                        "graph": bool(args.graph), "autotune": bool(args.autotune),
-                       "fp64_kernel": (FP64_BY_NUMBER.get(prof.last_fp64_kernel)
+                       "fp64_kernel": (fp64_kernel_run(prof.last_fp64_kernel, fk, args.autotune)
                                        if args.precision == "fp64" else None),
                        "a_blocks": A.nblk, "c_blocks": nb_c, "c_nnz": nnz_c,
                        "kept_products": st.kept, "dropped_products": st.dropped,

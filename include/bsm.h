@@ -70,9 +70,7 @@ enum {
 
 /* FP64 numeric kernels. bsm_opts.fp64_kernel = 1 + one of these forces that
  * kernel for every shape class (no autotuning); 0 leaves the choice to the
- * library: the tuned one with autotune, else PK12, or T16_B2 when the last
- * multiply into the same C had fewer than 4 block products per C block (there
- * the per-block setup of PK costs more than its fuller lanes save).
+ * library (bsm_opts.fp64_kernel says how).
  *   T16: one output element per lane slot, 16 x 16 tiles, 2 or 3 blocks/SM;
  *   T32: 32 x 32 tiles, synchronous staging;
  *   PK12, PK16: packed lane slots (output element, k-group) over the products
@@ -97,8 +95,8 @@ enum {
  *   PANEL:  one C block row at a time as a dense panel product on the
  *           tcgen05 tensor cores (MMA M = the row's C columns, N = its block
  *           row size x slices, K = A's row), accumulators in tensor memory;
- *   BLOCKS: one C block per warp, its products one after another on mma.sync
- *           tiles, each product's operands streamed through shared memory;
+ *   BLOCKS: one C block (or some of its tiles) per warp, its products one after
+ *           another on mma.sync tiles, operands loaded straight into registers;
  *   CHUNKS: one C block per warp on mma.sync tiles, its products concatenated
  *           along k and staged into shared memory in chunks of whole products
  *           (C blocks larger than 16 x 16 go to the BLOCKS kernel).
@@ -149,8 +147,8 @@ typedef struct {
   double *host_values; /* NULL, or page-locked host memory (cudaHostAlloc /
                           cudaHostRegister, device-mapped) of host_cap doubles that also
                           receives the result's values, in bsm_mat_get_values order,
-                          written by the device while the multiply runs (the packed and g8
-                          FP64 kernels and the split-precision kernels store each C block
+                          written by the device while the multiply runs (the default, packed and
+                          g8 FP64 kernels and the split-precision kernels store each C block
                           there as they complete it; the other kernels are followed by a
                           device copy). Written only if the
                           result has at most host_cap values (bsm_mat_nblocks tells); valid
@@ -270,7 +268,8 @@ typedef struct {
   int64_t multiplies;  /* multiplies profiled */
   int64_t launches;    /* kernels launched by this context since profiling started */
   int32_t last_fp64_kernel; /* BSM_FP64_* of the last FP64 numeric launch enqueued by the
-                               context (forced, tuned or default), -1 if none */
+                               context (forced, tuned or default), -1 if none; PK12 also for
+                               its form on the tensor cores (bsm_opts.fp64_kernel) */
   int32_t last_split_kernel; /* BSM_SPLIT_* of the last split-precision numeric launch, -1 if
                                 none */
 } bsm_profile;
