@@ -74,9 +74,9 @@ __device__ __forceinline__ int lower_bound_i32(const int32_t *a, int lo, int hi,
 // Block norms: canonical Frobenius norm, column-major, no fused multiply-add; the
 // block count is read on the device so that a matrix produced by an earlier multiply
 // needs no host round trip. And the scales of the digit representation in the same
-// launch (rexp, cexp: where they are wanted): the first thread blocks take the norms, the others the scales, a warp per block: each
-// lane's elements go to their row's and column's maximum in shared memory, and a
-// maximum that the array does not hold yet there.
+// launch (rexp, cexp: where they are wanted): the first thread blocks take the norms,
+// the others the scales, a warp per block: each lane's elements go to their row's and
+// column's maximum in shared memory, and a maximum that the array does not hold yet there.
 //
 // A norm's additions have a fixed order, so a block's chain of them is one lane's. The
 // FP64 pipe takes a warp's instruction in 64 clocks of a quarter SM, whatever its
@@ -91,7 +91,6 @@ constexpr int kScaleWarps = 8;
 constexpr int kNormAhead = 8;   // loads of a lane in flight
 constexpr int kNormBlocksPerSm = 8;
 constexpr int kScaleRows = 64;  // rows and columns kept in shared memory
-
 
 // The sum of squares of the n values at x, in order; LANES lanes of a warp have the
 // same x and n, sub is the lane's number among them. All lanes of the warp take part.
