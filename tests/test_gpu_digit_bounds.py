@@ -97,3 +97,37 @@ def test_zero_rows_columns_and_blocks(bsm_lib):
     a[4], a[20:25], b[:, 3], a[:, 14] = 0.0, 0.0, 0.0, 0.0
     a[:13, :13], b[13:18] = np.diag(np.arange(13.0)), 0.0
     check(bsm_lib, blocks_of(a, rs, ks), blocks_of(b, ks, cs))
+
+
+def digits(x):
+    """The eight signed base-256 digits of x on the scale 1 (x times 2^62 is an integer here)."""
+    v = int(x * 2.0 ** 62)
+    assert v == x * 2.0 ** 62
+    out = []
+    for _ in range(7):
+        d = (v + 128) % 256 - 128
+        out.append(d)
+        v = (v - d) >> 8
+    return [v] + out[::-1]
+
+
+@pytest.mark.parametrize("low", [-128, 127])
+@pytest.mark.parametrize("rs,cs", [([16], [8]), ([8, 5], [13, 16]), ([16, 33], [5, 32])])
+def test_digits_at_their_extreme(bsm_lib, rs, cs, low):
+    """144 values of k, as many as are added up in FP32 between two reads, with every digit
+    but the first at its extreme: 7 x 2^14 x 144 = 16.5 M of 2^24 on a diagonal. A large value
+    on either side that meets a zero sets the scales. The result is that of exact integers
+    over the kept digit pairs, rounded once."""
+    ks = [8] * 18 + [2]
+    x = sum(low * 256 ** (7 - i) for i in range(1, 8)) * 2.0 ** -62
+    a, b = np.full((sum(rs), sum(ks)), x), np.full((sum(ks), sum(cs)), x)
+    a[:, -2:], b[-2:] = [0.5, 0.0], np.array([[0.0], [0.5]])
+    d = digits(x)
+    kept = 144 * sum(d[i] * d[j] * 256 ** (14 - i - j) for i in range(8) for j in range(8) if i + j < 9)
+    with bsm_lib.Context(0) as ctx:
+        A, B = blocks_of(a, rs, ks), blocks_of(b, ks, cs)
+        dA, dB, dC = ctx.from_blocks(A), ctx.from_blocks(B), ctx.empty(A.row_sizes, B.col_sizes)
+        ctx.multiply(1.0, dA, dB, 0.0, dC, 0.0, blocking=True)
+        assert (dC.values() == kept / 2 ** 124).all()  # of integers: rounded to nearest
+    # more than FP64 FMAs of the values would give without an error: not by accident
+    assert kept != int(x * 2.0 ** 62) ** 2 * 144

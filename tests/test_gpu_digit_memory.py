@@ -45,8 +45,8 @@ def multiply(ctx, A, C, kern=None):
 """
 
 
-def child(code, cap):
-    env = dict(os.environ, BSM_DEVICE_MEMORY_CAP=str(cap))
+def child(code, cap, **more):
+    env = dict(os.environ, BSM_DEVICE_MEMORY_CAP=str(cap), **more)
     p = subprocess.run([sys.executable, "-c", COMMON + code], cwd=ROOT, env=env, capture_output=True,
                        text=True, timeout=600)
     assert p.returncode == 0, p.stderr[-2000:]
@@ -141,3 +141,26 @@ print(json.dumps(bad))
 @pytest.mark.parametrize("cap", [28, 36, 48])
 def test_threads_take_digits_from_each_other(bsm_lib, cap):
     assert child(THREADS, cap << 20) == []
+
+
+# A tuned choice of the digit kernel (value 6 of the cache file), without and with the memory.
+TUNED = r"""
+A = banded(8000, 9)
+with Context(0) as ctx:
+    dA, dC = ctx.from_blocks(A), ctx.empty(A.row_sizes, A.col_sizes)
+    want = [multiply(ctx, dA, dC, BSM_FP64_PK12) for _ in range(2)][1]  # both of C's buffers
+    held = ballast(ctx, 256 << 10)
+    without = multiply(ctx, dA, dC)
+    for m in held:
+        m.destroy()
+    full = multiply(ctx, dA, dC)
+print(json.dumps(dict(without=bool(np.array_equal(without, want)), full=bool(np.array_equal(full, want)),
+                      off=H.rel_frobenius(full, want))))
+"""
+
+
+def test_a_tuned_digit_kernel_without_memory_is_the_packed_one(bsm_lib, tmp_path):
+    cache = tmp_path / "tuned"
+    cache.write_text("fp64/all/1,|1,|1, 6 0.0\n")
+    out = child(TUNED, 48 << 20, BSM_AUTOTUNE_CACHE=str(cache))
+    assert out["without"] and not out["full"] and out["off"] <= 1e-15
