@@ -132,7 +132,8 @@ double est_run_ms(int64_t macs, int precision) {
 // a result can be handed to the caller without a copy. Freed blocks are kept
 // for reuse (cudaHostAlloc is slow), up to kPinnedCap bytes.
 constexpr size_t kPinnedCap = 16ull << 30;
-constexpr size_t kHeapInput = 8u << 20;
+constexpr size_t kHeapInput = 8u << 20;  // inputs that may go to the heap, at most
+constexpr size_t kOwedBlocks = 64;       // blocks that a lane adds for such inputs when idle, at most
 constexpr int64_t kHostValuesCap = 128ll << 20;  // values (1 GiB) a lane's multiply stores directly
 
 struct PinnedPool {
@@ -500,8 +501,17 @@ static bool pick_batch(bsm_server s, std::vector<Request *> &batch) {
 static void worker_loop(bsm_server s, int lane) {
   cudaSetDevice(s->device);
   std::vector<Request *> batch;
+  std::vector<size_t> owed;  // sizes of inputs that found no page-locked block
   std::unique_lock<std::mutex> lk(s->mu);
   for (;;) {
+    if (!owed.empty() && s->queue.empty() && !s->stop) {  // the next ones of these sizes find one
+      lk.unlock();
+      std::vector<void *> blocks;
+      for (size_t b : owed) blocks.push_back(s->pinned.get(b));
+      for (void *p : blocks) s->pinned.put(p);
+      owed.clear();
+      lk.lock();
+    }
     s->cv.wait(lk, [&] { return s->stop || pick_batch(s, batch); });
     if (s->stop) {  // queued requests are dropped by bsm_server_destroy
       for (Request *r : batch) s->queue.push_front(r);
@@ -509,10 +519,10 @@ static void worker_loop(bsm_server s, int lane) {
     }
     int64_t held = 0;
     const double t = now_ms();
-    std::vector<size_t> heap;  // inputs that found no page-locked block
     for (Request *r : batch) {
       held += r->footprint;
-      if (r->heap) heap.push_back(8 * (size_t)std::max<int64_t>(r->nvals, 1));
+      if (r->heap && owed.size() < kOwedBlocks)
+        owed.push_back(8 * (size_t)std::max<int64_t>(r->nvals, 1));
       r->state = kRunning;
       r->slot = lane;
       r->t_start = t;
@@ -538,13 +548,6 @@ static void worker_loop(bsm_server s, int lane) {
     s->completed += (int64_t)batch.size();
     batch.clear();
     s->cv.notify_all();  // a head that waited for memory may fit now
-    if (!heap.empty()) {  // the next inputs of these sizes find one
-      lk.unlock();
-      std::vector<void *> blocks;
-      for (size_t b : heap) blocks.push_back(s->pinned.get(b));
-      for (void *p : blocks) s->pinned.put(p);
-      lk.lock();
-    }
   }
 }
 
