@@ -115,8 +115,9 @@ constexpr uint32_t kDigitOutside = 1u << 31;
 // class (7, digit_sum_of)
 constexpr int kDigitPadAt = 13, kDigitClassAt = 16, kDigitSumAt = 22;
 // How far a row may lie below its block's class before all C blocks of the block are FP64
-// FMAs'. A wider range keeps more C blocks on the tensor cores: two sign iterations of 192
-// water molecules 18.6 ms at 9, 15.3 at 11, 14.4 at 12, 13 and 15.
+// FMAs' at once. A wider range keeps more C blocks on the tensor cores, as far as dg_enough
+// does: two sign iterations of 192 water molecules, without it, 18.6 ms at 9, 15.3 at 11,
+// 14.4 at 12, 13 and 15.
 constexpr int kDigitRange = 12;
 constexpr int kDigitMaxRows = 128;
 constexpr int kDigitMaxOctets = 0x1FFF;
