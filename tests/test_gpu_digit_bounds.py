@@ -131,3 +131,12 @@ def test_digits_at_their_extreme(bsm_lib, rs, cs, low):
         assert (dC.values() == kept / 2 ** 124).all()  # of integers: rounded to nearest
     # more than FP64 FMAs of the values would give without an error: not by accident
     assert kept != int(x * 2.0 ** 62) ** 2 * 144
+
+
+@pytest.mark.parametrize("k", [65528, 65529, 70001])
+def test_the_longest_k_that_digits_take(bsm_lib, k):
+    """8191 octets of k in a block are the digits' limit; longer ones are the packed kernel's."""
+    rng = np.random.default_rng(k)
+    rs, ks, cs = [5, 3], [k, 9, k, 2, k, 4], [4]
+    a, b = rng.standard_normal((sum(rs), sum(ks))), rng.standard_normal((sum(ks), sum(cs)))
+    assert check(bsm_lib, blocks_of(a, rs, ks), blocks_of(b, ks, cs)) <= 1e-13
